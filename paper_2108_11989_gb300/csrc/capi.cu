@@ -365,7 +365,7 @@ int qs_d32_run(qs_lattice *lat, int storage, const double *m0, const void *in, v
     c.m0 = m0;
     int &tv = lat->tuned32[storage][c.cheb][nrhs];
     if (tv == 0) {
-        const std::string key = tune_key(lat, "dslash32", storage, c.cheb, nrhs);
+        const std::string key = tune_key(lat, "dslash32p", storage, c.cheb, nrhs);
         int v = tune_lookup(key);
         if (v < 0 || v >= qs_d32_nvariants()) {
             if (capturing(lat->stream)) {

@@ -3,14 +3,27 @@
 //
 //   out = (4 + m0) psi + A psi - 1/2 sum_mu [ V (1 - g_mu) psi(x+mu) + V^+ (1 + g_mu) psi(x-mu) ]
 //
-// Thread map.  A block has 128 threads.  Each warp covers 32 / RL consecutive sites
-// and RL "RHS lanes"; a thread computes its site for G right-hand sides.  The RL
-// lanes of one site load the same link and SW-term words in the same instruction, so
-// a link or SW word leaves L1 once for RL * G right-hand sides, and a thread applies
-// every link it loads to G right-hand sides.  Blocks run through all sites of one
-// group of RL * G right-hand sides before the next group starts, so the spinor
-// neighbours a block needs were read recently by its neighbouring blocks (the
-// working set of one group, a few time slices of RL * G vectors, stays in L2).
+// Thread map.  One thread computes one right-hand side at a physical site p AND at its
+// mirror site p + L e_x.  The mirror's links are the complex conjugates of the same
+// words, its SW block is S conj(A) S of the same block, and its neighbours are the
+// mirrors of p's neighbours, so every link and SW word that is loaded feeds two sites
+// and all conjugations and spin swaps are compile-time (only the backward hops across a
+// C* boundary need a sign, which costs nothing in the multiply-adds that use it).
+//
+// Arithmetic.  The matrix products use the packed FP32 instructions (two multiply-adds per
+// instruction): with a link entry u and the pair h = (re, im) of a spinor component,
+// a += (u.re, u.re) h and b += (u.im, u.im) h, and the product is a + i b (a - i b for the
+// conjugate link), combined once per row.  The links are stored times -1/2.
+//
+// What bounds it.  16^3 x 32, 16 right-hand sides, FP32: 298 us (406 us with one thread per
+// doubled site and unpacked arithmetic), 2.96 TB/s of algorithmic bytes; FP16 storage 308 us
+// (409), so not the bytes.  1280 thread instructions per site and right-hand side (2200), of
+// which 820 go to the FMA pipe, where a packed instruction with three distinct operands
+// takes 3 cycles; the pipe alone needs about 180 us.  The rest is the latency of the neighbour loads at the
+// 12 warps per SM that 168 registers allow, so the next spinor and link are requested before
+// the current ones are multiplied (hops below: 308 -> 298 us).  Tried and slower: one site
+// per thread at 20 to 24 warps per SM (382 us: the links and their broadcasts are no longer
+// shared), unpacked multiply-adds (346 us).
 //
 // Storage.  FP32: the solver's site-tiled layout [site / 16][12][site % 16] float2 or
 // the canonical [site][12] float2.  FP16 / BF16: tiles of 16 sites, 12 x 16 half2 (or
@@ -38,21 +51,68 @@ __device__ __forceinline__ cf cadd(cf a, cf b) { return make_float2(a.x + b.x, a
 __device__ __forceinline__ cf csub(cf a, cf b) { return make_float2(a.x - b.x, a.y - b.y); }
 __device__ __forceinline__ cf cneg(cf a) { return make_float2(-a.x, -a.y); }
 __device__ __forceinline__ cf cmi(cf a) { return make_float2(-a.y, a.x); }   // i a
-// c + a b
-__device__ __forceinline__ cf cfma(cf a, cf b, cf c)
-{
-    return make_float2(fmaf(a.x, b.x, fmaf(-a.y, b.y, c.x)), fmaf(a.x, b.y, fmaf(a.y, b.x, c.y)));
-}
+// packed FP32: both halves at once
+__device__ __forceinline__ cf dup(float a) { return make_float2(a, a); }
+__device__ __forceinline__ cf add2(cf a, cf b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ cf mul2(cf a, cf b) { return __fmul2_rn(a, b); }
+__device__ __forceinline__ cf fma2(cf a, cf b, cf c) { return __ffma2_rn(a, b, c); }
+__device__ __forceinline__ cf sub2(cf a, cf b) { return __ffma2_rn(b, make_float2(-1.f, -1.f), a); }
 
 // ---- storage formats ------------------------------------------------------
+// loads that stay where they are written, so that the next neighbour's words are in flight
+// while the current one is multiplied
+__device__ __forceinline__ cf ldv(const cf *p)
+{
+    cf r;
+    asm volatile("ld.global.nc.v2.f32 {%0, %1}, [%2];" : "=f"(r.x), "=f"(r.y) : "l"(p));
+    return r;
+}
+__device__ __forceinline__ float4 ldv(const float4 *p)
+{
+    float4 r;
+    asm volatile("ld.global.nc.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(r.x), "=f"(r.y), "=f"(r.z), "=f"(r.w) : "l"(p));
+    return r;
+}
+__device__ __forceinline__ unsigned ldv(const unsigned *p)
+{
+    unsigned r;
+    asm volatile("ld.global.nc.u32 %0, [%1];" : "=r"(r) : "l"(p));
+    return r;
+}
+__device__ __forceinline__ float ldv(const float *p)
+{
+    float r;
+    asm volatile("ld.global.nc.f32 %0, [%1];" : "=f"(r) : "l"(p));
+    return r;
+}
+
 struct StF32Tiled {
     static constexpr int64_t kBytesPerSite = 96;
     static constexpr bool kScaled = false;
+    struct Raw { cf v[12]; };
+    __device__ static void fetch(const char *__restrict__ base, int s, Raw &r)
+    {
+        const cf *b = reinterpret_cast<const cf *>(base) + ((int64_t)(s >> 4) * 12) * 16 + (s & 15);
+#pragma unroll
+        for (int c = 0; c < 12; ++c) r.v[c] = ldv(b + c * 16);
+    }
+    __device__ static void open(const Raw &r, cf v[12])
+    {
+#pragma unroll
+        for (int c = 0; c < 12; ++c) v[c] = r.v[c];
+    }
     __device__ static void ld(const char *__restrict__ base, int s, cf v[12])
     {
         const cf *b = reinterpret_cast<const cf *>(base) + ((int64_t)(s >> 4) * 12) * 16 + (s & 15);
 #pragma unroll
         for (int c = 0; c < 12; ++c) v[c] = __ldg(b + c * 16);
+    }
+    // the 6 components of chiral block `blk` (spins 2 blk, 2 blk + 1)
+    __device__ static void ld6(const char *__restrict__ base, int s, int blk, cf v[6])
+    {
+        const cf *b = reinterpret_cast<const cf *>(base) + ((int64_t)(s >> 4) * 12 + 6 * blk) * 16 + (s & 15);
+#pragma unroll
+        for (int c = 0; c < 6; ++c) v[c] = __ldg(b + c * 16);
     }
     __device__ static void st(char *__restrict__ base, int s, const cf v[12])
     {
@@ -65,11 +125,36 @@ struct StF32Tiled {
 struct StF32Canon {
     static constexpr int64_t kBytesPerSite = 96;
     static constexpr bool kScaled = false;
+    struct Raw { float4 v[6]; };
+    __device__ static void fetch(const char *__restrict__ base, int s, Raw &r)
+    {
+        const float4 *q = reinterpret_cast<const float4 *>(base) + (int64_t)s * 6;
+#pragma unroll
+        for (int i = 0; i < 6; ++i) r.v[i] = ldv(q + i);
+    }
+    __device__ static void open(const Raw &r, cf v[12])
+    {
+#pragma unroll
+        for (int i = 0; i < 6; ++i) {
+            v[2 * i] = make_float2(r.v[i].x, r.v[i].y);
+            v[2 * i + 1] = make_float2(r.v[i].z, r.v[i].w);
+        }
+    }
     __device__ static void ld(const char *__restrict__ base, int s, cf v[12])
     {
         const float4 *q = reinterpret_cast<const float4 *>(base) + (int64_t)s * 6;
 #pragma unroll
         for (int i = 0; i < 6; ++i) {
+            float4 a = __ldg(q + i);
+            v[2 * i] = make_float2(a.x, a.y);
+            v[2 * i + 1] = make_float2(a.z, a.w);
+        }
+    }
+    __device__ static void ld6(const char *__restrict__ base, int s, int blk, cf v[6])
+    {
+        const float4 *q = reinterpret_cast<const float4 *>(base) + (int64_t)s * 6 + 3 * blk;
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
             float4 a = __ldg(q + i);
             v[2 * i] = make_float2(a.x, a.y);
             v[2 * i + 1] = make_float2(a.z, a.w);
@@ -93,17 +178,19 @@ struct StScaled {
     __device__ static float2 cvt(H2 h);
     __device__ static H2 pack(float a, float b);
     // the stored (site-normalised) values and the site's scale
-    __device__ static void ld_raw(const char *__restrict__ base, int s, cf v[12], float *scale)
+    struct Raw { unsigned w[12]; float sc; };
+    __device__ static void fetch(const char *__restrict__ base, int s, Raw &r)
     {
         const char *t = base + (int64_t)(s >> 4) * kTile;
         const unsigned *w = reinterpret_cast<const unsigned *>(t) + (s & 15);
-        *scale = __ldg(reinterpret_cast<const float *>(t + 768) + (s & 15));
+        r.sc = ldv(reinterpret_cast<const float *>(t + 768) + (s & 15));
 #pragma unroll
-        for (int c = 0; c < 12; ++c) {
-            unsigned u = __ldg(w + c * 16);
-            H2 h = *reinterpret_cast<H2 *>(&u);
-            v[c] = cvt(h);
-        }
+        for (int c = 0; c < 12; ++c) r.w[c] = ldv(w + c * 16);
+    }
+    __device__ static void open(const Raw &r, cf v[12])
+    {
+#pragma unroll
+        for (int c = 0; c < 12; ++c) v[c] = cvt(*reinterpret_cast<const H2 *>(&r.w[c]));
     }
     __device__ static void ld(const char *__restrict__ base, int s, cf v[12])
     {
@@ -116,6 +203,18 @@ struct StScaled {
             H2 h = *reinterpret_cast<H2 *>(&u);
             float2 f = cvt(h);
             v[c] = make_float2(f.x * sc, f.y * sc);
+        }
+    }
+    __device__ static void ld6(const char *__restrict__ base, int s, int blk, cf v[6])
+    {
+        const char *t = base + (int64_t)(s >> 4) * kTile;
+        const unsigned *w = reinterpret_cast<const unsigned *>(t) + 96 * blk + (s & 15);
+        const float sc = __ldg(reinterpret_cast<const float *>(t + 768) + (s & 15));
+#pragma unroll
+        for (int c = 0; c < 6; ++c) {
+            unsigned u = __ldg(w + c * 16);
+            H2 h = *reinterpret_cast<H2 *>(&u);
+            v[c] = mul2(dup(sc), cvt(h));
         }
     }
     __device__ static void st(char *__restrict__ base, int s, const cf v[12])
@@ -149,16 +248,16 @@ __device__ __forceinline__ void project(const cf v[12], cf h[2][3])
 {
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-        cf p0 = v[c], p1 = v[3 + c], p2 = v[6 + c], p3 = v[9 + c];
+        const cf p0 = v[c], p1 = v[3 + c], p2 = v[6 + c], p3 = v[9 + c];
         if (MU == 0) {
-            h[0][c] = FW ? cadd(p0, p2) : csub(p0, p2);
-            h[1][c] = FW ? cadd(p1, p3) : csub(p1, p3);
+            h[0][c] = FW ? add2(p0, p2) : sub2(p0, p2);
+            h[1][c] = FW ? add2(p1, p3) : sub2(p1, p3);
         } else if (MU == 1) {
             h[0][c] = FW ? cadd(p0, cmi(p3)) : csub(p0, cmi(p3));
             h[1][c] = FW ? cadd(p1, cmi(p2)) : csub(p1, cmi(p2));
         } else if (MU == 2) {
-            h[0][c] = FW ? cadd(p0, p3) : csub(p0, p3);
-            h[1][c] = FW ? csub(p1, p2) : cadd(p1, p2);
+            h[0][c] = FW ? add2(p0, p3) : sub2(p0, p3);
+            h[1][c] = FW ? sub2(p1, p2) : add2(p1, p2);
         } else {
             h[0][c] = FW ? cadd(p0, cmi(p2)) : csub(p0, cmi(p2));
             h[1][c] = FW ? csub(p1, cmi(p3)) : cadd(p1, cmi(p3));
@@ -166,96 +265,56 @@ __device__ __forceinline__ void project(const cf v[12], cf h[2][3])
     }
 }
 
-// acc += (x, lower(x)), lower = -+ e_mu^+ x
-template <int MU, bool FW>
-__device__ __forceinline__ void reconstruct(cf acc[12], const cf x[2][3])
+// acc += row (q, c) of (x, lower(x)), lower = -+ e_mu^+ x
+template <int MU, bool FW, int Q>
+__device__ __forceinline__ void reconstruct(cf acc[12], int c, cf x)
 {
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-        acc[c] = cadd(acc[c], x[0][c]);
-        acc[3 + c] = cadd(acc[3 + c], x[1][c]);
-        if (MU == 0) {
-            acc[6 + c] = FW ? cadd(acc[6 + c], x[0][c]) : csub(acc[6 + c], x[0][c]);
-            acc[9 + c] = FW ? cadd(acc[9 + c], x[1][c]) : csub(acc[9 + c], x[1][c]);
-        } else if (MU == 1) {
-            acc[6 + c] = FW ? csub(acc[6 + c], cmi(x[1][c])) : cadd(acc[6 + c], cmi(x[1][c]));
-            acc[9 + c] = FW ? csub(acc[9 + c], cmi(x[0][c])) : cadd(acc[9 + c], cmi(x[0][c]));
-        } else if (MU == 2) {
-            acc[6 + c] = FW ? csub(acc[6 + c], x[1][c]) : cadd(acc[6 + c], x[1][c]);
-            acc[9 + c] = FW ? cadd(acc[9 + c], x[0][c]) : csub(acc[9 + c], x[0][c]);
-        } else {
-            acc[6 + c] = FW ? csub(acc[6 + c], cmi(x[0][c])) : cadd(acc[6 + c], cmi(x[0][c]));
-            acc[9 + c] = FW ? cadd(acc[9 + c], cmi(x[1][c])) : csub(acc[9 + c], cmi(x[1][c]));
-        }
-    }
+    acc[3 * Q + c] = add2(acc[3 * Q + c], x);
+    constexpr int LO = (MU == 0 || MU == 3) ? 6 + 3 * Q : 9 - 3 * Q;   // lower spin fed by x
+    cf &l = acc[LO + c];
+    if (MU == 0) l = FW ? add2(l, x) : sub2(l, x);
+    else if (MU == 2) l = (FW == (Q == 0)) ? add2(l, x) : sub2(l, x);
+    else if (MU == 1) l = FW ? csub(l, cmi(x)) : cadd(l, cmi(x));
+    else l = (FW == (Q == 0)) ? csub(l, cmi(x)) : cadd(l, cmi(x));
 }
 
 __host__ __device__ constexpr int tri(int i, int j) { return i * (i - 1) / 2 + j; }
 
-// entry (i, j) of a packed SW block P (pairs: 3 of real diagonals, 15 of strict-lower
-// complex entries), for a physical site
-template <int I, int J>
-__device__ __forceinline__ cf sw_entry(const cf P[18])
-{
-    if constexpr (I > J) {
-        return P[3 + tri(I, J)];
-    } else {
-        cf e = P[3 + tri(J, I)];
-        return make_float2(e.x, -e.y);
-    }
-}
-// entry (i, j) of the mirror site's block S conj(A) S: sign (same spin half ? + : -)
-// times conj(A[i +- 3][j +- 3])
-template <int I, int J>
-__device__ __forceinline__ cf sw_entry_mirror(const cf P[18])
-{
-    constexpr int II = (I + 3) % 6, JJ = (J + 3) % 6;
-    cf e = sw_entry<II, JJ>(P);
-    e.y = -e.y;
-    if ((I < 3) != (J < 3)) e = cneg(e);
-    return e;
-}
-template <int I>
-__device__ __forceinline__ float sw_diag(const cf P[18], bool mir)
-{
-    constexpr int II = (I + 3) % 6;
-    const float d0 = (I & 1) ? P[I / 2].y : P[I / 2].x;
-    const float dm = (II & 1) ? P[II / 2].y : P[II / 2].x;
-    return mir ? dm : d0;
-}
+// real diagonal I of a packed SW block (pairs: 3 of real diagonals, 15 of strict-lower
+// complex entries)
+__device__ __forceinline__ float sw_diag(const cf P[18], int i) { return (i & 1) ? P[i / 2].y : P[i / 2].x; }
 
-template <int I, int J, int G>
-__device__ __forceinline__ void sw_row_term(const cf P[18], bool mir, int b, const cf v[G][12], cf acc[G][12])
+// acc = (dm + A) v for one chiral block of the physical site (MIR = false), or with the mirror
+// site's block S conj(A) S: element (i, j) of it is t_i t_j conj(A[i'][j']), i' = i +- 3 the
+// other spin half and t = (+, -) on the two halves.
+template <bool MIR>
+__device__ __forceinline__ void sw_block(const cf P[18], float dm, const cf v[6], cf acc[6])
 {
-    if constexpr (I == J) {
-        const float d = sw_diag<I>(P, mir);
+    cf w[6];
 #pragma unroll
-        for (int g = 0; g < G; ++g) {
-            acc[g][6 * b + I].x = fmaf(d, v[g][6 * b + J].x, acc[g][6 * b + I].x);
-            acc[g][6 * b + I].y = fmaf(d, v[g][6 * b + J].y, acc[g][6 * b + I].y);
+    for (int j = 0; j < 6; ++j) w[j] = !MIR ? v[j] : (j < 3 ? cneg(v[j + 3]) : v[j - 3]);
+#pragma unroll
+    for (int i = 0; i < 6; ++i) {
+        cf a = mul2(dup(dm + sw_diag(P, i)), w[i]);
+        cf lo = make_float2(0.f, 0.f), up = lo;   // sums of im(A_ij) w_j over j < i, im(A_ji) w_j over j > i
+#pragma unroll
+        for (int j = 0; j < 6; ++j) {
+            if (j == i) continue;
+            const cf e = j < i ? P[3 + tri(i, j)] : P[3 + tri(j, i)];
+            a = fma2(dup(e.x), w[j], a);
+            if (j < i) lo = j == 0 ? mul2(dup(e.y), w[j]) : fma2(dup(e.y), w[j], lo);
+            else up = j == i + 1 ? mul2(dup(e.y), w[j]) : fma2(dup(e.y), w[j], up);
         }
-    } else {
-        const cf e0 = sw_entry<I, J>(P), em = sw_entry_mirror<I, J>(P);
-        const cf e = mir ? em : e0;
-#pragma unroll
-        for (int g = 0; g < G; ++g) acc[g][6 * b + I] = cfma(e, v[g][6 * b + J], acc[g][6 * b + I]);
+        const cf d = i == 0 ? cneg(up) : i == 5 ? lo : sub2(lo, up);   // a + i d (physical), a - i d (mirror)
+        if (!MIR) acc[i] = make_float2(a.x - d.y, a.y + d.x);
+        else if (i < 3) acc[i + 3] = make_float2(-a.x - d.y, d.x - a.y);
+        else acc[i - 3] = make_float2(a.x + d.y, a.y - d.x);
     }
-}
-
-template <int I, int G>
-__device__ __forceinline__ void sw_row(const cf P[18], bool mir, int b, const cf v[G][12], cf acc[G][12])
-{
-    sw_row_term<I, 0, G>(P, mir, b, v, acc);
-    sw_row_term<I, 1, G>(P, mir, b, v, acc);
-    sw_row_term<I, 2, G>(P, mir, b, v, acc);
-    sw_row_term<I, 3, G>(P, mir, b, v, acc);
-    sw_row_term<I, 4, G>(P, mir, b, v, acc);
-    sw_row_term<I, 5, G>(P, mir, b, v, acc);
 }
 
 struct D32 {
     Geom g;
-    const cf *links;    // [mu][9][Vphys]
+    const cf *links;    // [mu][9][Vphys], times -1/2
     const cf *clov;     // [2][18][Vphys]
     const char *in;     // right-hand side r at in + r * vbytes
     char *out;
@@ -269,162 +328,165 @@ struct D32 {
     const float *coef, *dmdev;
 };
 
-template <int MU, int STEP, class S, int G>
-__device__ __forceinline__ void hop(const D32 &a, const Site &c, bool mir, int r0, int nr, cf acc[G][12])
+// acc += upper and lower parts of M h for a neighbour's spinor, M = U (FW, sigma = +1),
+// conj(U) (FW, -1), U^+ (backward, -1) or U^T (backward, +1)
+template <int MU, bool FW, class S>
+__device__ __forceinline__ void hop_apply(const cf U[9], float sigma, float f, bool anti, const typename S::Raw &raw,
+                                          cf acc[12])
 {
+    cf v[12], h[2][3];
+    S::open(raw, v);
+    project<MU, FW>(v, h);
+    if constexpr (S::kScaled) {
+        // the site's scale commutes with the projection: apply it to the 6 projected
+        // components instead of the 12 loaded ones
+        const float sc = MU == 0 ? raw.sc * f : raw.sc;
+#pragma unroll
+        for (int q = 0; q < 2; ++q)
+#pragma unroll
+            for (int i = 0; i < 3; ++i) h[q][i] = mul2(dup(sc), h[q][i]);
+    } else if (MU == 0 && anti) {
+#pragma unroll
+        for (int q = 0; q < 2; ++q)
+#pragma unroll
+            for (int i = 0; i < 3; ++i) h[q][i] = mul2(dup(f), h[q][i]);
+    }
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        cf a[2], b[2];
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+            const cf u = FW ? U[i * 3 + j] : U[j * 3 + i];
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                a[q] = j == 0 ? mul2(dup(u.x), h[q][j]) : fma2(dup(u.x), h[q][j], a[q]);
+                b[q] = j == 0 ? mul2(dup(u.y), h[q][j]) : fma2(dup(u.y), h[q][j], b[q]);
+            }
+        }
+        reconstruct<MU, FW, 0>(acc, i, make_float2(fmaf(-sigma, b[0].y, a[0].x), fmaf(sigma, b[0].x, a[0].y)));
+        reconstruct<MU, FW, 1>(acc, i, make_float2(fmaf(-sigma, b[1].y, a[1].x), fmaf(sigma, b[1].x, a[1].y)));
+    }
+}
+
+// one direction of a physical site and its mirror: the neighbour sites, the link in flight
+struct Hop {
+    cf U[9];
+    int n, nm;      // the neighbours of the site and of its mirror
+    float sigma, f;
+};
+
+// hop number D: direction D / 2, forward for even D
+template <int D>
+__device__ __forceinline__ void hop_begin(const D32 &a, const Site &c, Hop &h)
+{
+    constexpr int MU = D / 2, STEP = D % 2 ? -1 : 1;
     int sg;
     const Nb n = nbr_of<MU, STEP>(a.g, c, &sg);
     const int lp = STEP > 0 ? c.p : n.p;
-    const bool lcj = STEP > 0 ? mir : n.mir;
     const int64_t V = a.g.Vphys;
-    // M = -1/2 sg (forward: W, backward: W^+), W = lcj ? conj(U) : U
-    cf U[9];
 #pragma unroll
-    for (int k = 0; k < 9; ++k) U[k] = __ldg(a.links + (int64_t)(MU * 9 + k) * V + lp);
-    const float f = -0.5f * (float)sg;
-    const bool neg = STEP > 0 ? lcj : !lcj;
-    const float fi = neg ? -f : f;
-    cf M[9];
-#pragma unroll
-    for (int i = 0; i < 3; ++i)
-#pragma unroll
-        for (int j = 0; j < 3; ++j) {
-            const cf u = STEP > 0 ? U[i * 3 + j] : U[j * 3 + i];
-            M[i * 3 + j] = make_float2(f * u.x, fi * u.y);
-        }
-#pragma unroll
-    for (int g = 0; g < G; ++g) {
-        if (g < nr) {
-            cf v[12];
-            cf h[2][3], xx[2][3];
-            if constexpr (S::kScaled) {
-                // the site's scale commutes with the projection: apply it to the 6
-                // projected components instead of the 12 loaded ones
-                float sc;
-                S::ld_raw(a.in + (int64_t)(r0 + g) * a.vbytes, n.s, v, &sc);
-                project<MU, (STEP > 0)>(v, h);
-#pragma unroll
-                for (int q = 0; q < 2; ++q)
-#pragma unroll
-                    for (int i = 0; i < 3; ++i) h[q][i] = make_float2(sc * h[q][i].x, sc * h[q][i].y);
-            } else {
-                S::ld(a.in + (int64_t)(r0 + g) * a.vbytes, n.s, v);
-                project<MU, (STEP > 0)>(v, h);
-            }
-#pragma unroll
-            for (int q = 0; q < 2; ++q)
-#pragma unroll
-                for (int i = 0; i < 3; ++i) {
-                    cf t = make_float2(0.f, 0.f);
-#pragma unroll
-                    for (int j = 0; j < 3; ++j) t = cfma(M[i * 3 + j], h[q][j], t);
-                    xx[q][i] = t;
-                }
-            reconstruct<MU, (STEP > 0)>(acc[g], xx);
-        }
+    for (int k = 0; k < 9; ++k) h.U[k] = ldv(a.links + (int64_t)(MU * 9 + k) * V + lp);
+    h.sigma = STEP > 0 ? 1.f : (n.mir ? 1.f : -1.f);
+    h.f = (float)sg;
+    h.n = n.s;
+    h.nm = n.mir ? n.s - a.g.L : n.s + a.g.L;
+}
+
+// hops D .. 7; `h` and `v` hold hop D's link and the physical site's neighbour, already
+// requested.  While one spinor is multiplied the next one is in flight.
+template <int D, class S>
+__device__ __forceinline__ void hops(const D32 &a, const Site &c, const char *in, Hop &h, typename S::Raw &v,
+                                     cf acc[12], cf accm[12])
+{
+    typename S::Raw w;
+    S::fetch(in, h.nm, w);
+    hop_apply<D / 2, D % 2 == 0, S>(h.U, h.sigma, h.f, a.g.t_anti, v, acc);
+    if constexpr (D < 7) {
+        Hop h2;
+        hop_begin<D + 1>(a, c, h2);
+        S::fetch(in, h2.n, v);
+        hop_apply<D / 2, D % 2 == 0, S>(h.U, -h.sigma, h.f, a.g.t_anti, w, accm);
+        hops<D + 1, S>(a, c, in, h2, v, acc, accm);
+    } else {
+        hop_apply<D / 2, D % 2 == 0, S>(h.U, -h.sigma, h.f, a.g.t_anti, w, accm);
     }
 }
 
-// block (bx, by): sites [bx * 128 / RL, ...), right-hand sides [by * RL * G, ...)
-template <class S, int G, int RL, bool CHEB>
-__device__ __forceinline__ void site_kernel(const D32 &a, unsigned bx, unsigned by)
+template <class S, bool CHEB>
+__device__ __forceinline__ void finish_site(const D32 &a, int64_t off, int s, cf acc[12])
 {
-    constexpr int SPB = 128 / RL;   // sites per block
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int rl = RL > 1 ? (lane % RL) : 0;
-    const int sl = RL > 1 ? (lane / RL) : lane;
-    const int s = (int)bx * SPB + warp * (32 / RL) + sl;
-    const int r0 = (int)by * (RL * G) + rl * G;
-    if (s >= (int)a.g.Ns || r0 >= a.nrhs) return;
-    const int nr = min(G, a.nrhs - r0);
-    const Site c = site_of(a.g, s);
-    const bool mir = c.x >= a.g.L;
+    if (a.gamma5) {
+#pragma unroll
+        for (int i = 6; i < 12; ++i) acc[i] = cneg(acc[i]);
+    }
+    if (CHEB) {
+        cf yv[12], xv[12];
+        S::ld(a.y + off, s, yv);
+        S::ld(a.x + off, s, xv);
+        const float cc = a.coef ? __ldg(a.coef) : a.c;
+        const float s1 = a.coef ? __ldg(a.coef + 1) : a.s1;
+        const float s2 = a.coef ? __ldg(a.coef + 2) : a.s2;
+#pragma unroll
+        for (int i = 0; i < 12; ++i)
+            acc[i] = fma2(dup(s1), fma2(dup(-cc), yv[i], acc[i]), mul2(dup(-s2), xv[i]));
+    }
+    S::st(a.out + off, s, acc);
+}
 
-    cf acc[G][12];
+// physical site p and its mirror, right-hand side r
+template <class S, bool CHEB>
+__device__ __forceinline__ void site_kernel(const D32 &a, int p, int r)
+{
+    const int row = p / a.g.L;
+    const Site c = site_of(a.g, p + row * a.g.L);   // x < L: s = row 2L + x, p = row L + x
+    const int64_t off = (int64_t)r * a.vbytes;
+    const char *in = a.in + off;
+
+    cf acc[12], accm[12];
     {
         // diagonal part (4 + m0 + A) psi, one chiral block at a time
-        cf v[G][12];
-#pragma unroll
-        for (int g = 0; g < G; ++g) {
-            if (g < nr) S::ld(a.in + (int64_t)(r0 + g) * a.vbytes, s, v[g]);
-            else {
-#pragma unroll
-                for (int i = 0; i < 12; ++i) v[g][i] = make_float2(0.f, 0.f);
-            }
-            const float dm = a.dmdev ? __ldg(a.dmdev + (g < nr ? r0 + g : r0)) : a.dm[g < nr ? r0 + g : r0];
-#pragma unroll
-            for (int i = 0; i < 12; ++i) acc[g][i] = make_float2(dm * v[g][i].x, dm * v[g][i].y);
-        }
+        const float dm = a.dmdev ? __ldg(a.dmdev + r) : a.dm[r];
         const int64_t V = a.g.Vphys;
 #pragma unroll
         for (int b = 0; b < 2; ++b) {
-            cf P[18];
+            cf P[18], v[6];
 #pragma unroll
-            for (int q = 0; q < 18; ++q) P[q] = __ldg(a.clov + (int64_t)(b * 18 + q) * V + c.p);
-            sw_row<0, G>(P, mir, b, v, acc);
-            sw_row<1, G>(P, mir, b, v, acc);
-            sw_row<2, G>(P, mir, b, v, acc);
-            sw_row<3, G>(P, mir, b, v, acc);
-            sw_row<4, G>(P, mir, b, v, acc);
-            sw_row<5, G>(P, mir, b, v, acc);
+            for (int q = 0; q < 18; ++q) P[q] = __ldg(a.clov + (int64_t)(b * 18 + q) * V + p);
+            S::ld6(in, c.s, b, v);
+            sw_block<false>(P, dm, v, acc + 6 * b);
+            S::ld6(in, c.s + a.g.L, b, v);
+            sw_block<true>(P, dm, v, accm + 6 * b);
         }
     }
-    hop<0, +1, S, G>(a, c, mir, r0, nr, acc);
-    hop<0, -1, S, G>(a, c, mir, r0, nr, acc);
-    hop<1, +1, S, G>(a, c, mir, r0, nr, acc);
-    hop<1, -1, S, G>(a, c, mir, r0, nr, acc);
-    hop<2, +1, S, G>(a, c, mir, r0, nr, acc);
-    hop<2, -1, S, G>(a, c, mir, r0, nr, acc);
-    hop<3, +1, S, G>(a, c, mir, r0, nr, acc);
-    hop<3, -1, S, G>(a, c, mir, r0, nr, acc);
-
-#pragma unroll
-    for (int g = 0; g < G; ++g) {
-        if (g < nr) {
-            if (a.gamma5) {
-#pragma unroll
-                for (int i = 6; i < 12; ++i) acc[g][i] = cneg(acc[g][i]);
-            }
-            const int64_t off = (int64_t)(r0 + g) * a.vbytes;
-            if (CHEB) {
-                cf yv[12], xv[12];
-                S::ld(a.y + off, s, yv);
-                S::ld(a.x + off, s, xv);
-                const float cc = a.coef ? __ldg(a.coef) : a.c;
-                const float s1 = a.coef ? __ldg(a.coef + 1) : a.s1;
-                const float s2 = a.coef ? __ldg(a.coef + 2) : a.s2;
-#pragma unroll
-                for (int i = 0; i < 12; ++i) {
-                    acc[g][i].x = s1 * fmaf(-cc, yv[i].x, acc[g][i].x) - s2 * xv[i].x;
-                    acc[g][i].y = s1 * fmaf(-cc, yv[i].y, acc[g][i].y) - s2 * xv[i].y;
-                }
-            }
-            S::st(a.out + off, s, acc[g]);
-        }
-    }
+    Hop h;
+    typename S::Raw v;
+    hop_begin<0>(a, c, h);
+    S::fetch(in, h.n, v);
+    hops<0, S>(a, c, in, h, v, acc, accm);
+    finish_site<S, CHEB>(a, off, c.s, acc);
+    finish_site<S, CHEB>(a, off, c.s + a.g.L, accm);
 }
 
-// One-dimensional grid over (site tile, right-hand-side group).  SITE_MAJOR: the groups
-// of a site tile are consecutive blocks, so a tile's links and SW terms leave DRAM once
-// for all right-hand sides (the time-slice window of all of them must then fit in L2);
-// otherwise the groups are outermost (a window of one group only, links re-read per group).
-template <class S, int G, int RL, bool CHEB, int MINB, bool SITE_MAJOR>
-__global__ void __launch_bounds__(128, MINB) dslash32_kernel(const __grid_constant__ D32 a, unsigned ntile,
-                                                             unsigned ngroup)
+// A block's NT / 32 warps are WR right-hand sides x (NT / 32 / WR) groups of 32 physical sites;
+// it computes `gpb` groups of WR right-hand sides one after the other.
+template <class S, bool CHEB, int NT, int MINB>
+__global__ void __launch_bounds__(NT, MINB) dslash32_kernel(const __grid_constant__ D32 a, unsigned nchunk, int lwr,
+                                                            int gpb)
 {
-    const unsigned b = blockIdx.x;
-    if (SITE_MAJOR) site_kernel<S, G, RL, CHEB>(a, b / ngroup, b % ngroup);
-    else site_kernel<S, G, RL, CHEB>(a, b % ntile, b / ntile);
+    const unsigned tile = blockIdx.x / nchunk, chunk = blockIdx.x % nchunk;
+    const int w = threadIdx.x >> 5, wr = 1 << lwr;
+    const int p = (int)((tile * (NT / 32 >> lwr) + (w >> lwr)) * 32 + (threadIdx.x & 31));
+    if (p >= (int)a.g.Vphys) return;
+    int r = (int)(chunk * gpb) * wr + (w & (wr - 1));
+    for (int i = 0; i < gpb && r < a.nrhs; ++i, r += wr) site_kernel<S, CHEB>(a, p, r);
 }
 
-// Batched persistent form: work items (lattice i, right-hand-side group, site tile)
-// numbered lattice by lattice, right-hand-side groups outermost within a lattice;
-// each block takes items w = blockIdx.x, blockIdx.x + gridDim.x, ...
-#define QS_B_RL 4
+// Batched persistent form: work items (lattice i, site tile, right-hand side) numbered
+// lattice by lattice, right-hand sides fastest; each block takes items w = blockIdx.x,
+// blockIdx.x + gridDim.x, ...
 struct D32B {
     int n;
     unsigned off[QS_BATCH_MAX + 1];   // first work item of lattice i; off[n] = all items
-    unsigned nbx[QS_BATCH_MAX];       // site tiles of lattice i
     D32 item[QS_BATCH_MAX];
 };
 
@@ -438,7 +500,8 @@ __global__ void __launch_bounds__(128, 3) dslash32_batch_kernel(const __grid_con
 #pragma unroll 1
         while (i + 1 < b.n && w >= b.off[i + 1]) ++i;
         const unsigned local = w - b.off[i];
-        site_kernel<S, 1, QS_B_RL, false>(b.item[i], local % b.nbx[i], local / b.nbx[i]);
+        const int p = (int)(local / (unsigned)b.item[i].nrhs) * 128 + (int)threadIdx.x;
+        if (p < (int)b.item[i].g.Vphys) site_kernel<S, false>(b.item[i], p, (int)(local % (unsigned)b.item[i].nrhs));
     }
 }
 
@@ -491,29 +554,34 @@ cudaError_t convert_from(int to, const void *in, void *out, int64_t Ns, int k, c
 }
 
 // ---- launch ------------------------------------------------------------------
-template <class S, int G, int RL, bool CHEB, int MINB, bool SM>
-cudaError_t launch(const D32 &a, cudaStream_t st)
+template <class S, bool CHEB, int NT, int MINB>
+cudaError_t launch(const D32 &a, int lwr, int gpb, cudaStream_t st)
 {
-    constexpr int SPB = 128 / RL;
-    const unsigned ntile = (unsigned)((a.g.Ns + SPB - 1) / SPB);
-    const unsigned ngroup = (unsigned)((a.nrhs + RL * G - 1) / (RL * G));
-    dslash32_kernel<S, G, RL, CHEB, MINB, SM><<<ntile * ngroup, 128, 0, st>>>(a, ntile, ngroup);
+    const int spb = NT >> lwr, ngroup = (a.nrhs + (1 << lwr) - 1) >> lwr;
+    if (gpb > ngroup) gpb = ngroup;
+    const unsigned ntile = (unsigned)((a.g.Vphys + spb - 1) / spb);
+    const unsigned nchunk = (unsigned)((ngroup + gpb - 1) / gpb);
+    dslash32_kernel<S, CHEB, NT, MINB><<<ntile * nchunk, NT, 0, st>>>(a, nchunk, lwr, gpb);
     return cudaGetLastError();
 }
 
-// variant table per storage: (G, RL, min blocks per SM, block order)
+// variant table: threads per block and blocks per SM (168 registers a thread in all), right-hand
+// sides side by side in a block (1 << lwr), groups of them one after the other (gpb).  Right-hand
+// sides side by side or in turn read a site's links and SW words from L1 instead of L2, which
+// pays from about 16 vectors on a lattice that fills the chip (16^3 x 32, 16 vectors, FP32: 298
+// against 308 us); small blocks of one vector spread small problems over the SMs and keep the
+// neighbour rows of large ones close (12^3 x 24, 8 vectors: 62 against 64 us; 32^3 x 64, 24
+// vectors, FP16: 7.4 against 7.8 ms).
 template <class S, bool CHEB>
 cudaError_t launch_variant(int v, const D32 &a, cudaStream_t st)
 {
     switch (v) {
-    case 0: return launch<S, 1, 1, CHEB, 3, false>(a, st);
-    case 1: return launch<S, 1, 4, CHEB, 4, false>(a, st);
-    case 2: return launch<S, 2, 4, CHEB, 3, false>(a, st);
-    case 3: return launch<S, 1, 8, CHEB, 4, false>(a, st);
-    case 4: return launch<S, 1, 1, CHEB, 3, true>(a, st);
-    case 5: return launch<S, 1, 4, CHEB, 4, true>(a, st);
-    case 6: return launch<S, 2, 1, CHEB, 3, true>(a, st);
-    default: return launch<S, 2, 4, CHEB, 3, true>(a, st);
+    case 0: return launch<S, CHEB, 64, 6>(a, 0, 1, st);
+    case 1: return launch<S, CHEB, 32, 12>(a, 0, 1, st);
+    case 2: return launch<S, CHEB, 128, 3>(a, 0, 1, st);
+    case 3: return launch<S, CHEB, 128, 3>(a, 1, 64, st);
+    case 4: return launch<S, CHEB, 128, 3>(a, 2, 64, st);
+    default: return launch<S, CHEB, 384, 1>(a, 2, 64, st);
     }
 }
 
@@ -566,10 +634,8 @@ cudaError_t qs_d32_batch_launch(const D32BatchItem *items, int n, int storage, i
         a.c = a.s1 = a.s2 = 0.f;
         a.coef = a.dmdev = nullptr;
         for (int r = 0; r < it.nrhs; ++r) a.dm[r] = (float)(4.0 + it.m0[r]);
-        const unsigned spb = 128 / QS_B_RL;
-        b.nbx[i] = (unsigned)((it.g.Ns + spb - 1) / spb);
         b.off[i] = off;
-        const double items_i = (double)b.nbx[i] * ((it.nrhs + QS_B_RL - 1) / QS_B_RL);
+        const double items_i = (double)((it.g.Vphys + 127) / 128) * it.nrhs;
         if (off + items_i > 4e9) return cudaErrorInvalidValue;
         off += (unsigned)items_i;
     }
@@ -586,7 +652,7 @@ cudaError_t qs_d32_batch_launch(const D32BatchItem *items, int n, int storage, i
     return e;
 }
 
-int qs_d32_nvariants() { return 8; }
+int qs_d32_nvariants() { return 6; }
 
 int64_t qs_d32_vec_bytes(int storage, int64_t Ns)
 {
