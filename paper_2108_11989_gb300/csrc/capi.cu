@@ -310,7 +310,7 @@ static int run64(qs_lattice *lat, const double *m0, const void *in, void *out, i
     DslashArgs<double> d = make_args64(lat, m0, in, out, nrhs, gamma5);
     int &tv = lat->tuned64[soa ? 1 : 0][nrhs];
     if (tv == 0) {
-        const std::string key = tune_key(lat, "dslash64", soa, 0, nrhs);
+        const std::string key = tune_key(lat, "dslash64s", soa, 0, nrhs);
         int v = tune_lookup(key);
         if (v < 0 || v >= qs_dslash_nvariants<double>()) {
             if (capturing(lat->stream)) {
@@ -513,7 +513,7 @@ static int batch64(const qs_batch_item *items, int n, int tiled, cudaStream_t st
         it.nrhs = items[i].nrhs;
         for (int r = 0; r < it.nrhs; ++r) it.m0[r] = items[i].m0[r];
         a.off[i] = off;
-        double nb = (double)((lat->g.Ns + 127) / 128) * it.nrhs;
+        double nb = (double)((lat->g.Ns + 63) / 64) * it.nrhs;   // 64 sites a block
         if (off + nb > 2147483647.0) return QS_EINVAL;
         off += (unsigned)nb;
     }

@@ -11,7 +11,7 @@ template <> struct LinkT<float> { typedef float2 T; };
 template <typename R>
 struct DslashArgs {
     Geom g;
-    const typename LinkT<R>::T *links;   // [mu][9][Vphys]
+    const typename LinkT<R>::T *links;   // [mu][9][Vphys], times -1/2
     const R *clov;                        // [72][Vphys]
     const R *in;                          // [nrhs][Ns][24]
     R *out;
@@ -57,7 +57,7 @@ enum { QS_D32_F32_TILED = 0, QS_D32_F32_CANON = 1, QS_D32_F16 = 2, QS_D32_BF16 =
 
 struct D32Call {
     Geom g;
-    const float2 *links;   // [mu][9][Vphys] FP32
+    const float2 *links;   // [mu][9][Vphys] FP32, times -1/2
     const float2 *clov;    // [2][18][Vphys] FP32 pairs (packed SW blocks)
     const void *in;        // nrhs vectors, vector r at in + r * qs_d32_vec_bytes(storage, Ns)
     void *out;

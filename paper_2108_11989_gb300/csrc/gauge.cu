@@ -150,8 +150,8 @@ __global__ void clover_build_kernel(Geom g, const double2 *su3, const double *th
     }
 }
 
-// V = U exp(i theta) into the SoA layout [mu][9][Vphys], FP64, and -V / 2 in FP32 (the
-// hopping term's factor, exact).
+// -V / 2, V = U exp(i theta), into the SoA layout [mu][9][Vphys], FP64 and FP32 (the factor
+// of the hopping term, exact).
 __global__ void pack_links_kernel(Geom g, const double2 *su3, const double *th, double2 *l64, float2 *l32)
 {
     int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
@@ -163,7 +163,7 @@ __global__ void pack_links_kernel(Geom g, const double2 *su3, const double *th, 
             double2 u = su3[(p * 4 + mu) * 9 + k];
             double2 v = make_double2(u.x * c - u.y * sn, u.x * sn + u.y * c);
             int64_t o = (int64_t)(mu * 9 + k) * g.Vphys + p;
-            l64[o] = v;
+            l64[o] = make_double2(-0.5 * v.x, -0.5 * v.y);
             l32[o] = make_float2((float)(-0.5 * v.x), (float)(-0.5 * v.y));
         }
     }

@@ -43,7 +43,7 @@ struct qs_lattice {
     int gauge_loaded;
     double csw_su3, csw_u1;
     double clov_norm;      // max over sites of ||A(x)||_F (bounds ||A(x)||)
-    // V = U exp(i theta) on the physical lattice, SoA [mu][9][Vphys] complex (links32: -V / 2)
+    // -V / 2, V = U exp(i theta), on the physical lattice, SoA [mu][9][Vphys] complex
     double2 *links64;
     float2 *links32;
     // SW term A on the physical lattice (two packed 6x6 Hermitian blocks); the mirror

@@ -1,10 +1,11 @@
-"""Every launch variant of the FP32-arithmetic operator against the oracle.
+"""Every launch variant of the operator against the oracle.
 
 The autotuner picks one variant per shape, so each is forced in turn (a child process with a
 tune cache that names it) on lattices whose sites fill no block (2^3 x 3: 24 physical sites,
 6^3 x 5: 1080) and on blocks of vectors that fill no group of 2 or 4.  Tolerances, max-norm
 relative to the largest output component: 1e-5 for FP32 storage; for FP16 storage half a unit
-in the last place at 1 relative to the site's largest component (2^-11), twice that allowed.
+in the last place at 1 relative to the site's largest component (2^-11), twice that allowed.  FP64: 1e-13 (about 300 roundings of
+2^-53 each on the longest chain, of terms no larger than the output's scale).
 """
 import os
 import subprocess
@@ -67,3 +68,45 @@ def test_forced_variant_matches_oracle(variant, tmp_path):
                        env=dict(os.environ, QS_TUNE_CACHE=str(cache)), capture_output=True, text=True, timeout=300)
     assert r.returncode == 0, r.stderr[-2000:]
     assert len(cache.read_text().splitlines()) == len(SHAPES) * len(NRHS) * 4   # nothing was timed: the forced one ran
+
+
+CHILD64 = r"""
+import sys
+sys.path[:0] = [%(root)r, %(root)r + "/tests"]
+import numpy as np
+import torch
+import paper_2108_11989_gb300 as qs
+from oracle.dirac import WilsonDirac
+from synth_inputs import make_config, random_spinor
+for L, T, mask, anti in %(shapes)r:
+    cfg = make_config(T=T, L=L, eps=0.6, theta_sigma=0.4, csw_su3=1.9, csw_u1=1.0, seed=3, cstar_mask=mask,
+                      t_antiperiodic=anti)
+    lat = qs.Lattice(L, T, mask, anti)
+    lat.load_gauge(cfg.su3, cfg.theta, cfg.csw_su3, cfg.csw_u1)
+    op, ns = WilsonDirac(cfg), cfg.n_sites
+    for nrhs in %(nrhs)r:
+        psi = random_spinor(7, T, L, nrhs)
+        ref = np.stack([op.apply_D(psi[r].reshape(-1), 0.07) for r in range(nrhs)]).reshape(nrhs, ns, 12)
+        x = torch.from_numpy(np.ascontiguousarray(psi).view(np.float64).copy()).cuda().reshape(-1)
+        for tiled in (False, True):
+            xin = qs.to_tiled(x, ns) if tiled else x
+            y = torch.full_like(xin, float("nan"))
+            lat.apply_Dw(0.07, xin, y, tiled=tiled)
+            y = qs.from_tiled(y, ns) if tiled else y
+            got = y.cpu().numpy().view(np.complex128).reshape(nrhs, ns, 12)
+            assert np.abs(got - ref).max() <= 1e-13 * np.abs(ref).max(), (L, T, nrhs, tiled)
+    lat.close()
+"""
+
+
+@pytest.mark.parametrize("variant", range(3))
+def test_forced_fp64_variant_matches_oracle(variant, tmp_path):
+    import torch
+    gpu = torch.cuda.get_device_name(0).replace(" ", "_")
+    cache = tmp_path / "tune"
+    cache.write_text("".join(f"{gpu}|dslash64s|{soa}|0|{n}|{L}x{T} {variant}\n"
+                             for L, T, _, _ in SHAPES for n in NRHS for soa in range(2)))
+    r = subprocess.run([sys.executable, "-c", CHILD64 % {"root": ROOT, "shapes": SHAPES, "nrhs": NRHS}],
+                       env=dict(os.environ, QS_TUNE_CACHE=str(cache)), capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0, r.stderr[-2000:]
+    assert len(cache.read_text().splitlines()) == len(SHAPES) * len(NRHS) * 2
