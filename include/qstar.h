@@ -329,8 +329,8 @@ QS_API int qs_ratapprox(int n, double ra, double rb, double *A, double *nu, doub
  * Shifted inverses: FP64 conjugate gradients on Q_hat^2 + shift^2, each to
  * ||r|| <= tol ||b||, at most max_iter iterations (QS_ENOCONV beyond).  q: HOST array of
  * n * nsrc; log_w, cg_iterations (total over all solves): HOST, may be NULL.  Allocates
- * 12 nsrc vectors of work and the odd-site block inverses at m and m' (2 x 1152 bytes per
- * odd physical site); synchronises the lattice's stream.  QS_EINVAL for odd T or L. */
+ * 10 nsrc half-lattice vectors of work and the odd-site block inverses at m and m' (2 x 1152
+ * bytes per odd physical site); synchronises the lattice's stream.  QS_EINVAL for odd T or L. */
 QS_API int qs_w_mass(qs_lattice *lat, double m, double mp, int n, const double *nu, const double *mu,
                      const void *eta, int nsrc, double tol, int max_iter, double *q, double *log_w,
                      int *cg_iterations);
@@ -341,8 +341,9 @@ QS_API int qs_w_mass(qs_lattice *lat, double m, double mp, int n, const double *
  * T and L.  even_odd = 0: conjugate gradients on the full-lattice Q^2 (for comparison).
  * b, x: DEVICE buffers of nrhs <= 64 FP64 spinors, canonical layout, not overlapping.  The CG
  * stops at ||r|| <= tol ||rhs|| for every right-hand side (QS_ENOCONV after max_iter);
- * *iterations (may be NULL) gets the count.  Allocates 11 nrhs vectors of work (plus the
- * odd-site inverses, 1152 bytes per odd physical site); synchronises the stream. */
+ * *iterations (may be NULL) gets the count.  Allocates 9 nrhs vectors of work (half-lattice ones
+ * with even_odd, plus the odd-site inverses, 1152 bytes per odd physical site); synchronises
+ * the stream. */
 QS_API int qs_solve_D(qs_lattice *lat, double m0, const void *b, void *x, int nrhs, int even_odd, double tol,
                       int max_iter, int *iterations);
 
@@ -386,8 +387,9 @@ QS_API int qs_w_eo(qs_lattice *lat, double m, double mp, double *w_eo, double *l
  * D_hat = D_ee - D_eo (D_oo)^-1 D_oe on the even sites (gamma5 = 1: Q_hat = gamma_5 D_hat).
  * in, out: DEVICE buffers of nrhs <= 64 FP64 spinors in the canonical layout of the full
  * doubled lattice; the odd-site entries of in are ignored and those of out set to zero.
- * FP64 arithmetic (two operator applications and a site-local 6 x 6 solve per odd site);
- * allocates three work vectors per call; synchronises the stream.  QS_EINVAL for an odd T
+ * FP64 arithmetic (two half-lattice operator applications and a site-local 6 x 6 inverse per odd site);
+ * allocates a work vector of the odd sites and the odd-site block inverses (1152 bytes per odd
+ * physical site) per call; synchronises the stream.  QS_EINVAL for an odd T
  * or L (then a hop can join two sites of one parity), overlapping or unaligned buffers.  det D = det D_oo det D_hat,
  * which is why W_eo carries the D_oo part of a mass reweighting. */
 QS_API int qs_apply_Dhat(qs_lattice *lat, double m0, const void *in, void *out, int nrhs, int gamma5);

@@ -57,28 +57,6 @@ __global__ void __launch_bounds__(128, 4) dslash_batch_kernel(const __grid_const
     dslash_site<AT>(it.g, it.links, it.clov, it.in, it.out, a.gamma5, it.m0[r], r, s);
 }
 
-// The FP64 operator on the sites of one parity only ((t + z + y + x) mod 2 == parity);
-// sites of the other parity get zeros.  Site j of that parity lies in row j / L (a row of 2L
-// sites holds L of each, at x = 2 jx or 2 jx + 1); its threads also zero the other site of its
-// x pair.
-__global__ void __launch_bounds__(128, 4) dslash64_parity_kernel(DslashArgs<double> a, int parity)
-{
-    const unsigned b = blockIdx.x;
-    const int r = (int)(b % (unsigned)a.nrhs);
-    const int j = (int)(b / (unsigned)a.nrhs) * 64 + (int)(threadIdx.x >> 5) * 16 + (int)(threadIdx.x & 15);
-    const bool on = j < (int)(a.g.Ns / 2);
-    const int row = (on ? j : 0) / a.g.L;
-    const int jx = (on ? j : 0) - row * a.g.L;
-    const int y = row % a.g.L, z = (row / a.g.L) % a.g.L, t = row / (a.g.L * a.g.L);
-    const int s = row * a.g.L2 + 2 * jx + ((parity + t + z + y) & 1);
-    if (on) {
-        double2 *o = (double2 *)(a.out + ((int64_t)r * a.g.Ns + (s ^ 1)) * 24) + ((threadIdx.x & 16) ? 6 : 0);
-#pragma unroll
-        for (int i = 0; i < 6; ++i) o[i] = make_double2(0.0, 0.0);
-    }
-    dslash_site<At64Canon>(a.g, a.links, a.clov, a.in, a.out, a.gamma5, a.m0[r], r, on ? s : (int)a.g.Ns);
-}
-
 template <int NT, int MINB>
 cudaError_t launch_variant(const DslashArgs<double> &a, int soa, cudaStream_t st)
 {
@@ -104,13 +82,6 @@ cudaError_t qs_dslash_launch<double>(DslashArgs<double> a, int nrhs, int variant
     case 1: return launch_variant<128, 3>(a, soa, st);
     default: return launch_variant<128, 4>(a, soa, st);
     }
-}
-
-cudaError_t qs_dslash64_parity_launch(const DslashArgs<double> &a, int parity, cudaStream_t st)
-{
-    const int64_t nb = ((a.g.Ns / 2 + 63) / 64) * a.nrhs;
-    dslash64_parity_kernel<<<(unsigned)nb, 128, 0, st>>>(a, parity);
-    return cudaGetLastError();
 }
 
 // canonical [site][12][re, im] <-> solver [site / 16][12][site % 16][re, im], per vector

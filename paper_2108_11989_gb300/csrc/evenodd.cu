@@ -8,6 +8,7 @@
 // sites and counts each twice.  One thread per physical site, a complex LU with
 // partial pivoting per block in FP64, then a fixed-order two-stage sum.
 #include "blas.cuh"
+#include "dslash64.cuh"
 #include "evenodd.cuh"
 
 #include <math.h>
@@ -142,366 +143,341 @@ extern "C" int qs_w_eo(qs_lattice *lat, double m, double mp, double *w_eo, doubl
 }
 
 // ---- the even-odd preconditioned operator (Sec. 4) --------------------------------
-// D_hat = D_ee - D_eo (D_oo)^-1 D_oe on the even sites, Q_hat = gamma_5 D_hat.  With x the
-// even part of the input (odd entries zero): (D x)_e = D_ee x_e and (D x)_o = D_oe x_e, so
-//   D_hat x_e = (D x)_e - (D u)_e,  u = (D_oo)^-1 (D x)_o  (u zero on even sites),
-// two applications of the full FP64 operator, a site-local solve and parity masks.
+// D_hat = D_ee - D_eo (D_oo)^-1 D_oe on the even sites, Q_hat = gamma_5 D_hat, in two passes:
+//   v_o = -(D_oo)^-1 (D_oe x_e)  (hops, then the stored 6 x 6 inverses of the odd sites),
+//   D_hat x_e = D_ee x_e + D_eo v_o.
+// Vectors of one parity are stored alone, N_s / 2 sites in the site-tiled layout (site j of a
+// parity is site s / 2 of the doubled lattice: a row of 2L sites holds L of each), so nothing
+// is moved or computed for the other parity and the first pass has no SW term.  Bound by the
+// FP64 pipe: 840 + 288 instructions per odd site and 1164 per even one, against 2 x 1650 + 430
+// for two full-lattice site computations and a separate inverse.
+// D_hat on 8^3 x 16, 2 vectors: 2 x (75 + 26) + 8 us before, see qs_solve_D for the solves.
 namespace {
 
-__device__ __forceinline__ int site_parity(const Geom &g, int64_t s)
+struct Hat64 {
+    Geom g;
+    const double2 *links;
+    const double *clov;
+    const double2 *inv;
+    int nrhs, gamma5;
+    double dm;
+    const int *live;      // NULL, or right-hand sides with live[r] = 0 are skipped
+    // even pass: out += sigma add, part[r][tile] = Re (add, out)
+    const double2 *add;
+    double sigma;
+    double *part;
+};
+
+// doubled site of the j-th site of a parity
+__device__ __forceinline__ int parity_site(const Geom &g, int j, int parity)
 {
-    const int x = (int)(s % g.L2);
-    int64_t r = s / g.L2;
-    const int y = (int)(r % g.L);
-    r /= g.L;
-    const int z = (int)(r % g.L);
-    const int t = (int)(r / g.L);
-    return (t + z + y + x) & 1;
+    const int row = j / g.L, jx = j - row * g.L;
+    const int y = row % g.L, z = (row / g.L) % g.L, t = row / (g.L * g.L);
+    return row * g.L2 + 2 * jx + ((parity + t + z + y) & 1);
 }
 
-// out = in on sites of parity `keep`, 0 elsewhere (canonical FP64 layout, k vectors)
-__global__ void parity_mask_kernel(const double2 *__restrict__ in, double2 *__restrict__ out, Geom g, int k,
-                                   int keep)
+// rows of spin q of f (4 + m0 + A)^-1 v for chiral block b (stored inverse M; the mirror site's is
+// S conj(M) S), v = own (spin q) and oth
+__device__ __forceinline__ void inv_rows(const double2 *__restrict__ inv, int64_t V2, int64_t q, int b, double f,
+                                         const Lane64 &ln, const double2 own[3], const double2 oth[3], double2 out[3])
 {
-    const int64_t n = g.Ns * 12 * k;
-    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const int64_t s = (i / 12) % g.Ns;
-    out[i] = site_parity(g, s) == keep ? in[i] : make_double2(0, 0);
-}
-
-// v = x on even sites and v = -(4 + m0 + A(x))^-1 t on odd sites (two 6 x 6 chiral blocks,
-// complex Gaussian elimination with partial pivoting in FP64); one thread per (vector, site).
-// The mirror site's block is S conj(A) S: entry (i, j) = sign * conj(A[i +- 3][j +- 3]),
-// sign = -1 across the two spin halves.
-__global__ void clover_solve_odd_kernel(const double *__restrict__ clov, const double2 *__restrict__ t,
-                                        const double2 *__restrict__ xe, double2 *__restrict__ u, Geom g, int k,
-                                        double dm)
-{
-    const int64_t n = g.Ns * k;
-    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const int64_t s = i % g.Ns;
-    const double2 *ti = t + i * 12;
-    double2 *ui = u + i * 12;
-    if (site_parity(g, s) == 0) {
-        const double2 *xi = xe + i * 12;
-        for (int c = 0; c < 12; ++c) ui[c] = xi[c];
-        return;
+    const int hq = ln.q ^ (ln.mir ? 1 : 0);
+    const double2 *m = inv + ((int64_t)b * 36 + 18 * hq) * V2 + q;
+#pragma unroll
+    for (int r = 0; r < 3; ++r) {
+        double2 o;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            double2 e = __ldg(m + (int64_t)(6 * r + 3 * hq + c) * V2);
+            e.y = qs_flip(e.y, ln.mir);
+            o = c == 0 ? qs_cmul(e, own[c]) : qs_cfma(e, own[c], o);
+        }
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            double2 e = __ldg(m + (int64_t)(6 * r + 3 - 3 * hq + c) * V2);
+            e.x = qs_flip(e.x, ln.mir);
+            o = qs_cfma(e, oth[c], o);
+        }
+        out[r] = make_double2(f * o.x, f * o.y);
     }
-    const int x = (int)(s % g.L2);
-    const bool mir = x >= g.L;
-    const int64_t p = (s / g.L2) * g.L + (mir ? x - g.L : x);
-    const int64_t V = g.Vphys;
+}
+
+__device__ __forceinline__ double2 partner_spin(double2 v)
+{
+    return make_double2(__shfl_xor_sync(0xffffffffu, v.x, 16), __shfl_xor_sync(0xffffffffu, v.y, 16));
+}
+
+// out_o = f (D_oo)^-1 (D_oe in_e) (HOP) or f (D_oo)^-1 in_o; in by AT, out tiled by parity
+template <class AT, bool HOP>
+__global__ void __launch_bounds__(128, 4) hat_odd_kernel(const __grid_constant__ Hat64 a, const double2 *__restrict__ in,
+                                                         int64_t in_len, double2 *__restrict__ out, double f)
+{
+    const int r = (int)(blockIdx.x % (unsigned)a.nrhs);
+    if (a.live && !a.live[r]) return;
+    const int nh = (int)(a.g.Ns / 2);
+    const int j0 = (int)(blockIdx.x / (unsigned)a.nrhs) * 64 + (int)(threadIdx.x >> 5) * 16 + (int)(threadIdx.x & 15);
+    const int j = j0 < nh ? j0 : nh - 1;
+    const Lane64 ln = qs_lane64(a.g, parity_site(a.g, j, 1));
+    const double2 *v = in + r * in_len;
+    double2 w[2][3];
+    if constexpr (HOP) {
+        qs_hops64<AT>(a.g, a.links, v, ln, w[0], w[1]);
+    } else {
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+            w[0][i] = __ldg(v + AT::at(ln.c.s, 3 * ln.q + i));
+            w[1][i] = __ldg(v + AT::at(ln.c.s, 6 + 3 * ln.q + i));
+        }
+    }
+    double2 *o = out + (int64_t)r * nh * 12;
+#pragma unroll
     for (int b = 0; b < 2; ++b) {
-        const double *cb = clov + (int64_t)b * 36 * V + p;
-        double ar[6][6], ai[6][6], rr[6], ri[6];
-        for (int r = 0; r < 6; ++r)
-            for (int c = 0; c < 6; ++c) {
-                const int ii = mir ? (r + 3) % 6 : r, jj = mir ? (c + 3) % 6 : c;
-                double er, ei;
-                if (ii == jj) { er = cb[(int64_t)ii * V]; ei = 0; }
-                else if (ii > jj) {
-                    const int kk = 6 + 2 * qs_tri(ii, jj);
-                    er = cb[(int64_t)kk * V]; ei = cb[(int64_t)(kk + 1) * V];
-                } else {
-                    const int kk = 6 + 2 * qs_tri(jj, ii);
-                    er = cb[(int64_t)kk * V]; ei = -cb[(int64_t)(kk + 1) * V];
-                }
-                if (mir) {
-                    ei = -ei;
-                    if ((r < 3) != (c < 3)) { er = -er; ei = -ei; }
-                }
-                ar[r][c] = er + (r == c ? dm : 0.0);
-                ai[r][c] = ei;
-            }
-        for (int r = 0; r < 6; ++r) { rr[r] = ti[6 * b + r].x; ri[r] = ti[6 * b + r].y; }
-        for (int c = 0; c < 6; ++c) {
-            int piv = c;
-            double best = ar[c][c] * ar[c][c] + ai[c][c] * ai[c][c];
-            for (int r = c + 1; r < 6; ++r) {
-                const double a2 = ar[r][c] * ar[r][c] + ai[r][c] * ai[r][c];
-                if (a2 > best) { best = a2; piv = r; }
-            }
-            if (piv != c) {
-                for (int j = 0; j < 6; ++j) {
-                    double tt = ar[c][j]; ar[c][j] = ar[piv][j]; ar[piv][j] = tt;
-                    tt = ai[c][j]; ai[c][j] = ai[piv][j]; ai[piv][j] = tt;
-                }
-                double tt = rr[c]; rr[c] = rr[piv]; rr[piv] = tt;
-                tt = ri[c]; ri[c] = ri[piv]; ri[piv] = tt;
-            }
-            const double ir = ar[c][c] / best, ii2 = -ai[c][c] / best;   // 1 / pivot
-            for (int r = c + 1; r < 6; ++r) {
-                const double lr = ar[r][c] * ir - ai[r][c] * ii2, li = ar[r][c] * ii2 + ai[r][c] * ir;
-                for (int j = c; j < 6; ++j) {
-                    ar[r][j] -= lr * ar[c][j] - li * ai[c][j];
-                    ai[r][j] -= lr * ai[c][j] + li * ar[c][j];
-                }
-                rr[r] -= lr * rr[c] - li * ri[c];
-                ri[r] -= lr * ri[c] + li * rr[c];
-            }
+        double2 oth[3], u[3];
+#pragma unroll
+        for (int i = 0; i < 3; ++i) oth[i] = partner_spin(w[b][i]);
+        inv_rows(a.inv, a.g.Vphys / 2, ln.c.p >> 1, b, f, ln, w[b], oth, u);
+        if (j0 < nh) {
+#pragma unroll
+            for (int i = 0; i < 3; ++i) o[At64Tiled::at(j, 6 * b + 3 * ln.q + i)] = u[i];
         }
-        for (int r = 5; r >= 0; --r) {   // back substitution
-            double sr = rr[r], si = ri[r];
-            for (int j = r + 1; j < 6; ++j) {
-                sr -= ar[r][j] * rr[j] - ai[r][j] * ri[j];
-                si -= ar[r][j] * ri[j] + ai[r][j] * rr[j];
-            }
-            const double d2 = ar[r][r] * ar[r][r] + ai[r][r] * ai[r][r];
-            rr[r] = (sr * ar[r][r] + si * ai[r][r]) / d2;
-            ri[r] = (si * ar[r][r] - sr * ai[r][r]) / d2;
-        }
-        for (int r = 0; r < 6; ++r) ui[6 * b + r] = make_double2(-rr[r], -ri[r]);
     }
 }
 
-// inv = (4 + m0 + A(x))^-1 for every odd physical site x, both chiral blocks, by Gauss-Jordan
-// elimination with partial pivoting in FP64; layout [block][6][6][V_phys / 2] complex, the odd
-// physical site p at index p / 2 (L is even, so the odd sites of a row of L alternate).  The mirror site's block S conj(M) S has the inverse
-// S conj(M^-1) S, formed on the fly when it is applied.
+// out_e = [gamma_5] (DIAG: (4 + m0 + A) x_e +) D_eo v_o (+ sigma add); v tiled by parity; x and out
+// by AT, which for the full lattice also zeroes the odd site next to each even one.  part != NULL:
+// the block's share of Re (add, out).
+template <class AT, bool DIAG>
+__global__ void __launch_bounds__(128, 4) hat_even_kernel(const __grid_constant__ Hat64 a, const double2 *__restrict__ v,
+                                                          const double2 *__restrict__ x, double2 *__restrict__ out,
+                                                          int64_t len, bool full)
+{
+    const int r = (int)(blockIdx.x % (unsigned)a.nrhs);
+    if (a.live && !a.live[r]) return;
+    const int nh = (int)(a.g.Ns / 2);
+    const unsigned tile = blockIdx.x / (unsigned)a.nrhs;
+    const int j0 = (int)tile * 64 + (int)(threadIdx.x >> 5) * 16 + (int)(threadIdx.x & 15);
+    const int j = j0 < nh ? j0 : nh - 1;
+    const Lane64 ln = qs_lane64(a.g, parity_site(a.g, j, 0));
+    double2 w[2][3];
+    qs_hops64<At64Half>(a.g, a.links, v + (int64_t)r * nh * 12, ln, w[0], w[1]);
+    if constexpr (DIAG) qs_diag64<AT>(a.g, a.clov, x + r * len, ln, a.dm, w[0], w[1]);
+    const unsigned g5 = a.gamma5 ? 0x80000000u : 0u;
+    double acc = 0.0;
+    double2 *o = out + r * len;
+#pragma unroll
+    for (int b = 0; b < 2; ++b)
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+            double2 y = w[b][i];
+            if (b) y = make_double2(qs_flip(y.x, g5), qs_flip(y.y, g5));
+            const int64_t at = AT::at(ln.c.s, 6 * b + 3 * ln.q + i);
+            if (a.add) {
+                const double2 p = __ldg(a.add + r * len + at);
+                y = make_double2(fma(a.sigma, p.x, y.x), fma(a.sigma, p.y, y.y));
+                if (a.part) acc = fma(p.y, y.y, fma(p.x, y.x, acc));
+            }
+            if (j0 < nh) {
+                o[at] = y;
+                if (full) o[AT::at(ln.c.s ^ 1, 6 * b + 3 * ln.q + i)] = make_double2(0.0, 0.0);
+            }
+        }
+    if (a.part) {
+        __shared__ double sh[4];
+        if (j0 >= nh) acc = 0.0;
+        for (int d = 16; d > 0; d >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, d);
+        if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = acc;
+        __syncthreads();
+        if (threadIdx.x == 0) a.part[(int64_t)r * (gridDim.x / a.nrhs) + tile] = (sh[0] + sh[1]) + (sh[2] + sh[3]);
+    }
+}
+
+// canonical full-lattice vectors <-> tiled vectors of one parity; thread = (vector, site, component)
+__global__ void parity_pack_kernel(const double2 *__restrict__ in, double2 *__restrict__ out, Geom g, int k, int parity)
+{
+    const int64_t n = g.Ns / 2 * 12 * k;
+    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    const int64_t r = i / (g.Ns / 2 * 12), e = i - r * (g.Ns / 2 * 12);
+    const int j = (int)(e / 12), c = (int)(e - 12 * (int64_t)j);
+    const int s = parity_site(g, j, parity);
+    out[r * (g.Ns / 2) * 12 + At64Tiled::at(j, c)] = in[(r * g.Ns + s) * 12 + c];
+}
+
+// x on the sites of `parity` of the full lattice = a (- b)
+__global__ void parity_unpack_kernel(const double2 *__restrict__ a, const double2 *__restrict__ b,
+                                     double2 *__restrict__ x, Geom g, int k, int parity)
+{
+    const int64_t n = g.Ns / 2 * 12 * k;
+    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    const int64_t r = i / (g.Ns / 2 * 12), e = i - r * (g.Ns / 2 * 12);
+    const int j = (int)(e / 12), c = (int)(e - 12 * (int64_t)j);
+    const int64_t at = r * (g.Ns / 2) * 12 + At64Tiled::at(j, c);
+    double2 v = a[at];
+    if (b) v = make_double2(v.x - b[at].x, v.y - b[at].y);
+    x[(r * g.Ns + parity_site(g, j, parity)) * 12 + c] = v;
+}
+
+// inv = (4 + m0 + A(x))^-1 for every odd physical site x and chiral block (one thread each), by
+// Gauss-Jordan elimination with partial pivoting in FP64; layout [block][6][6][V_phys / 2]
+// complex, the odd physical site p at index p / 2 (L is even, so the odd sites of a row of L
+// alternate).  The mirror site's block S conj(M) S has the inverse S conj(M^-1) S, formed on
+// the fly when it is applied.
 __global__ void clover_inverse_kernel(const double *__restrict__ clov, Geom g, double dm, double2 *__restrict__ inv)
 {
-    const int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (p >= g.Vphys) return;
-    const int x = (int)(p % g.L);
-    int64_t row = p / g.L;
-    const int y = (int)(row % g.L);
-    row /= g.L;
-    const int z = (int)(row % g.L);
-    const int t = (int)(row / g.L);
-    if (((t + z + y + x) & 1) == 0) return;
-    const int64_t V = g.Vphys;
-    for (int b = 0; b < 2; ++b) {
-        const double *cb = clov + (int64_t)b * 36 * V + p;
-        double ar[6][6], ai[6][6], br[6][6], bi[6][6];
-        for (int i = 0; i < 6; ++i) {
-            ar[i][i] = dm + cb[(int64_t)i * V];
-            ai[i][i] = 0.0;
-            for (int j = 0; j < i; ++j) {
-                const int k = 6 + 2 * qs_tri(i, j);
-                ar[i][j] = cb[(int64_t)k * V];
-                ai[i][j] = cb[(int64_t)(k + 1) * V];
-                ar[j][i] = ar[i][j];      // Hermitian: upper = conj(lower)
-                ai[j][i] = -ai[i][j];
-            }
-            for (int j = 0; j < 6; ++j) { br[i][j] = i == j ? 1.0 : 0.0; bi[i][j] = 0.0; }
+    const int64_t V = g.Vphys, V2 = V / 2;
+    const int64_t i0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (i0 >= 2 * V2) return;
+    const int b = i0 >= V2;
+    const int64_t q = i0 - b * V2;
+    int64_t p = 2 * q;   // the odd one of the sites 2q, 2q + 1 of a row
+    {
+        const int64_t row = p / g.L;
+        const int x = (int)(p - row * g.L);
+        const int y = (int)(row % g.L), z = (int)((row / g.L) % g.L), t = (int)(row / ((int64_t)g.L * g.L));
+        p += ((t + z + y + x) & 1) ? 0 : 1;
+    }
+    const double *cb = clov + (int64_t)b * 36 * V + p;
+    double ar[6][6], ai[6][6], br[6][6], bi[6][6];
+    for (int i = 0; i < 6; ++i) {
+        ar[i][i] = dm + cb[(int64_t)i * V];
+        ai[i][i] = 0.0;
+        for (int j = 0; j < i; ++j) {
+            const int k = 6 + 2 * qs_tri(i, j);
+            ar[i][j] = cb[(int64_t)k * V];
+            ai[i][j] = cb[(int64_t)(k + 1) * V];
+            ar[j][i] = ar[i][j];      // Hermitian: upper = conj(lower)
+            ai[j][i] = -ai[i][j];
         }
-        for (int c = 0; c < 6; ++c) {
-            int piv = c;
-            double best = ar[c][c] * ar[c][c] + ai[c][c] * ai[c][c];
-            for (int r = c + 1; r < 6; ++r) {
-                const double a2 = ar[r][c] * ar[r][c] + ai[r][c] * ai[r][c];
-                if (a2 > best) { best = a2; piv = r; }
-            }
-            if (piv != c)
-                for (int j = 0; j < 6; ++j) {
-                    double q = ar[c][j]; ar[c][j] = ar[piv][j]; ar[piv][j] = q;
-                    q = ai[c][j]; ai[c][j] = ai[piv][j]; ai[piv][j] = q;
-                    q = br[c][j]; br[c][j] = br[piv][j]; br[piv][j] = q;
-                    q = bi[c][j]; bi[c][j] = bi[piv][j]; bi[piv][j] = q;
-                }
-            const double pr = ar[c][c] / best, pim = -ai[c][c] / best;   // 1 / pivot
+        for (int j = 0; j < 6; ++j) { br[i][j] = i == j ? 1.0 : 0.0; bi[i][j] = 0.0; }
+    }
+    for (int c = 0; c < 6; ++c) {
+        int piv = c;
+        double best = ar[c][c] * ar[c][c] + ai[c][c] * ai[c][c];
+        for (int r = c + 1; r < 6; ++r) {
+            const double a2 = ar[r][c] * ar[r][c] + ai[r][c] * ai[r][c];
+            if (a2 > best) { best = a2; piv = r; }
+        }
+        if (piv != c)
             for (int j = 0; j < 6; ++j) {
-                double q = ar[c][j] * pr - ai[c][j] * pim;
-                ai[c][j] = ar[c][j] * pim + ai[c][j] * pr;
-                ar[c][j] = q;
-                q = br[c][j] * pr - bi[c][j] * pim;
-                bi[c][j] = br[c][j] * pim + bi[c][j] * pr;
-                br[c][j] = q;
+                double w = ar[c][j]; ar[c][j] = ar[piv][j]; ar[piv][j] = w;
+                w = ai[c][j]; ai[c][j] = ai[piv][j]; ai[piv][j] = w;
+                w = br[c][j]; br[c][j] = br[piv][j]; br[piv][j] = w;
+                w = bi[c][j]; bi[c][j] = bi[piv][j]; bi[piv][j] = w;
             }
-            for (int r = 0; r < 6; ++r) {
-                if (r == c) continue;
-                const double fr = ar[r][c], fi = ai[r][c];
-                for (int j = 0; j < 6; ++j) {
-                    ar[r][j] -= fr * ar[c][j] - fi * ai[c][j];
-                    ai[r][j] -= fr * ai[c][j] + fi * ar[c][j];
-                    br[r][j] -= fr * br[c][j] - fi * bi[c][j];
-                    bi[r][j] -= fr * bi[c][j] + fi * br[c][j];
-                }
+        const double pr = ar[c][c] / best, pim = -ai[c][c] / best;   // 1 / pivot
+        for (int j = 0; j < 6; ++j) {
+            double w = ar[c][j] * pr - ai[c][j] * pim;
+            ai[c][j] = ar[c][j] * pim + ai[c][j] * pr;
+            ar[c][j] = w;
+            w = br[c][j] * pr - bi[c][j] * pim;
+            bi[c][j] = br[c][j] * pim + bi[c][j] * pr;
+            br[c][j] = w;
+        }
+        for (int r = 0; r < 6; ++r) {
+            if (r == c) continue;
+            const double fr = ar[r][c], fi = ai[r][c];
+            for (int j = 0; j < 6; ++j) {
+                ar[r][j] -= fr * ar[c][j] - fi * ai[c][j];
+                ai[r][j] -= fr * ai[c][j] + fi * ar[c][j];
+                br[r][j] -= fr * br[c][j] - fi * bi[c][j];
+                bi[r][j] -= fr * bi[c][j] + fi * br[c][j];
             }
         }
-        const int64_t V2 = V / 2, q = p >> 1;   // odd sites of a row of L have one index parity each
-        for (int i = 0; i < 6; ++i)
-            for (int j = 0; j < 6; ++j) inv[((int64_t)b * 36 + i * 6 + j) * V2 + q] = make_double2(br[i][j], bi[i][j]);
     }
+    for (int i = 0; i < 6; ++i)
+        for (int j = 0; j < 6; ++j) inv[((int64_t)b * 36 + i * 6 + j) * V2 + q] = make_double2(br[i][j], bi[i][j]);
 }
 
-// v = x on even sites, v = -(4 + m0 + A(x))^-1 t on odd sites from the stored inverses.  Thread
-// j takes the j-th odd site (x = 2 jx or 2 jx + 1 in its row) and copies its even x partner.
-__global__ void clover_apply_inv_kernel(const double2 *__restrict__ inv, const double2 *__restrict__ t,
-                                        const double2 *__restrict__ xe, double2 *__restrict__ v, Geom g, int k)
+Hat64 hat_args(qs_lattice *lat, double m0, int nrhs, int gamma5, const double2 *inv, const int *live)
 {
-    const int64_t half = g.Ns / 2;
-    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i >= half * k) return;
-    const int64_t r = i / half, j = i - r * half;
-    const int64_t row = j / g.L;
-    const int jx = (int)(j - row * g.L);
-    const int y = (int)(row % g.L), z = (int)((row / g.L) % g.L), tt = (int)(row / ((int64_t)g.L * g.L));
-    const int x = 2 * jx + ((1 + tt + z + y) & 1);
-    const int64_t s = row * g.L2 + x;
-    {
-        const int64_t e = (r * g.Ns + (s ^ 1)) * 12;
-        for (int c = 0; c < 12; ++c) v[e + c] = xe[e + c];
-    }
-    const double2 *ti = t + (r * g.Ns + s) * 12;
-    double2 *vi = v + (r * g.Ns + s) * 12;
-    const bool mir = x >= g.L;
-    const int64_t p = row * g.L + (mir ? x - g.L : x);
-    const int64_t V2 = g.Vphys / 2, q = p >> 1;
-    for (int b = 0; b < 2; ++b)
-        for (int rr = 0; rr < 6; ++rr) {
-            double accr = 0, acci = 0;
-            for (int c = 0; c < 6; ++c) {
-                const int ii = mir ? (rr + 3) % 6 : rr, jj = mir ? (c + 3) % 6 : c;
-                double2 e = inv[((int64_t)b * 36 + ii * 6 + jj) * V2 + q];
-                if (mir) {
-                    e.y = -e.y;
-                    if ((rr < 3) != (c < 3)) { e.x = -e.x; e.y = -e.y; }
-                }
-                const double2 w = ti[6 * b + c];
-                accr += e.x * w.x - e.y * w.y;
-                acci += e.x * w.y + e.y * w.x;
-            }
-            vi[6 * b + rr] = make_double2(-accr, -acci);
-        }
+    Hat64 a;
+    a.g = lat->g;
+    a.links = lat->links64;
+    a.clov = lat->clov64;
+    a.inv = inv;
+    a.nrhs = nrhs;
+    a.gamma5 = gamma5;
+    a.dm = 4.0 + m0;
+    a.live = live;
+    a.add = nullptr;
+    a.sigma = 0.0;
+    a.part = nullptr;
+    return a;
 }
 
-// out = scale (4 + m0 + A(x))^-1 t on odd sites (stored inverses), 0 on even sites; thread j
-// takes the j-th odd site and zeroes its even x partner
-__global__ void oo_inverse_kernel(const double2 *__restrict__ inv, const double2 *__restrict__ t,
-                                  double2 *__restrict__ out, Geom g, int k, double scale)
+unsigned hat_grid(const Geom &g, int nrhs) { return (unsigned)(((g.Ns / 2 + 63) / 64) * nrhs); }
+
+int launched(int n, const char *where)
 {
-    const int64_t half = g.Ns / 2;
-    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i >= half * k) return;
-    const int64_t r = i / half, j = i - r * half;
-    const int64_t row = j / g.L;
-    const int jx = (int)(j - row * g.L);
-    const int y = (int)(row % g.L), z = (int)((row / g.L) % g.L), tt = (int)(row / ((int64_t)g.L * g.L));
-    const int x = 2 * jx + ((1 + tt + z + y) & 1);
-    const int64_t s = row * g.L2 + x;
-    {
-        double2 *o = out + (r * g.Ns + (s ^ 1)) * 12;
-        for (int c = 0; c < 12; ++c) o[c] = make_double2(0.0, 0.0);
-    }
-    const double2 *ti = t + (r * g.Ns + s) * 12;
-    double2 *oi = out + (r * g.Ns + s) * 12;
-    const bool mir = x >= g.L;
-    const int64_t p = row * g.L + (mir ? x - g.L : x);
-    const int64_t V2 = g.Vphys / 2, q = p >> 1;
-    for (int b = 0; b < 2; ++b)
-        for (int rr = 0; rr < 6; ++rr) {
-            double accr = 0, acci = 0;
-            for (int c = 0; c < 6; ++c) {
-                const int ii = mir ? (rr + 3) % 6 : rr, jj = mir ? (c + 3) % 6 : c;
-                double2 e = inv[((int64_t)b * 36 + ii * 6 + jj) * V2 + q];
-                if (mir) {
-                    e.y = -e.y;
-                    if ((rr < 3) != (c < 3)) { e.x = -e.x; e.y = -e.y; }
-                }
-                const double2 w = ti[6 * b + c];
-                accr += e.x * w.x - e.y * w.y;
-                acci += e.x * w.y + e.y * w.x;
-            }
-            oi[6 * b + rr] = make_double2(scale * accr, scale * acci);
-        }
+    qs_note_launches(n);
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) { qs_record_cuda_error(e, where); return QS_ECUDA; }
+    return QS_OK;
 }
 
 }  // namespace
 
-// D_hat (or Q_hat) of nrhs FP64 vectors, asynchronous on the lattice's stream; work holds
-// 3 * nrhs * N_s * 24 doubles.  in and out must not overlap work; in may equal out.
-// With x the even part of the input, u = (D_oo)^-1 (D x)_o and v = x - u (even part x,
-// odd part -u):  D_hat x = (D x)_e - (D u)_e = (D v)_e, so the operator is applied twice,
-// each time on the output sites of one parity only.
-int qs_oo_inverse_apply(qs_lattice *lat, const double2 *inv, const double *in, double *out, int nrhs, double scale)
-{
-    const int64_t n = lat->g.Ns / 2 * nrhs;
-    oo_inverse_kernel<<<(unsigned)((n + 127) / 128), 128, 0, lat->stream>>>(inv, (const double2 *)in, (double2 *)out,
-                                                                          lat->g, nrhs, scale);
-    qs_note_launches(1);
-    const cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) { qs_record_cuda_error(e, "qs_oo_inverse_apply"); return QS_ECUDA; }
-    return QS_OK;
-}
-
-int qs_dslash64_parity(qs_lattice *lat, double m0, const double *in, double *out, int nrhs, int parity)
-{
-    DslashArgs<double> d;
-    d.g = lat->g;
-    d.links = lat->links64;
-    d.clov = lat->clov64;
-    d.nrhs = nrhs;
-    for (int r = 0; r < nrhs; ++r) d.m0[r] = m0;
-    d.in = in;
-    d.out = out;
-    d.gamma5 = 0;
-    const cudaError_t e = qs_dslash64_parity_launch(d, parity, lat->stream);
-    qs_note_launches(1);
-    if (e != cudaSuccess) { qs_record_cuda_error(e, "qs_dslash64_parity"); return QS_ECUDA; }
-    return QS_OK;
-}
+int64_t qs_hat_tiles(const Geom &g) { return (g.Ns / 2 + 63) / 64; }
 
 int qs_clover_inverse_odd(qs_lattice *lat, double m0, double2 *inv)
 {
-    const int64_t V = lat->g.Vphys;
-    clover_inverse_kernel<<<(unsigned)((V + 127) / 128), 128, 0, lat->stream>>>(lat->clov64, lat->g, 4.0 + m0, inv);
-    qs_note_launches(1);
-    const cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) { qs_record_cuda_error(e, "qs_clover_inverse_odd"); return QS_ECUDA; }
-    return QS_OK;
+    const int64_t n = lat->g.Vphys;
+    clover_inverse_kernel<<<(unsigned)((n + 63) / 64), 64, 0, lat->stream>>>(lat->clov64, lat->g, 4.0 + m0, inv);
+    return launched(1, "qs_clover_inverse_odd");
+}
+
+int qs_parity_pack(qs_lattice *lat, const double *in, double *out, int nrhs, int parity)
+{
+    const int64_t n = lat->g.Ns / 2 * 12 * nrhs;
+    parity_pack_kernel<<<(unsigned)((n + 255) / 256), 256, 0, lat->stream>>>((const double2 *)in, (double2 *)out, lat->g,
+                                                                             nrhs, parity);
+    return launched(1, "qs_parity_pack");
+}
+
+int qs_parity_unpack(qs_lattice *lat, const double *a, const double *b, double *x, int nrhs, int parity)
+{
+    const int64_t n = lat->g.Ns / 2 * 12 * nrhs;
+    parity_unpack_kernel<<<(unsigned)((n + 255) / 256), 256, 0, lat->stream>>>(
+        (const double2 *)a, (const double2 *)b, (double2 *)x, lat->g, nrhs, parity);
+    return launched(1, "qs_parity_unpack");
+}
+
+int qs_hat_odd(qs_lattice *lat, const double2 *inv, const double *in, double *out, int nrhs, int hop, double f,
+               const int *live)
+{
+    const Hat64 a = hat_args(lat, 0.0, nrhs, 0, inv, live);
+    const int64_t len = lat->g.Ns / 2 * 12;
+    if (hop)
+        hat_odd_kernel<At64Half, true><<<hat_grid(a.g, nrhs), 128, 0, lat->stream>>>(a, (const double2 *)in, len,
+                                                                                     (double2 *)out, f);
+    else
+        hat_odd_kernel<At64Half, false><<<hat_grid(a.g, nrhs), 128, 0, lat->stream>>>(a, (const double2 *)in, len,
+                                                                                      (double2 *)out, f);
+    return launched(1, "qs_hat_odd");
+}
+
+int qs_hat_hop_even(qs_lattice *lat, const double *v, const double *add, double sigma, double *out, int nrhs)
+{
+    Hat64 a = hat_args(lat, 0.0, nrhs, 0, nullptr, nullptr);
+    a.add = (const double2 *)add;
+    a.sigma = sigma;
+    hat_even_kernel<At64Half, false><<<hat_grid(a.g, nrhs), 128, 0, lat->stream>>>(
+        a, (const double2 *)v, nullptr, (double2 *)out, a.g.Ns / 2 * 12, false);
+    return launched(1, "qs_hat_hop_even");
 }
 
 int qs_dhat_run(qs_lattice *lat, double m0, const double *in, double *out, int nrhs, int gamma5, double *work,
-                const double2 *inv)
+                const double2 *inv, const int *live, const double *add, double sigma, double *part)
 {
-    const Geom &g = lat->g;
-    cudaStream_t st = lat->stream;
-    const int64_t vlen = (int64_t)nrhs * g.Ns * 24;
-    double *x = work, *dx = work + vlen, *v = work + 2 * vlen;
-    DslashArgs<double> d;
-    d.g = g;
-    d.links = lat->links64;
-    d.clov = lat->clov64;
-    d.nrhs = nrhs;
-    for (int r = 0; r < nrhs; ++r) d.m0[r] = m0;
-    const int64_t n = g.Ns * 12 * nrhs;
-    const unsigned nb = (unsigned)((n + 255) / 256), nbs = (unsigned)((g.Ns * nrhs + 127) / 128);
-    parity_mask_kernel<<<nb, 256, 0, st>>>((const double2 *)in, (double2 *)x, g, nrhs, 0);
-    d.in = x;
-    d.out = dx;
-    d.gamma5 = 0;
-    cudaError_t e = qs_dslash64_parity_launch(d, 1, st);                                     // (D x)_o
-    if (e == cudaSuccess) {
-        if (inv)
-            clover_apply_inv_kernel<<<(unsigned)((g.Ns / 2 * nrhs + 127) / 128), 128, 0, st>>>(
-                inv, (const double2 *)dx, (const double2 *)x, (double2 *)v, g, nrhs);          // v = x - u
-        else
-            clover_solve_odd_kernel<<<nbs, 128, 0, st>>>(lat->clov64, (const double2 *)dx, (const double2 *)x,
-                                                         (double2 *)v, g, nrhs, 4.0 + m0);
-
-        d.in = v;
-        d.out = out;
-        d.gamma5 = gamma5;
-        e = qs_dslash64_parity_launch(d, 0, st);                                             // (D v)_e
-    }
-    qs_note_launches(4);
-    if (e == cudaSuccess) e = cudaGetLastError();
-    if (e != cudaSuccess) { qs_record_cuda_error(e, "qs_dhat_run"); return QS_ECUDA; }
-    return QS_OK;
-}
-
-int qs_even_mask(qs_lattice *lat, const double *in, double *out, int nrhs)
-{
-    const int64_t n = lat->g.Ns * 12 * nrhs;
-    parity_mask_kernel<<<(unsigned)((n + 255) / 256), 256, 0, lat->stream>>>((const double2 *)in, (double2 *)out,
-                                                                             lat->g, nrhs, 0);
-    qs_note_launches(1);
-    const cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) { qs_record_cuda_error(e, "qs_even_mask"); return QS_ECUDA; }
-    return QS_OK;
+    QS_TRY(qs_hat_odd(lat, inv, in, work, nrhs, 1, -1.0, live));
+    Hat64 a = hat_args(lat, m0, nrhs, gamma5, inv, live);
+    a.add = (const double2 *)add;
+    a.sigma = sigma;
+    a.part = part;
+    hat_even_kernel<At64Half, true><<<hat_grid(a.g, nrhs), 128, 0, lat->stream>>>(
+        a, (const double2 *)work, (const double2 *)in, (double2 *)out, a.g.Ns / 2 * 12, false);
+    return launched(1, "qs_dhat_run");
 }
 
 extern "C" int qs_apply_Dhat(qs_lattice *lat, double m0, const void *in, void *out, int nrhs, int gamma5)
@@ -511,13 +487,23 @@ extern "C" int qs_apply_Dhat(qs_lattice *lat, double m0, const void *in, void *o
     const Geom &g = lat->g;
     if ((g.T | g.L) & 1) return QS_EINVAL;   // hopping must connect opposite parities only
     const size_t bytes = (size_t)nrhs * g.Ns * 24 * sizeof(double);
-    const char *a = (const char *)in, *b = (const char *)out;
-    if (a < b + bytes && b < a + bytes) return QS_EINVAL;
+    const char *pa = (const char *)in, *pb = (const char *)out;
+    if (pa < pb + bytes && pb < pa + bytes) return QS_EINVAL;
     if (((uintptr_t)in | (uintptr_t)out) & 15) return QS_EINVAL;
     QS_CUDA(cudaSetDevice(lat->device));
     double *buf = nullptr;
-    QS_CUDA(cudaMalloc(&buf, 3 * bytes));
-    int s = qs_dhat_run(lat, m0, (const double *)in, (double *)out, nrhs, gamma5, buf, nullptr);
+    const size_t inv_len = (size_t)36 * g.Vphys;
+    QS_CUDA(cudaMalloc(&buf, bytes / 2 + inv_len * sizeof(double2)));
+    double2 *inv = (double2 *)(buf + bytes / 2 / sizeof(double));
+    int s = qs_clover_inverse_odd(lat, m0, inv);
+    if (s == QS_OK) {
+        const Hat64 a = hat_args(lat, m0, nrhs, gamma5, inv, nullptr);
+        hat_odd_kernel<At64Canon, true><<<hat_grid(g, nrhs), 128, 0, lat->stream>>>(a, (const double2 *)in, g.Ns * 12,
+                                                                                    (double2 *)buf, -1.0);
+        hat_even_kernel<At64Canon, true><<<hat_grid(g, nrhs), 128, 0, lat->stream>>>(
+            a, (const double2 *)buf, (const double2 *)in, (double2 *)out, g.Ns * 12, true);
+        s = launched(2, "qs_apply_Dhat");
+    }
     if (s == QS_OK) {
         const cudaError_t e = cudaStreamSynchronize(lat->stream);
         if (e != cudaSuccess) { qs_record_cuda_error(e, "qs_apply_Dhat"); s = QS_ECUDA; }

@@ -266,27 +266,13 @@ extern "C" int qs_ratapprox(int n, double ra, double rb, double *A, double *nu, 
 namespace {
 
 #define RW_PARTS 304   // blocks per right-hand side in the reductions (2 x 152 SMs)
+#define RW_LAG 2       // iterations the host may be ahead of the convergence flags it has seen
 
-struct Coef {
-    double v[64];
-};
-
-// y_r += a_r x_r over vectors of len doubles each
-__global__ void rw_axpy(double *__restrict__ y, const double *__restrict__ x, Coef a, int64_t len)
+// y += c x over n doubles
+__global__ void rw_axpy(double *__restrict__ y, const double *__restrict__ x, double c, int64_t n)
 {
-    const int r = blockIdx.y;
-    const double c = a.v[r];
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < len; i += (int64_t)gridDim.x * blockDim.x)
-        y[r * len + i] += c * x[r * len + i];
-}
-
-// p_r = z_r + b_r p_r
-__global__ void rw_xpby(double *__restrict__ p, const double *__restrict__ z, Coef b, int64_t len)
-{
-    const int r = blockIdx.y;
-    const double c = b.v[r];
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < len; i += (int64_t)gridDim.x * blockDim.x)
-        p[r * len + i] = z[r * len + i] + c * p[r * len + i];
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
+        y[i] += c * x[i];
 }
 
 // out = in + c i x (complex, c real); in may equal out
@@ -298,59 +284,171 @@ __global__ void rw_add_ix(double2 *out, const double2 *in, const double2 *__rest
     }
 }
 
+// component of element i of a vector: [site][12], or [site / 16][12][site % 16]
+__device__ __forceinline__ int rw_comp(int64_t i, int tiled) { return (int)((tiled ? i >> 4 : i) % 12); }
+
 // out = c i gamma_5 x (c real; chiral basis: spins 2, 3 negated); out may equal x
-__global__ void rw_ig5(double2 *out, const double2 *x, double c, int64_t n)
+__global__ void rw_ig5(double2 *out, const double2 *x, double c, int64_t n, int tiled)
 {
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const double s = (i % 12) >= 6 ? -c : c;
+        const double s = rw_comp(i, tiled) >= 6 ? -c : c;
         const double2 b = x[i];
         out[i] = make_double2(-s * b.y, s * b.x);
     }
 }
 
 // out = gamma_5 x; out may equal x
-__global__ void rw_g5(double2 *out, const double2 *x, int64_t n)
+__global__ void rw_g5(double2 *out, const double2 *x, int64_t n, int tiled)
 {
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         const double2 b = x[i];
-        out[i] = (i % 12) >= 6 ? make_double2(-b.x, -b.y) : b;
+        out[i] = rw_comp(i, tiled) >= 6 ? make_double2(-b.x, -b.y) : b;
     }
 }
 
-// part[r][blk] = sum over the block's share of conj(x_r) y_r (complex), fixed order
-__global__ void rw_dot_part(const double2 *__restrict__ x, const double2 *__restrict__ y, int64_t n,
-                            double2 *__restrict__ part)
+// sum over the block (256 threads), fixed order; valid in thread 0
+__device__ double rw_block_sum(double v)
 {
-    __shared__ double2 sh[256];
+    __shared__ double sh[8];
+    for (int d = 16; d > 0; d >>= 1) v += __shfl_xor_sync(0xffffffffu, v, d);
+    __syncthreads();
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
+    __syncthreads();
+    v = threadIdx.x < 8 ? sh[threadIdx.x] : 0.0;
+    for (int d = 4; d > 0; d >>= 1) v += __shfl_xor_sync(0xffffffffu, v, d);
+    return v;
+}
+
+// part[r][blk] = the block's share of Re (x_r, y_r)
+__global__ void __launch_bounds__(256) rw_dot_part(const double2 *__restrict__ x, const double2 *__restrict__ y, int64_t n,
+                                                   double *__restrict__ part)
+{
     const int r = blockIdx.y;
-    double re = 0, im = 0;
+    double re = 0;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         const double2 a = x[r * n + i], b = y[r * n + i];
-        re += a.x * b.x + a.y * b.y;
-        im += a.x * b.y - a.y * b.x;
+        re = fma(a.y, b.y, fma(a.x, b.x, re));
     }
-    sh[threadIdx.x] = make_double2(re, im);
-    __syncthreads();
-    for (int s = 128; s > 0; s >>= 1) {
-        if (threadIdx.x < s) {
-            sh[threadIdx.x].x += sh[threadIdx.x + s].x;
-            sh[threadIdx.x].y += sh[threadIdx.x + s].y;
-        }
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) part[r * gridDim.x + blockIdx.x] = sh[0];
+    re = rw_block_sum(re);
+    if (threadIdx.x == 0) part[r * gridDim.x + blockIdx.x] = re;
 }
 
-__global__ void rw_dot_sum(const double2 *__restrict__ part, int nparts, double2 *__restrict__ out)
+__device__ double rw_sum_parts(const double *part, int nparts)
+{
+    double s = 0;
+    for (int i = threadIdx.x; i < nparts; i += 256) s += part[i];
+    return rw_block_sum(s);
+}
+
+__global__ void __launch_bounds__(256) rw_dot_sum(const double *__restrict__ part, int nparts, double *__restrict__ out)
+{
+    const double s = rw_sum_parts(part + (int64_t)blockIdx.x * nparts, nparts);
+    if (threadIdx.x == 0) out[blockIdx.x] = s;
+}
+
+// ---- conjugate gradients with the scalars on the device --------------------------------------
+// Per right-hand side: |r|^2, its stopping value and whether it still iterates (live), in two
+// slots: an iteration reads slot `o` and writes slot 1 - o.  Every block sums the partial sums
+// it needs itself (a few hundred words from L2, in a fixed order), so an iteration is the
+// operator's launches and two more; with separate launches for the scalars the launch gaps
+// were a tenth of an iteration on 8^3 x 16.  A right-hand side that has converged is skipped by
+// every kernel that follows.
+struct RwScal {
+    double *rr[2], *stop;
+    int *live[2];
+};
+
+// x = 0, r = p = b, part = shares of |b|^2
+__global__ void __launch_bounds__(256) rw_cg_start(const double2 *__restrict__ b, double2 *__restrict__ x,
+                                                   double2 *__restrict__ r, double2 *__restrict__ p, int64_t n, double *part)
+{
+    const int64_t o = blockIdx.y * n;
+    double acc = 0;
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+        const double2 v = b[o + i];
+        x[o + i] = make_double2(0.0, 0.0);
+        r[o + i] = v;
+        p[o + i] = v;
+        acc = fma(v.y, v.y, fma(v.x, v.x, acc));
+    }
+    acc = rw_block_sum(acc);
+    if (threadIdx.x == 0) part[blockIdx.y * gridDim.x + blockIdx.x] = acc;
+}
+
+__global__ void __launch_bounds__(256) rw_cg_first(RwScal s, const double *part, int nparts, double tol2)
 {
     const int r = blockIdx.x;
+    const double d = rw_sum_parts(part + (int64_t)r * nparts, nparts);
     if (threadIdx.x != 0) return;
-    double re = 0, im = 0;
-    for (int b = 0; b < nparts; ++b) {
-        re += part[r * nparts + b].x;
-        im += part[r * nparts + b].y;
+    s.rr[0][r] = d;
+    s.stop[r] = tol2 * d;
+    s.live[0][r] = d > 0;
+}
+
+// the sum of the partials, known to every thread of the block
+__device__ double rw_all_parts(const double *part, int nparts)
+{
+    __shared__ double d;
+    const double v = rw_sum_parts(part, nparts);
+    if (threadIdx.x == 0) d = v;
+    __syncthreads();
+    return d;
+}
+
+// r -= alpha A p, alpha = |r|^2 / (p, A p); rpart = shares of |r|^2
+__global__ void __launch_bounds__(256) rw_cg_r(double2 *__restrict__ r, const double2 *__restrict__ ap, RwScal s, int o,
+                                               int64_t n, const double *__restrict__ ppart, int nparts,
+                                               double *__restrict__ rpart)
+{
+    const int k = blockIdx.y;
+    if (!s.live[o][k]) return;
+    const double pap = rw_all_parts(ppart + (int64_t)k * nparts, nparts);
+    const double c = pap > 0 ? -s.rr[o][k] / pap : 0.0;
+    double2 *rk = r + k * n;
+    const double2 *ak = ap + k * n;
+    double acc = 0;
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+        const double2 a = ak[i];
+        double2 v = rk[i];
+        v = make_double2(fma(c, a.x, v.x), fma(c, a.y, v.y));
+        rk[i] = v;
+        acc = fma(v.y, v.y, fma(v.x, v.x, acc));
     }
-    out[r] = make_double2(re, im);
+    acc = rw_block_sum(acc);
+    if (threadIdx.x == 0) rpart[k * gridDim.x + blockIdx.x] = acc;
+}
+
+// x += alpha p, p = r + beta p, beta = |r|^2 / |r_old|^2; the right-hand side lives on unless |r|^2
+// has reached its stopping value
+__global__ void __launch_bounds__(256) rw_cg_xp(double2 *__restrict__ x, double2 *__restrict__ p,
+                                                const double2 *__restrict__ r, RwScal s, int o, int64_t n,
+                                                const double *__restrict__ ppart, int nparts,
+                                                const double *__restrict__ rpart)
+{
+    const int k = blockIdx.y;
+    const bool first = blockIdx.x == 0 && threadIdx.x == 0;
+    if (!s.live[o][k]) {
+        if (first) s.live[1 - o][k] = 0;
+        return;
+    }
+    const double rr = s.rr[o][k];
+    const double pap = rw_all_parts(ppart + (int64_t)k * nparts, nparts);
+    __syncthreads();
+    const double rn = rw_all_parts(rpart + (int64_t)k * gridDim.x, (int)gridDim.x);
+    const double a = pap > 0 ? rr / pap : 0.0, b = rr > 0 ? rn / rr : 0.0;
+    if (first) {
+        s.rr[1 - o][k] = rn;
+        s.live[1 - o][k] = !(rn <= s.stop[k]);
+    }
+    double2 *xk = x + k * n, *pk = p + k * n;
+    const double2 *rk = r + k * n;
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+        const double2 q = pk[i], v = rk[i];
+        double2 y = xk[i];
+        y = make_double2(fma(a, q.x, y.x), fma(a, q.y, y.y));
+        xk[i] = y;
+        pk[i] = make_double2(fma(b, q.x, v.x), fma(b, q.y, v.y));
+    }
 }
 
 struct RwWork {
@@ -358,13 +456,47 @@ struct RwWork {
     int nrhs;
     int64_t len;          // doubles per vector
     double *eta, *t, *x, *r, *p, *ap, *tmp, *dwork;
-    double2 *part, *dots;
+    double *part, *rpart, *dots;
+    RwScal sc;
+    int *hflag;           // pinned, RW_LAG + 1 copies of the live flags
+    cudaEvent_t ev[RW_LAG + 1];
     int full;             // 1: Q^2 of the full-lattice operator instead of Q_hat^2
     // odd-site block inverses at the two masses of the estimate
     double mass[2];
     const double2 *inv[2];
-    const double2 *inv_for(double m) const { return m == mass[0] ? inv[0] : m == mass[1] ? inv[1] : nullptr; }
+    const double2 *inv_for(double m) const { return m == mass[0] ? inv[0] : inv[1]; }
 };
+
+int64_t rw_parts(const Geom &g) { return std::max<int64_t>(RW_PARTS, qs_hat_tiles(g)); }
+// doubles of scalar and reduction storage
+int64_t rw_small(const Geom &g, int nrhs) { return nrhs * (rw_parts(g) + RW_PARTS + 8); }
+
+// lays out the small arrays at `buf` (rw_small doubles) and makes the pinned flags and events
+int rw_begin(RwWork &w, double *buf)
+{
+    w.part = buf;
+    w.rpart = buf + w.nrhs * rw_parts(w.lat->g);
+    double *d = w.rpart + w.nrhs * RW_PARTS;
+    w.dots = d;
+    w.sc.stop = d + w.nrhs;
+    for (int o = 0; o < 2; ++o) {
+        w.sc.rr[o] = d + (2 + o) * w.nrhs;
+        w.sc.live[o] = (int *)(d + (4 + o) * w.nrhs);
+    }
+    w.hflag = nullptr;
+    for (auto &e : w.ev) e = nullptr;
+    QS_CUDA(cudaMallocHost(&w.hflag, (RW_LAG + 1) * 64 * sizeof(int)));
+    for (auto &e : w.ev) QS_CUDA(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
+    return QS_OK;
+}
+
+void rw_end(RwWork &w)
+{
+    cudaStreamSynchronize(w.lat->stream);   // no flag copy may be in flight when its buffer goes
+    for (auto e : w.ev)
+        if (e) cudaEventDestroy(e);
+    if (w.hflag) cudaFreeHost(w.hflag);
+}
 
 int rw_check(const char *where)
 {
@@ -373,89 +505,96 @@ int rw_check(const char *where)
     return QS_OK;
 }
 
-// out[r] = (x_r, y_r) on the host
-int rw_dot(RwWork &w, const double *x, const double *y, double2 *out)
+unsigned rw_blocks(int64_t n) { return (unsigned)std::max<int64_t>(1, std::min<int64_t>((n + 511) / 512, RW_PARTS)); }
+
+// out[r] = Re (x_r, y_r) on the host
+int rw_dot(RwWork &w, const double *x, const double *y, double *out)
 {
     cudaStream_t st = w.lat->stream;
-    rw_dot_part<<<dim3(RW_PARTS, w.nrhs), 256, 0, st>>>((const double2 *)x, (const double2 *)y, w.len / 2, w.part);
-    rw_dot_sum<<<w.nrhs, 32, 0, st>>>(w.part, RW_PARTS, w.dots);
+    const unsigned nb = rw_blocks(w.len / 2);
+    rw_dot_part<<<dim3(nb, w.nrhs), 256, 0, st>>>((const double2 *)x, (const double2 *)y, w.len / 2, w.part);
+    rw_dot_sum<<<w.nrhs, 256, 0, st>>>(w.part, (int)nb, w.dots);
     qs_note_launches(2);
     QS_TRY(rw_check("rw_dot"));
-    QS_CUDA(cudaMemcpyAsync(out, w.dots, w.nrhs * sizeof(double2), cudaMemcpyDeviceToHost, st));
+    QS_CUDA(cudaMemcpyAsync(out, w.dots, w.nrhs * sizeof(double), cudaMemcpyDeviceToHost, st));
     QS_CUDA(cudaStreamSynchronize(st));
     return QS_OK;
 }
 
 unsigned rw_grid(int64_t n) { return (unsigned)std::min<int64_t>((n + 255) / 256, 4 * 152); }
 
-// out = Q_hat(m)^2 in + sigma in
-int rw_q2(RwWork &w, double m, double sigma, const double *in, double *out)
+// ap = (Q_hat(m)^2 + sigma) p for the live right-hand sides, and the shares of (p, ap) in
+// w.part; *nparts of them per right-hand side
+int rw_q2(RwWork &w, double m, double sigma, const int *live, int *nparts)
 {
     if (w.full) {
         double mm[64];
         for (int r = 0; r < w.nrhs; ++r) mm[r] = m;
-        QS_TRY(qs_dslash_run(w.lat, QS_F64, mm, in, w.tmp, w.nrhs, 1, 0));
-        QS_TRY(qs_dslash_run(w.lat, QS_F64, mm, w.tmp, out, w.nrhs, 1, 0));
-    } else {
-        QS_TRY(qs_dhat_run(w.lat, m, in, w.tmp, w.nrhs, 1, w.dwork, w.inv_for(m)));
-        QS_TRY(qs_dhat_run(w.lat, m, w.tmp, out, w.nrhs, 1, w.dwork, w.inv_for(m)));
+        QS_TRY(qs_dslash_run(w.lat, QS_F64, mm, w.p, w.tmp, w.nrhs, 1, 0));
+        QS_TRY(qs_dslash_run(w.lat, QS_F64, mm, w.tmp, w.ap, w.nrhs, 1, 0));
+        if (sigma != 0.0) {
+            const int64_t n = w.nrhs * w.len;
+            rw_axpy<<<rw_grid(n), 256, 0, w.lat->stream>>>(w.ap, w.p, sigma, n);
+            qs_note_launches(1);
+        }
+        *nparts = (int)rw_blocks(w.len / 2);
+        rw_dot_part<<<dim3(*nparts, w.nrhs), 256, 0, w.lat->stream>>>((const double2 *)w.p, (const double2 *)w.ap, w.len / 2,
+                                                                     w.part);
+        qs_note_launches(1);
+        return rw_check("rw_q2");
     }
-    Coef c;
-    for (int r = 0; r < w.nrhs; ++r) c.v[r] = sigma;
-    rw_axpy<<<dim3(rw_grid(w.len), w.nrhs), 256, 0, w.lat->stream>>>(out, in, c, w.len);
-    qs_note_launches(1);
-    return rw_check("rw_q2");
+    const double2 *inv = w.inv_for(m);
+    QS_TRY(qs_dhat_run(w.lat, m, w.p, w.tmp, w.nrhs, 1, w.dwork, inv, live));
+    *nparts = (int)qs_hat_tiles(w.lat->g);
+    return qs_dhat_run(w.lat, m, w.tmp, w.ap, w.nrhs, 1, w.dwork, inv, live, w.p, sigma, w.part);
 }
 
 // x = (Q_hat(m)^2 + sigma)^-1 b by conjugate gradients (x0 = 0), every right-hand side to
-// ||r|| <= tol ||b||; *iters: iterations taken
+// ||r|| <= tol ||b||; *iters: iterations taken.  No iteration waits for the host: it reads the
+// convergence flags RW_LAG iterations late, and the iterations it has launched by then find
+// every right-hand side converged and return at once.
 int rw_cg(RwWork &w, double m, double sigma, const double *b, double *x, double tol, int max_iter, int *iters)
 {
     cudaStream_t st = w.lat->stream;
-    const size_t bytes = (size_t)w.nrhs * w.len * sizeof(double);
-    QS_CUDA(cudaMemsetAsync(x, 0, bytes, st));
-    QS_CUDA(cudaMemcpyAsync(w.r, b, bytes, cudaMemcpyDeviceToDevice, st));
-    QS_CUDA(cudaMemcpyAsync(w.p, b, bytes, cudaMemcpyDeviceToDevice, st));
-    double2 d[64];
-    QS_TRY(rw_dot(w, w.r, w.r, d));
-    double rr[64], stop[64];
-    bool live[64];
-    for (int r = 0; r < w.nrhs; ++r) {
-        rr[r] = d[r].x;
-        stop[r] = tol * tol * rr[r];
-        live[r] = rr[r] > 0;
-    }
-    const unsigned gx = rw_grid(w.len);
-    for (int it = 0; it < max_iter; ++it) {
-        bool any = false;
-        for (int r = 0; r < w.nrhs; ++r) any |= live[r];
-        if (!any) { *iters = it; return QS_OK; }
-        QS_TRY(rw_q2(w, m, sigma, w.p, w.ap));
-        QS_TRY(rw_dot(w, w.p, w.ap, d));
-        Coef a, na;
-        for (int r = 0; r < w.nrhs; ++r) {
-            a.v[r] = live[r] && d[r].x > 0 ? rr[r] / d[r].x : 0.0;
-            na.v[r] = -a.v[r];
+    const int64_t n = w.len / 2;
+    const unsigned nb = rw_blocks(n);
+    const dim3 grid(nb, w.nrhs);
+    rw_cg_start<<<grid, 256, 0, st>>>((const double2 *)b, (double2 *)x, (double2 *)w.r, (double2 *)w.p, n, w.part);
+    rw_cg_first<<<w.nrhs, 256, 0, st>>>(w.sc, w.part, (int)nb, tol * tol);
+    qs_note_launches(2);
+    QS_TRY(rw_check("rw_cg"));
+    QS_CUDA(cudaMemcpyAsync(w.hflag, w.sc.live[0], w.nrhs * sizeof(int), cudaMemcpyDeviceToHost, st));
+    QS_CUDA(cudaStreamSynchronize(st));
+    auto any = [&](const int *f) {
+        for (int r = 0; r < w.nrhs; ++r)
+            if (f[r]) return true;
+        return false;
+    };
+    if (!any(w.hflag)) { *iters = 0; return QS_OK; }
+    int it = 0, seen = 0;   // iterations launched, and those whose flags have been read
+    while (seen < max_iter) {
+        if (it < max_iter && it <= seen + RW_LAG) {
+            const int o = it & 1;
+            int np = 0;
+            QS_TRY(rw_q2(w, m, sigma, w.sc.live[o], &np));
+            rw_cg_r<<<grid, 256, 0, st>>>((double2 *)w.r, (const double2 *)w.ap, w.sc, o, n, w.part, np, w.rpart);
+            rw_cg_xp<<<grid, 256, 0, st>>>((double2 *)x, (double2 *)w.p, (const double2 *)w.r, w.sc, o, n, w.part, np,
+                                           w.rpart);
+            qs_note_launches(2);
+            QS_TRY(rw_check("rw_cg"));
+            const int slot = it % (RW_LAG + 1);
+            QS_CUDA(cudaMemcpyAsync(w.hflag + 64 * slot, w.sc.live[1 - o], w.nrhs * sizeof(int), cudaMemcpyDeviceToHost, st));
+            QS_CUDA(cudaEventRecord(w.ev[slot], st));
+            ++it;
+            continue;
         }
-        rw_axpy<<<dim3(gx, w.nrhs), 256, 0, st>>>(x, w.p, a, w.len);
-        rw_axpy<<<dim3(gx, w.nrhs), 256, 0, st>>>(w.r, w.ap, na, w.len);
-        qs_note_launches(2);
-        QS_TRY(rw_dot(w, w.r, w.r, d));
-        Coef beta;
-        for (int r = 0; r < w.nrhs; ++r) {
-            const double rn = d[r].x;
-            beta.v[r] = live[r] && rr[r] > 0 ? rn / rr[r] : 0.0;
-            if (live[r] && rn <= stop[r]) live[r] = false;
-            rr[r] = rn;
-        }
-        rw_xpby<<<dim3(gx, w.nrhs), 256, 0, st>>>(w.p, w.r, beta, w.len);
-        qs_note_launches(1);
-        QS_TRY(rw_check("rw_cg"));
+        const int slot = seen % (RW_LAG + 1);
+        QS_CUDA(cudaEventSynchronize(w.ev[slot]));
+        ++seen;
+        if (!any(w.hflag + 64 * slot)) { *iters = seen; return QS_OK; }
     }
     *iters = max_iter;
-    for (int r = 0; r < w.nrhs; ++r)
-        if (live[r]) return QS_ENOCONV;
-    return QS_OK;
+    return QS_ENOCONV;
 }
 
 // out = a^-1 in with a = D_hat(m) + i gamma_5 shift: (Q_hat(m) - i shift)(Q_hat^2 + shift^2)^-1 gamma_5 in
@@ -464,7 +603,7 @@ int rw_shifted_inverse(RwWork &w, double m, double shift, const double *in, doub
 {
     const int64_t nc = (int64_t)w.nrhs * w.len / 2;
     cudaStream_t st = w.lat->stream;
-    rw_g5<<<rw_grid(nc), 256, 0, st>>>((double2 *)w.t, (const double2 *)in, nc);
+    rw_g5<<<rw_grid(nc), 256, 0, st>>>((double2 *)w.t, (const double2 *)in, nc, 1);
     qs_note_launches(1);
     QS_TRY(rw_cg(w, m, shift * shift, w.t, w.x, tol, max_iter, iters));
     QS_TRY(qs_dhat_run(w.lat, m, w.x, out, w.nrhs, 1, w.dwork, w.inv_for(m)));
@@ -491,12 +630,11 @@ extern "C" int qs_w_mass(qs_lattice *lat, double m, double mp, int n, const doub
     w.lat = lat;
     w.full = 0;
     w.nrhs = nsrc;
-    w.len = g.Ns * 24;
+    w.len = g.Ns * 12;                      // half vectors
     const int64_t vl = (int64_t)nsrc * w.len;   // doubles per block of nsrc vectors
     double *buf = nullptr;
     const size_t inv_len = (size_t)36 * g.Vphys;   // complex entries of the inverses at one mass
-    QS_CUDA(cudaMalloc(&buf, 12 * vl * sizeof(double) + (size_t)nsrc * (RW_PARTS + 1) * sizeof(double2) +
-                                 2 * inv_len * sizeof(double2)));
+    QS_CUDA(cudaMalloc(&buf, (10 * vl + rw_small(g, nsrc)) * sizeof(double) + 2 * inv_len * sizeof(double2)));
     w.eta = buf;
     w.t = buf + vl;
     w.x = buf + 2 * vl;
@@ -504,21 +642,20 @@ extern "C" int qs_w_mass(qs_lattice *lat, double m, double mp, int n, const doub
     w.p = buf + 4 * vl;
     w.ap = buf + 5 * vl;
     w.tmp = buf + 6 * vl;
-    w.dwork = buf + 7 * vl;   // 3 blocks
-    double *v1 = buf + 10 * vl, *v2 = buf + 11 * vl;
-    w.part = (double2 *)(buf + 12 * vl);
-    w.dots = w.part + (size_t)nsrc * RW_PARTS;
-    double2 *inv = w.dots + nsrc;
+    w.dwork = buf + 7 * vl;
+    double *v1 = buf + 8 * vl, *v2 = buf + 9 * vl;
+    double2 *inv = (double2 *)(buf + 10 * vl);
     w.mass[0] = m;
     w.mass[1] = mp;
     w.inv[0] = inv;
     w.inv[1] = inv + inv_len;
     cudaStream_t st = lat->stream;
     const int64_t nc = vl / 2;
-    int s = QS_OK, total_it = 0;
+    int total_it = 0;
+    int s = rw_begin(w, (double *)(inv + 2 * inv_len));
     double lw = 0;
-    do {
-        if ((s = qs_even_mask(lat, (const double *)eta, w.eta, nsrc)) != QS_OK) break;
+    if (s == QS_OK) do {
+        if ((s = qs_parity_pack(lat, (const double *)eta, w.eta, nsrc, 0)) != QS_OK) break;
         if ((s = qs_clover_inverse_odd(lat, m, (double2 *)w.inv[0])) != QS_OK) break;
         if ((s = qs_clover_inverse_odd(lat, mp, (double2 *)w.inv[1])) != QS_OK) break;
         for (int j = 0; j < n && s == QS_OK; ++j) {
@@ -526,24 +663,22 @@ extern "C" int qs_w_mass(qs_lattice *lat, double m, double mp, int n, const doub
             // v1 = i gamma_5 (mu - nu) a^-1 eta, v2 = b^-1 v1 = S_j eta
             if ((s = rw_shifted_inverse(w, m, nu[j], w.eta, v1, tol, max_iter, &it)) != QS_OK) break;
             total_it += it;
-            rw_ig5<<<rw_grid(nc), 256, 0, st>>>((double2 *)v1, (const double2 *)v1, mu[j] - nu[j], nc);
+            rw_ig5<<<rw_grid(nc), 256, 0, st>>>((double2 *)v1, (const double2 *)v1, mu[j] - nu[j], nc, 1);
             qs_note_launches(1);
             if ((s = rw_shifted_inverse(w, mp, mu[j], v1, v2, tol, max_iter, &it)) != QS_OK) break;
             total_it += it;
             // v1 = X eta = D_hat(m') S_j eta - D_hat(m) S_j eta
             if ((s = qs_dhat_run(lat, mp, v2, v1, nsrc, 0, w.dwork, w.inv_for(mp))) != QS_OK) break;
             if ((s = qs_dhat_run(lat, m, v2, w.tmp, nsrc, 0, w.dwork, w.inv_for(m))) != QS_OK) break;
-            Coef c;
-            for (int r = 0; r < nsrc; ++r) c.v[r] = -1.0;
-            rw_axpy<<<dim3(rw_grid(w.len), nsrc), 256, 0, st>>>(v1, w.tmp, c, w.len);
+            rw_axpy<<<rw_grid(vl), 256, 0, st>>>(v1, w.tmp, -1.0, vl);
             qs_note_launches(1);
             // q = (eta, R_j eta) = 2 Re (eta, X eta) + ||X eta||^2
-            double2 ex[64], xx[64];
+            double ex[64], xx[64];
             if ((s = rw_dot(w, w.eta, v1, ex)) != QS_OK) break;
             if ((s = rw_dot(w, v1, v1, xx)) != QS_OK) break;
             double mx = -INFINITY;
             for (int l = 0; l < nsrc; ++l) {
-                q[(size_t)j * nsrc + l] = 2 * ex[l].x + xx[l].x;
+                q[(size_t)j * nsrc + l] = 2 * ex[l] + xx[l];
                 mx = std::max(mx, -q[(size_t)j * nsrc + l]);
             }
             double sum = 0;   // log of the mean of exp(-q), shifted by the largest exponent
@@ -551,6 +686,7 @@ extern "C" int qs_w_mass(qs_lattice *lat, double m, double mp, int n, const doub
             lw += mx + log(sum / nsrc);
         }
     } while (0);
+    rw_end(w);
     cudaFree(buf);
     if (cg_iterations) *cg_iterations = total_it;
     if (s == QS_OK && log_w) *log_w = lw;
@@ -558,15 +694,6 @@ extern "C" int qs_w_mass(qs_lattice *lat, double m, double mp, int n, const doub
 }
 
 // ---- the even-odd preconditioned solve of D x = b (Sec. 4) ---------------------------------
-namespace {
-int rw_copy(void *dst, const void *src, size_t bytes, cudaStream_t st)
-{
-    const cudaError_t e = cudaMemcpyAsync(dst, src, bytes, cudaMemcpyDeviceToDevice, st);
-    if (e != cudaSuccess) { qs_record_cuda_error(e, "qs_solve_D copy"); return QS_ECUDA; }
-    return QS_OK;
-}
-}  // namespace
-
 // even_odd = 1:  b'_e = b_e - D_eo (D_oo)^-1 b_o;  D_hat x_e = b'_e by CG on Q_hat^2
 // (x_e = Q_hat (Q_hat^2)^-1 gamma_5 b'_e);  x_o = (D_oo)^-1 (b_o - D_oe x_e).
 // even_odd = 0:  x = Q (Q^2)^-1 gamma_5 b by CG on the full-lattice Q^2 (the comparison).
@@ -586,12 +713,11 @@ extern "C" int qs_solve_D(qs_lattice *lat, double m0, const void *b, void *x, in
     w.lat = lat;
     w.full = even_odd ? 0 : 1;
     w.nrhs = nrhs;
-    w.len = g.Ns * 24;
+    w.len = even_odd ? g.Ns * 12 : g.Ns * 24;
     const int64_t vl = (int64_t)nrhs * w.len;
     const size_t inv_len = even_odd ? (size_t)36 * g.Vphys : 0;
     double *buf = nullptr;
-    QS_CUDA(cudaMalloc(&buf, 11 * vl * sizeof(double) + (size_t)nrhs * (RW_PARTS + 1) * sizeof(double2) +
-                                 inv_len * sizeof(double2)));
+    QS_CUDA(cudaMalloc(&buf, (9 * vl + rw_small(g, nrhs)) * sizeof(double) + inv_len * sizeof(double2)));
     w.eta = nullptr;
     w.t = buf;
     w.x = buf + vl;
@@ -599,40 +725,30 @@ extern "C" int qs_solve_D(qs_lattice *lat, double m0, const void *b, void *x, in
     w.p = buf + 3 * vl;
     w.ap = buf + 4 * vl;
     w.tmp = buf + 5 * vl;
-    w.dwork = buf + 6 * vl;   // 3 blocks
-    double *a1 = buf + 9 * vl, *a2 = buf + 10 * vl;
-    w.part = (double2 *)(buf + 11 * vl);
-    w.dots = w.part + (size_t)nrhs * RW_PARTS;
-    double2 *inv = even_odd ? w.dots + nrhs : nullptr;
+    w.dwork = buf + 6 * vl;
+    double *a1 = buf + 7 * vl, *a2 = buf + 8 * vl;
+    double2 *inv = (double2 *)(buf + 9 * vl);
     w.mass[0] = w.mass[1] = m0;
     w.inv[0] = w.inv[1] = inv;
     cudaStream_t st = lat->stream;
     const int64_t nc = vl / 2;
-    Coef minus, plus;
-    for (int r = 0; r < nrhs; ++r) { minus.v[r] = -1.0; plus.v[r] = 1.0; }
-    const dim3 ga(rw_grid(w.len), nrhs);
-    int s = QS_OK, it = 0;
-    do {
+    int s = rw_begin(w, (double *)(inv + inv_len)), it = 0;
+    if (s == QS_OK) do {
         if (even_odd) {
             if ((s = qs_clover_inverse_odd(lat, m0, inv)) != QS_OK) break;
-            if ((s = qs_oo_inverse_apply(lat, inv, (const double *)b, a1, nrhs, 1.0)) != QS_OK) break;
-            if ((s = qs_dslash64_parity(lat, m0, a1, a2, nrhs, 0)) != QS_OK) break;   // D_eo D_oo^-1 b_o
-            if ((s = qs_even_mask(lat, (const double *)b, w.t, nrhs)) != QS_OK) break;
-            rw_axpy<<<ga, 256, 0, st>>>(w.t, a2, minus, w.len);                          // b'_e
-            rw_g5<<<rw_grid(nc), 256, 0, st>>>((double2 *)w.t, (const double2 *)w.t, nc);
-            qs_note_launches(2);
+            if ((s = qs_parity_pack(lat, (const double *)b, w.tmp, nrhs, 1)) != QS_OK) break;
+            if ((s = qs_hat_odd(lat, inv, w.tmp, a2, nrhs, 0, -1.0)) != QS_OK) break;       // -D_oo^-1 b_o
+            if ((s = qs_parity_pack(lat, (const double *)b, w.tmp, nrhs, 0)) != QS_OK) break;
+            if ((s = qs_hat_hop_even(lat, a2, w.tmp, 1.0, w.t, nrhs)) != QS_OK) break;      // b'_e
+            rw_g5<<<rw_grid(nc), 256, 0, st>>>((double2 *)w.t, (const double2 *)w.t, nc, 1);
+            qs_note_launches(1);
             if ((s = rw_cg(w, m0, 0.0, w.t, w.x, tol, max_iter, &it)) != QS_OK) break;
-            if ((s = qs_dhat_run(lat, m0, w.x, a1, nrhs, 1, w.dwork, inv)) != QS_OK) break;   // x_e
-            if ((s = qs_dslash64_parity(lat, m0, a1, a2, nrhs, 1)) != QS_OK) break;            // D_oe x_e
-            if ((s = rw_copy(w.t, b, bytes, st)) != QS_OK) break;
-            rw_axpy<<<ga, 256, 0, st>>>(w.t, a2, minus, w.len);                          // b_o - D_oe x_e
-            qs_note_launches(1);
-            if ((s = qs_oo_inverse_apply(lat, inv, w.t, a2, nrhs, 1.0)) != QS_OK) break;     // x_o
-            if ((s = rw_copy(x, a1, bytes, st)) != QS_OK) break;
-            rw_axpy<<<ga, 256, 0, st>>>((double *)x, a2, plus, w.len);
-            qs_note_launches(1);
+            if ((s = qs_dhat_run(lat, m0, w.x, a1, nrhs, 1, w.dwork, inv)) != QS_OK) break; // x_e
+            if ((s = qs_hat_odd(lat, inv, a1, w.t, nrhs, 1, -1.0)) != QS_OK) break;         // -D_oo^-1 D_oe x_e
+            if ((s = qs_parity_unpack(lat, a1, nullptr, (double *)x, nrhs, 0)) != QS_OK) break;
+            if ((s = qs_parity_unpack(lat, w.t, a2, (double *)x, nrhs, 1)) != QS_OK) break; // x_o
         } else {
-            rw_g5<<<rw_grid(nc), 256, 0, st>>>((double2 *)w.t, (const double2 *)b, nc);
+            rw_g5<<<rw_grid(nc), 256, 0, st>>>((double2 *)w.t, (const double2 *)b, nc, 0);
             qs_note_launches(1);
             if ((s = rw_cg(w, m0, 0.0, w.t, w.x, tol, max_iter, &it)) != QS_OK) break;
             double mm[64];
@@ -643,6 +759,7 @@ extern "C" int qs_solve_D(qs_lattice *lat, double m0, const void *b, void *x, in
         const cudaError_t e = cudaStreamSynchronize(st);
         if (e != cudaSuccess) { qs_record_cuda_error(e, "qs_solve_D"); s = QS_ECUDA; }
     } while (0);
+    rw_end(w);
     cudaFree(buf);
     if (iterations) *iterations = it;
     return s;
