@@ -36,6 +36,7 @@
 // storage (saves a separate pass over four vectors).
 #include "qs_internal.cuh"
 #include "dslash.cuh"
+#include "dslash64.cuh"
 #include "stencil.cuh"
 
 #include <cuda_bf16.h>
@@ -107,6 +108,19 @@ struct StF32Tiled {
 #pragma unroll
         for (int c = 0; c < 12; ++c) v[c] = __ldg(b + c * 16);
     }
+    // the 3 components of one spin
+    __device__ static void ld3(const char *__restrict__ base, int s, int spin, cf v[3])
+    {
+        const cf *b = reinterpret_cast<const cf *>(base) + ((int64_t)(s >> 4) * 12 + 3 * spin) * 16 + (s & 15);
+#pragma unroll
+        for (int c = 0; c < 3; ++c) v[c] = __ldg(b + c * 16);
+    }
+    __device__ static void st3(char *__restrict__ base, int s, int spin, const cf v[3], float)
+    {
+        cf *b = reinterpret_cast<cf *>(base) + ((int64_t)(s >> 4) * 12 + 3 * spin) * 16 + (s & 15);
+#pragma unroll
+        for (int c = 0; c < 3; ++c) b[c * 16] = v[c];
+    }
     // the 6 components of chiral block `blk` (spins 2 blk, 2 blk + 1)
     __device__ static void ld6(const char *__restrict__ base, int s, int blk, cf v[6])
     {
@@ -149,6 +163,18 @@ struct StF32Canon {
             v[2 * i] = make_float2(a.x, a.y);
             v[2 * i + 1] = make_float2(a.z, a.w);
         }
+    }
+    __device__ static void ld3(const char *__restrict__ base, int s, int spin, cf v[3])
+    {
+        const cf *b = reinterpret_cast<const cf *>(base) + (int64_t)s * 12 + 3 * spin;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) v[c] = __ldg(b + c);
+    }
+    __device__ static void st3(char *__restrict__ base, int s, int spin, const cf v[3], float)
+    {
+        cf *b = reinterpret_cast<cf *>(base) + (int64_t)s * 12 + 3 * spin;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) b[c] = v[c];
     }
     __device__ static void ld6(const char *__restrict__ base, int s, int blk, cf v[6])
     {
@@ -204,6 +230,30 @@ struct StScaled {
             float2 f = cvt(h);
             v[c] = make_float2(f.x * sc, f.y * sc);
         }
+    }
+    __device__ static void ld3(const char *__restrict__ base, int s, int spin, cf v[3])
+    {
+        const char *t = base + (int64_t)(s >> 4) * kTile;
+        const unsigned *w = reinterpret_cast<const unsigned *>(t) + 48 * spin + (s & 15);
+        const float sc = __ldg(reinterpret_cast<const float *>(t + 768) + (s & 15));
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            const unsigned u = __ldg(w + c * 16);
+            v[c] = mul2(dup(sc), cvt(*reinterpret_cast<const H2 *>(&u)));
+        }
+    }
+    // m: the site's largest component
+    __device__ static void st3(char *__restrict__ base, int s, int spin, const cf v[3], float m)
+    {
+        char *t = base + (int64_t)(s >> 4) * kTile;
+        const float inv = m > 0.f ? 1.0f / m : 0.f;
+        unsigned *w = reinterpret_cast<unsigned *>(t) + 48 * spin + (s & 15);
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            H2 h = pack(v[c].x * inv, v[c].y * inv);
+            w[c * 16] = *reinterpret_cast<unsigned *>(&h);
+        }
+        if (spin == 0) reinterpret_cast<float *>(t + 768)[s & 15] = m;
     }
     __device__ static void ld6(const char *__restrict__ base, int s, int blk, cf v[6])
     {
@@ -481,6 +531,79 @@ __global__ void __launch_bounds__(NT, MINB) dslash32_kernel(const __grid_constan
     for (int i = 0; i < gpb && r < a.nrhs; ++i, r += wr) site_kernel<S, CHEB>(a, p, r);
 }
 
+// ---- small problems: two threads per site (dslash64.cuh in FP32) ------------------------
+template <class S>
+struct Mem32 {
+    typedef float R;
+    typedef float2 V2;
+    __device__ static void ld3(const cf *__restrict__ in, int s, int spin, cf v[3])
+    {
+        S::ld3(reinterpret_cast<const char *>(in), s, spin, v);
+    }
+};
+
+// A pair thread's chain of loads and products is about 17 k cycles long, which is all the time
+// there is when the lattice has too few sites to fill the SMs; a quarter of the work per
+// thread then wins although links and SW words are loaded four times as often.  Up to 16 k
+// sites x right-hand sides 6.2 us against 8.2 us back to back, the same at 32 k, and slower from 48 k
+// on (FP32 and FP16 alike), hence the line at 24 k.  It is a line in the sites and vectors
+// alone, so the layouts of one problem always take the same arithmetic.
+constexpr int64_t kSplitSites = 24576;
+
+template <class S, bool CHEB>
+__global__ void __launch_bounds__(64, 10) dslash32_split_kernel(const __grid_constant__ D32 a)
+{
+    const int r = (int)(blockIdx.x % (unsigned)a.nrhs);
+    const int s0 = (int)(blockIdx.x / (unsigned)a.nrhs) * 32 + (int)(threadIdx.x >> 5) * 16 + (int)(threadIdx.x & 15);
+    const bool on = s0 < (int)a.g.Ns;
+    const Lane64 ln = qs_lane64(a.g, on ? s0 : (int)a.g.Ns - 1);
+    const int64_t off = (int64_t)r * a.vbytes;
+    const cf *in = reinterpret_cast<const cf *>(a.in + off);
+    const float dm = a.dmdev ? __ldg(a.dmdev + r) : a.dm[r];
+    cf up[3], low[3];
+    qs_hops64<Mem32<S>>(a.g, a.links, in, ln, up, low);
+    qs_diag64<Mem32<S>>(SwF32{a.clov + ln.c.p, a.g.Vphys}, in, ln, dm, up, low);
+    if (a.gamma5) {
+#pragma unroll
+        for (int i = 0; i < 3; ++i) low[i] = cneg(low[i]);
+    }
+    if (CHEB) {
+        const float cc = a.coef ? __ldg(a.coef) : a.c;
+        const float s1 = a.coef ? __ldg(a.coef + 1) : a.s1;
+        const float s2 = a.coef ? __ldg(a.coef + 2) : a.s2;
+#pragma unroll
+        for (int b = 0; b < 2; ++b) {
+            cf yv[3], xv[3];
+            S::ld3(a.y + off, ln.c.s, 2 * b + ln.q, yv);
+            S::ld3(a.x + off, ln.c.s, 2 * b + ln.q, xv);
+            cf *o = b ? low : up;
+#pragma unroll
+            for (int i = 0; i < 3; ++i) o[i] = fma2(dup(s1), fma2(dup(-cc), yv[i], o[i]), mul2(dup(-s2), xv[i]));
+        }
+    }
+    float m = 0.f;
+    if constexpr (S::kScaled) {
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+            m = fmaxf(m, fmaxf(fabsf(up[i].x), fabsf(up[i].y)));
+            m = fmaxf(m, fmaxf(fabsf(low[i].x), fabsf(low[i].y)));
+        }
+        m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 16));
+    }
+    if (!on) return;
+    S::st3(a.out + off, s0, ln.q, up, m);
+    S::st3(a.out + off, s0, 2 + ln.q, low, m);
+}
+
+template <class S>
+cudaError_t launch_split(const D32 &a, bool cheb, cudaStream_t st)
+{
+    const unsigned nb = (unsigned)((a.g.Ns + 31) / 32) * (unsigned)a.nrhs;
+    if (cheb) dslash32_split_kernel<S, true><<<nb, 64, 0, st>>>(a);
+    else dslash32_split_kernel<S, false><<<nb, 64, 0, st>>>(a);
+    return cudaGetLastError();
+}
+
 // Batched persistent form: work items (lattice i, site tile, right-hand side) numbered
 // lattice by lattice, right-hand sides fastest; each block takes items w = blockIdx.x,
 // blockIdx.x + gridDim.x, ...
@@ -588,6 +711,7 @@ cudaError_t launch_variant(int v, const D32 &a, cudaStream_t st)
 template <class S>
 cudaError_t launch_storage(int v, bool cheb, const D32 &a, cudaStream_t st)
 {
+    if (a.g.Ns * a.nrhs <= kSplitSites) return launch_split<S>(a, cheb, st);
     return cheb ? launch_variant<S, true>(v, a, st) : launch_variant<S, false>(v, a, st);
 }
 

@@ -1,8 +1,10 @@
 """Every launch variant of the operator against the oracle.
 
 The autotuner picks one variant per shape, so each is forced in turn (a child process with a
-tune cache that names it) on lattices whose sites fill no block (2^3 x 3: 24 physical sites,
-6^3 x 5: 1080) and on blocks of vectors that fill no group of 2 or 4.  Tolerances, max-norm
+tune cache that names it) on lattices whose sites fill no block (6^3 x 5: 1080 physical sites,
+10^3 x 3: 3000) and on blocks of vectors that fill no group of 2 or 4.  Problems of up to 24576
+sites x vectors (2^3 x 3, 4^4 and the small blocks of 6^3 x 5) take the FP32 kernel with two
+threads per site instead, whichever variant is named.  Tolerances, max-norm
 relative to the largest output component: 1e-5 for FP32 storage; for FP16 storage half a unit
 in the last place at 1 relative to the site's largest component (2^-11), twice that allowed.  FP64: 1e-13 (about 300 roundings of
 2^-53 each on the longest chain, of terms no larger than the output's scale).
@@ -15,8 +17,8 @@ import pytest
 
 pytestmark = pytest.mark.gpu
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
-SHAPES = [(2, 3, 0b001, False), (6, 5, 0b111, True), (4, 4, 0b011, False)]
-NRHS = [1, 3, 6]
+SHAPES = [(6, 5, 0b111, True, [12, 13, 15]), (10, 3, 0b011, False, [5])]
+SMALL = [(2, 3, 0b001, False, [1, 3, 6]), (6, 5, 0b111, True, [1, 3, 11]), (4, 4, 0b011, True, [6])]
 
 CHILD = r"""
 import sys
@@ -27,13 +29,13 @@ import paper_2108_11989_gb300 as qs
 from oracle.dirac import WilsonDirac
 from synth_inputs import make_config, random_spinor
 from test_gpu_dslash import TOL16, pack16
-for L, T, mask, anti in %(shapes)r:
+for L, T, mask, anti, rhs in %(shapes)r:
     cfg = make_config(T=T, L=L, eps=0.6, theta_sigma=0.4, csw_su3=1.9, csw_u1=1.0, seed=3, cstar_mask=mask,
                       t_antiperiodic=anti)
     lat = qs.Lattice(L, T, mask, anti)
     lat.load_gauge(cfg.su3, cfg.theta, cfg.csw_su3, cfg.csw_u1)
     op, ns = WilsonDirac(cfg), cfg.n_sites
-    for nrhs in %(nrhs)r:
+    for nrhs in rhs:
         psi = random_spinor(7, T, L, nrhs).astype(np.complex64).astype(np.complex128)
         ref = np.stack([op.apply_Q(psi[r].reshape(-1), 0.07) for r in range(nrhs)]).reshape(nrhs, ns, 12)
         x = torch.from_numpy(np.ascontiguousarray(psi).view(np.float64).copy()).float().cuda().reshape(-1)
@@ -63,11 +65,11 @@ def test_forced_variant_matches_oracle(variant, tmp_path):
     gpu = torch.cuda.get_device_name(0).replace(" ", "_")
     cache = tmp_path / "tune"
     cache.write_text("".join(f"{gpu}|dslash32p|{st}|0|{n}|{L}x{T} {variant}\n"
-                             for L, T, _, _ in SHAPES for n in NRHS for st in range(4)))
-    r = subprocess.run([sys.executable, "-c", CHILD % {"root": ROOT, "shapes": SHAPES, "nrhs": NRHS}],
+                             for L, T, _, _, rhs in SHAPES + SMALL for n in rhs for st in range(4)))
+    r = subprocess.run([sys.executable, "-c", CHILD % {"root": ROOT, "shapes": SHAPES + SMALL}],
                        env=dict(os.environ, QS_TUNE_CACHE=str(cache)), capture_output=True, text=True, timeout=300)
     assert r.returncode == 0, r.stderr[-2000:]
-    assert len(cache.read_text().splitlines()) == len(SHAPES) * len(NRHS) * 4   # nothing was timed: the forced one ran
+    assert len(cache.read_text().splitlines()) == 11 * 4   # nothing was timed: the forced one ran
 
 
 CHILD64 = r"""
@@ -78,13 +80,13 @@ import torch
 import paper_2108_11989_gb300 as qs
 from oracle.dirac import WilsonDirac
 from synth_inputs import make_config, random_spinor
-for L, T, mask, anti in %(shapes)r:
+for L, T, mask, anti, rhs in %(shapes)r:
     cfg = make_config(T=T, L=L, eps=0.6, theta_sigma=0.4, csw_su3=1.9, csw_u1=1.0, seed=3, cstar_mask=mask,
                       t_antiperiodic=anti)
     lat = qs.Lattice(L, T, mask, anti)
     lat.load_gauge(cfg.su3, cfg.theta, cfg.csw_su3, cfg.csw_u1)
     op, ns = WilsonDirac(cfg), cfg.n_sites
-    for nrhs in %(nrhs)r:
+    for nrhs in rhs:
         psi = random_spinor(7, T, L, nrhs)
         ref = np.stack([op.apply_D(psi[r].reshape(-1), 0.07) for r in range(nrhs)]).reshape(nrhs, ns, 12)
         x = torch.from_numpy(np.ascontiguousarray(psi).view(np.float64).copy()).cuda().reshape(-1)
@@ -105,8 +107,8 @@ def test_forced_fp64_variant_matches_oracle(variant, tmp_path):
     gpu = torch.cuda.get_device_name(0).replace(" ", "_")
     cache = tmp_path / "tune"
     cache.write_text("".join(f"{gpu}|dslash64s|{soa}|0|{n}|{L}x{T} {variant}\n"
-                             for L, T, _, _ in SHAPES for n in NRHS for soa in range(2)))
-    r = subprocess.run([sys.executable, "-c", CHILD64 % {"root": ROOT, "shapes": SHAPES, "nrhs": NRHS}],
+                             for L, T, _, _, rhs in SHAPES + SMALL for n in rhs for soa in range(2)))
+    r = subprocess.run([sys.executable, "-c", CHILD64 % {"root": ROOT, "shapes": SHAPES + SMALL}],
                        env=dict(os.environ, QS_TUNE_CACHE=str(cache)), capture_output=True, text=True, timeout=300)
     assert r.returncode == 0, r.stderr[-2000:]
-    assert len(cache.read_text().splitlines()) == len(SHAPES) * len(NRHS) * 2
+    assert len(cache.read_text().splitlines()) == 11 * 2
