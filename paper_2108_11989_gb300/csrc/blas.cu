@@ -30,16 +30,44 @@ __device__ __forceinline__ double block_sum(double v)
     return v;
 }
 
-template <typename R>
-__global__ void norm2_part(const R *__restrict__ v, int64_t nr, double *part)
+// (hi, lo) += x, with hi + lo exact to the rounding of the final add (Knuth's two-sum)
+__device__ __forceinline__ void two_sum_acc(float &hi, float &lo, float x)
 {
-    const R *x = v + (int64_t)blockIdx.y * nr;
-    R acc = 0;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < nr; i += (int64_t)gridDim.x * blockDim.x) {
-        R a = x[i];
-        acc += a * a;
-    }
-    double s = block_sum((double)acc);
+    const float s = hi + x;
+    const float bp = s - hi;
+    const float err = (hi - (s - bp)) + (x - bp);
+    hi = s;
+    lo += err;
+}
+__device__ __forceinline__ void two_sum_acc(double &hi, double &, double x) { hi += x; }
+
+template <typename R> struct Vec16;   // 16 bytes of reals
+template <> struct Vec16<float> { typedef float4 T; };
+template <> struct Vec16<double> { typedef double2 T; };
+__device__ __forceinline__ float sum_sq(float4 a) { return fmaf(a.w, a.w, fmaf(a.z, a.z, fmaf(a.y, a.y, a.x * a.x))); }
+__device__ __forceinline__ double sum_sq(double2 a) { return fma(a.y, a.y, a.x * a.x); }
+__device__ __forceinline__ float4 diff(float4 a, float t, float4 b)
+{
+    return make_float4(fmaf(-t, b.x, a.x), fmaf(-t, b.y, a.y), fmaf(-t, b.z, a.z), fmaf(-t, b.w, a.w));
+}
+__device__ __forceinline__ double2 diff(double2 a, double t, double2 b) { return make_double2(fma(-t, b.x, a.x), fma(-t, b.y, a.y)); }
+
+// Streaming kernels over [k][nr]: 16-byte words (nr is a multiple of 24 x 16), blocks of
+// red_blocks(nr, k) per vector, so that a block has some two thousand reals to itself; with 608
+// blocks per vector whatever its length, an 8^3 x 12 CG update of 16 vectors was 9728 blocks of
+// two reals per thread and took 69 us instead of 15.  FP32 sums are kept as a two-sum pair.
+template <typename R>
+__global__ void __launch_bounds__(256) norm2_part(const R *__restrict__ v, int64_t nr, double *part,
+                                                  const int *__restrict__ live = nullptr)
+{
+    typedef typename Vec16<R>::T T;
+    if (live && !live[blockIdx.y]) return;
+    const int64_t n = nr * (int64_t)sizeof(R) / 16;
+    const T *x = reinterpret_cast<const T *>(v) + (int64_t)blockIdx.y * n;
+    R acc = 0, lo = 0;
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
+        two_sum_acc(acc, lo, sum_sq(x[i]));
+    double s = block_sum((double)acc + (double)lo);
     if (threadIdx.x == 0) part[blockIdx.y * gridDim.x + blockIdx.x] = s;
 }
 
@@ -54,38 +82,18 @@ __global__ void finalize_sum(const double *part, int nb, int stride_out, double 
 }
 
 template <typename R>
-__global__ void dot_part(const R *__restrict__ a, const R *__restrict__ b, int64_t nr, double *part)
+__global__ void __launch_bounds__(256) resid_part(const R *__restrict__ a, const R *__restrict__ b, const double *theta,
+                                                  int64_t nr, double *part)
 {
-    const R *x = a + (int64_t)blockIdx.y * nr;
-    const R *y = b + (int64_t)blockIdx.y * nr;
-    R re = 0, im = 0;
-    int64_t nc = nr / 2;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < nc; i += (int64_t)gridDim.x * blockDim.x) {
-        R ar = x[2 * i], ai = x[2 * i + 1], br = y[2 * i], bi = y[2 * i + 1];
-        re += ar * br + ai * bi;
-        im += ar * bi - ai * br;
-    }
-    double sr = block_sum((double)re);
-    double si = block_sum((double)im);
-    if (threadIdx.x == 0) {
-        part[(2 * blockIdx.y) * gridDim.x + blockIdx.x] = sr;
-        part[(2 * blockIdx.y + 1) * gridDim.x + blockIdx.x] = si;
-    }
-}
-
-template <typename R>
-__global__ void resid_part(const R *__restrict__ a, const R *__restrict__ b, const double *theta,
-                           int64_t nr, double *part)
-{
-    const R *x = a + (int64_t)blockIdx.y * nr;
-    const R *y = b + (int64_t)blockIdx.y * nr;
+    typedef typename Vec16<R>::T T;
+    const int64_t n = nr * (int64_t)sizeof(R) / 16;
+    const T *x = reinterpret_cast<const T *>(a) + (int64_t)blockIdx.y * n;
+    const T *y = reinterpret_cast<const T *>(b) + (int64_t)blockIdx.y * n;
     const R t = (R)theta[blockIdx.y];
-    R acc = 0;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < nr; i += (int64_t)gridDim.x * blockDim.x) {
-        R d = x[i] - t * y[i];
-        acc += d * d;
-    }
-    double s = block_sum((double)acc);
+    R acc = 0, lo = 0;
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
+        two_sum_acc(acc, lo, sum_sq(diff(x[i], t, y[i])));
+    double s = block_sum((double)acc + (double)lo);
     if (threadIdx.x == 0) part[blockIdx.y * gridDim.x + blockIdx.x] = s;
 }
 
@@ -97,17 +105,6 @@ __global__ void resid_part(const R *__restrict__ a, const R *__restrict__ b, con
 // shared memory at the end, in a fixed order.  LOWP: values rounded to FP32, products
 // and the sum over one chunk in FP32, chunk sums added in FP64.
 #define GE 64
-// (hi, lo) += x, with hi + lo exact to the rounding of the final add (Knuth's two-sum)
-__device__ __forceinline__ void two_sum_acc(float &hi, float &lo, float x)
-{
-    const float s = hi + x;
-    const float bp = s - hi;
-    const float err = (hi - (s - bp)) + (x - bp);
-    hi = s;
-    lo += err;
-}
-__device__ __forceinline__ void two_sum_acc(double &hi, double &lo, double x) { hi += x; }
-
 template <bool LOWP, typename TIn = double2>
 __global__ void __launch_bounds__(256, LOWP ? 2 : 1) gram_tile_kernel(const TIn *__restrict__ A_, int ka,
                                                            const TIn *__restrict__ B_, int kb, int64_t nc,
@@ -411,66 +408,88 @@ __global__ void map_scalars_kernel(const double *in, double *out, int k, int mod
 }
 
 // ---- CG (FP32 vectors, FP64 scalars) ----------------------------------------
-__global__ void cg_update_kernel(float *__restrict__ x, float *__restrict__ r, const float *__restrict__ p,
-                                 const float *__restrict__ ap, CgScalars s, int64_t nr, double *part)
+// An iteration is the operator's launches, the sums of |Q p|^2 and the two kernels below, whose
+// blocks sum the partial sums they need themselves in a fixed order, so that no launch is spent
+// on scalars.  The scalars live in two slots: an iteration reads slot o and writes 1 - o.
+// Vectors that have converged are skipped.
+__device__ double all_parts(const double *part, int nb)
 {
-    int q = blockIdx.y;
-    double al = (s.active[q] && s.pap[q] > 0) ? s.rr[q] / s.pap[q] : 0.0;
-    float a = (float)al;
-    float *xq = x + (int64_t)q * nr, *rq = r + (int64_t)q * nr;
-    const float *pq = p + (int64_t)q * nr, *aq = ap + (int64_t)q * nr;
-    float acc = 0;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < nr; i += (int64_t)gridDim.x * blockDim.x) {
-        xq[i] += a * pq[i];
-        float rv = rq[i] - a * aq[i];
-        rq[i] = rv;
-        acc += rv * rv;
-    }
-    double sm = block_sum((double)acc);
-    if (threadIdx.x == 0) part[q * gridDim.x + blockIdx.x] = sm;
-}
-
-__global__ void cg_finalize_kernel(CgScalars s, double tol2, int k, const double *part, int nb, int *nactive)
-{
-    __shared__ int cnt;
-    if (threadIdx.x == 0) cnt = 0;
+    __shared__ double d;
+    double acc = 0;
+    for (int i = threadIdx.x; i < nb; i += blockDim.x) acc += part[i];
+    acc = block_sum(acc);
+    if (threadIdx.x == 0) d = acc;
     __syncthreads();
-    for (int q = 0; q < k; ++q) {
-        double acc = 0;
-        for (int i = threadIdx.x; i < nb; i += blockDim.x) acc += part[q * nb + i];
-        double rn = block_sum(acc);
-        if (threadIdx.x == 0) {
-            int act = s.active[q];
-            s.beta[q] = (act && s.rr[q] > 0) ? rn / s.rr[q] : 0.0;
-            if (act) s.rr[q] = rn;
-            act = act && (rn > tol2 * s.rr0[q]) && isfinite(rn);
-            s.active[q] = act;
-            cnt += act;
-        }
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) *nactive = cnt;
+    return d;
 }
 
-__global__ void cg_p_kernel(float *__restrict__ p, const float *__restrict__ r, CgScalars s, int64_t nr)
+// r -= alpha Q^2 p, alpha = |r|^2 / |Q p|^2; rpart = shares of |r|^2
+__global__ void __launch_bounds__(256) cg_r_kernel(float4 *__restrict__ r, const float4 *__restrict__ ap, CgScalars s, int o,
+                                                   int64_t n, const double *__restrict__ ppart, double *__restrict__ rpart)
 {
-    int q = blockIdx.y;
-    if (!s.active[q]) return;
-    float b = (float)s.beta[q];
-    float *pq = p + (int64_t)q * nr;
-    const float *rq = r + (int64_t)q * nr;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < nr; i += (int64_t)gridDim.x * blockDim.x)
-        pq[i] = rq[i] + b * pq[i];
+    const int q = blockIdx.y;
+    if (!s.live[o][q]) return;
+    const double pap = all_parts(ppart + (int64_t)q * gridDim.x, gridDim.x);
+    const float a = pap > 0 ? (float)(s.rr[o][q] / pap) : 0.f;
+    float4 *rq = r + q * n;
+    const float4 *aq = ap + q * n;
+    float acc = 0, lo = 0;
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+        const float4 v = diff(rq[i], a, aq[i]);
+        rq[i] = v;
+        two_sum_acc(acc, lo, sum_sq(v));
+    }
+    const double sm = block_sum((double)acc + (double)lo);
+    if (threadIdx.x == 0) rpart[q * gridDim.x + blockIdx.x] = sm;
+}
+
+// x += alpha p, p = r + beta p, beta = |r|^2 / |r_old|^2; the vector lives on while
+// |r|^2 > tol2 |r_0|^2
+__global__ void __launch_bounds__(256) cg_xp_kernel(float4 *__restrict__ x, float4 *__restrict__ p,
+                                                    const float4 *__restrict__ r, CgScalars s, int o, int64_t n,
+                                                    const double *__restrict__ ppart, const double *__restrict__ rpart,
+                                                    double tol2)
+{
+    const int q = blockIdx.y;
+    const bool first = blockIdx.x == 0 && threadIdx.x == 0;
+    if (!s.live[o][q]) {
+        if (first) s.live[1 - o][q] = 0;
+        return;
+    }
+    const double rr = s.rr[o][q];
+    const double pap = all_parts(ppart + (int64_t)q * gridDim.x, gridDim.x);
+    __syncthreads();
+    const double rn = all_parts(rpart + (int64_t)q * gridDim.x, gridDim.x);
+    const float a = pap > 0 ? (float)(rr / pap) : 0.f, b = rr > 0 ? (float)(rn / rr) : 0.f;
+    if (first) {
+        s.rr[1 - o][q] = rn;
+        s.live[1 - o][q] = rn > tol2 * s.rr0[q] && isfinite(rn);
+    }
+    float4 *xq = x + q * n, *pq = p + q * n;
+    const float4 *rq = r + q * n;
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+        const float4 v = pq[i];
+        xq[i] = diff(xq[i], -a, v);
+        pq[i] = diff(rq[i], -b, v);
+    }
 }
 
 __global__ void cg_init_kernel(CgScalars s, const double *rr, int k)
 {
     int q = threadIdx.x;
     if (q >= k) return;
-    s.rr[q] = rr[q];
+    s.rr[0][q] = rr[q];
     s.rr0[q] = rr[q];
-    s.beta[q] = 0;
-    s.active[q] = rr[q] > 0;
+    s.live[0][q] = rr[q] > 0;
+}
+
+// blocks per vector of the reductions: two to eight per SM over the k vectors
+inline int red_blocks(int64_t nr, int k)
+{
+    int64_t b = nr / 2048, top = 1216 / k;
+    if (b > top) b = top;
+    if (b > QS_RED_BLOCKS) b = QS_RED_BLOCKS;
+    return b < 1 ? 1 : (int)b;
 }
 
 inline int grid_for(int64_t n, int per = 256)
@@ -484,9 +503,9 @@ inline int grid_for(int64_t n, int per = 256)
 template <typename R>
 cudaError_t qs_norm2(const R *v, int k, int64_t nr, double *part, double *out, cudaStream_t st)
 {
-    dim3 g(QS_RED_BLOCKS, k);
-    norm2_part<R><<<g, QS_RED_THREADS, 0, st>>>(v, nr, part);
-    finalize_sum<<<k, 256, 0, st>>>(part, QS_RED_BLOCKS, 1, out);
+    const int nb = red_blocks(nr, k);
+    norm2_part<R><<<dim3(nb, k), 256, 0, st>>>(v, nr, part);
+    finalize_sum<<<k, 256, 0, st>>>(part, nb, 1, out);
     qs_note_launches(2);
     return cudaGetLastError();
 }
@@ -494,24 +513,12 @@ template cudaError_t qs_norm2<float>(const float *, int, int64_t, double *, doub
 template cudaError_t qs_norm2<double>(const double *, int, int64_t, double *, double *, cudaStream_t);
 
 template <typename R>
-cudaError_t qs_dot(const R *a, const R *b, int k, int64_t nr, double *part, double *out, cudaStream_t st)
-{
-    dim3 g(QS_RED_BLOCKS, k);
-    dot_part<R><<<g, QS_RED_THREADS, 0, st>>>(a, b, nr, part);
-    finalize_sum<<<2 * k, 256, 0, st>>>(part, QS_RED_BLOCKS, 1, out);
-    qs_note_launches(2);
-    return cudaGetLastError();
-}
-template cudaError_t qs_dot<float>(const float *, const float *, int, int64_t, double *, double *, cudaStream_t);
-template cudaError_t qs_dot<double>(const double *, const double *, int, int64_t, double *, double *, cudaStream_t);
-
-template <typename R>
 cudaError_t qs_resid2(const R *a, const R *b, const double *theta, int k, int64_t nr,
                       double *part, double *out, cudaStream_t st)
 {
-    dim3 g(QS_RED_BLOCKS, k);
-    resid_part<R><<<g, QS_RED_THREADS, 0, st>>>(a, b, theta, nr, part);
-    finalize_sum<<<k, 256, 0, st>>>(part, QS_RED_BLOCKS, 1, out);
+    const int nb = red_blocks(nr, k);
+    resid_part<R><<<dim3(nb, k), 256, 0, st>>>(a, b, theta, nr, part);
+    finalize_sum<<<k, 256, 0, st>>>(part, nb, 1, out);
     qs_note_launches(2);
     return cudaGetLastError();
 }
@@ -679,27 +686,17 @@ cudaError_t qs_map_scalars(const double *in, double *out, int k, int mode, cudaS
     return cudaGetLastError();
 }
 
-cudaError_t qs_cg_update(float *x, float *r, const float *p, const float *ap, CgScalars s, int k, int64_t nr,
-                         double *part, cudaStream_t st)
+// t = Q p, ap = Q t are computed; the rest of iteration `it`
+cudaError_t qs_cg_step(float *x, float *r, float *p, const float *t, const float *ap, const CgScalars &s, int it, double tol2,
+                       int k, int64_t nr, double *part, cudaStream_t st)
 {
-    dim3 g(QS_RED_BLOCKS, k);
-    cg_update_kernel<<<g, QS_RED_THREADS, 0, st>>>(x, r, p, ap, s, nr, part);
-    qs_note_launches(1);
-    return cudaGetLastError();
-}
-
-cudaError_t qs_cg_finalize(CgScalars s, double tol2, int k, double *part, int *nactive, cudaStream_t st)
-{
-    cg_finalize_kernel<<<1, 256, 0, st>>>(s, tol2, k, part, QS_RED_BLOCKS, nactive);
-    qs_note_launches(1);
-    return cudaGetLastError();
-}
-
-cudaError_t qs_cg_pupdate(float *p, const float *r, CgScalars s, int k, int64_t nr, cudaStream_t st)
-{
-    dim3 g(grid_for(nr) / k + 1, k);
-    cg_p_kernel<<<g, 256, 0, st>>>(p, r, s, nr);
-    qs_note_launches(1);
+    const int nb = red_blocks(nr, k), o = it & 1;
+    const dim3 g(nb, k);
+    double *rpart = part + (size_t)QS_RED_BLOCKS * 64;
+    norm2_part<float><<<g, 256, 0, st>>>(t, nr, part, s.live[o]);   // <p, Q^2 p> = |Q p|^2
+    cg_r_kernel<<<g, 256, 0, st>>>((float4 *)r, (const float4 *)ap, s, o, nr / 4, part, rpart);
+    cg_xp_kernel<<<g, 256, 0, st>>>((float4 *)x, (float4 *)p, (const float4 *)r, s, o, nr / 4, part, rpart, tol2);
+    qs_note_launches(3);
     return cudaGetLastError();
 }
 

@@ -2,15 +2,11 @@
 #pragma once
 #include "qs_internal.cuh"
 
-#define QS_RED_BLOCKS 608      // partial sums per vector (4 x 152 SMs)
-#define QS_RED_THREADS 256
+#define QS_RED_BLOCKS 608      // most partial sums per vector (4 x 152 SMs)
 
 // v has k vectors of nr reals each ([k][nr]); out[r] = sum over vector r of v^2 (FP64)
 template <typename R>
 cudaError_t qs_norm2(const R *v, int k, int64_t nr, double *part, double *out, cudaStream_t st);
-// out[r] = <a_r, b_r> (complex, conj on a), out as [k][2]
-template <typename R>
-cudaError_t qs_dot(const R *a, const R *b, int k, int64_t nr, double *part, double *out, cudaStream_t st);
 // out[r] = || a_r - theta[r] b_r ||^2 (FP64 or FP32 vectors, FP64 sum, theta on device)
 template <typename R>
 cudaError_t qs_resid2(const R *a, const R *b, const double *theta, int k, int64_t nr,
@@ -56,15 +52,13 @@ cudaError_t qs_partner32(const float *in, float *out, const Geom &g, int k, cuda
 cudaError_t qs_chol_rinv(const double2 *G, int k, double2 *Rinv, int *info, cudaStream_t st);
 cudaError_t qs_herm_eig(const double2 *H, int k, double *evals, double2 *Y, int *info, cudaStream_t st);
 
-// CG helpers (FP32 vectors, per-rhs scalars on device)
+// CG helpers (FP32 vectors, per-rhs scalars on device, two slots: see qs_cg_step)
 struct CgScalars {
-    double *rr, *rr0, *pap, *beta;
-    int *active;
+    double *rr[2], *rr0;
+    int *live[2];
 };
-cudaError_t qs_cg_update(float *x, float *r, const float *p, const float *ap, CgScalars s, int k, int64_t nr,
-                         double *part, cudaStream_t st);
-cudaError_t qs_cg_finalize(CgScalars s, double tol2, int k, double *part, int *nactive, cudaStream_t st);
-cudaError_t qs_cg_pupdate(float *p, const float *r, CgScalars s, int k, int64_t nr, cudaStream_t st);
+cudaError_t qs_cg_step(float *x, float *r, float *p, const float *t, const float *ap, const CgScalars &s, int it, double tol2,
+                       int k, int64_t nr, double *part, cudaStream_t st);
 cudaError_t qs_cg_init(CgScalars s, const double *rr, int k, cudaStream_t st);
 
 // Ritz values (sorted by |theta|) and residual norms of the current block

@@ -343,9 +343,10 @@ static int prec_of_storage(int storage)
 
 int qs_d32_run(qs_lattice *lat, int storage, const double *m0, const void *in, void *out, int nrhs, int gamma5,
                const void *cheb_y, const void *cheb_x, double cheb_c, double cheb_s1, double cheb_s2,
-               const float *coef_dev, const float *dm_dev)
+               const float *coef_dev, const float *dm_dev, const int *live_dev)
 {
     D32Call c;
+    c.live = live_dev;
     c.coef_dev = coef_dev;
     c.dm_dev = dm_dev;
     c.g = lat->g;

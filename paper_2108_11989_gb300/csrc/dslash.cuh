@@ -67,6 +67,7 @@ struct D32Call {
     const double *m0;      // host, nrhs masses (ignored where dm_dev is set)
     const float *coef_dev; // NULL, or device (c, s1, s2) of the Chebyshev epilogue
     const float *dm_dev;   // NULL, or device 4 + m0 per right-hand side
+    const int *live;       // NULL, or device flags: right-hand sides with 0 are skipped
 };
 int qs_d32_nvariants();
 int64_t qs_d32_vec_bytes(int storage, int64_t Ns);

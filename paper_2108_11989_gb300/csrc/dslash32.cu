@@ -376,6 +376,7 @@ struct D32 {
     // device-side overrides (for launches replayed from a CUDA graph): if set, (c, s1, s2)
     // are read from coef[0..2] and 4 + m0 of right-hand side r from dmdev[r]
     const float *coef, *dmdev;
+    const int *live;    // NULL, or flags: right-hand sides with live[r] = 0 are skipped
 };
 
 // acc += upper and lower parts of M h for a neighbour's spinor, M = U (FW, sigma = +1),
@@ -487,6 +488,7 @@ __device__ __forceinline__ void finish_site(const D32 &a, int64_t off, int s, cf
 template <class S, bool CHEB>
 __device__ __forceinline__ void site_kernel(const D32 &a, int p, int r)
 {
+    if (a.live && !a.live[r]) return;
     const int row = p / a.g.L;
     const Site c = site_of(a.g, p + row * a.g.L);   // x < L: s = row 2L + x, p = row L + x
     const int64_t off = (int64_t)r * a.vbytes;
@@ -554,6 +556,7 @@ template <class S, bool CHEB>
 __global__ void __launch_bounds__(64, 10) dslash32_split_kernel(const __grid_constant__ D32 a)
 {
     const int r = (int)(blockIdx.x % (unsigned)a.nrhs);
+    if (a.live && !a.live[r]) return;
     const int s0 = (int)(blockIdx.x / (unsigned)a.nrhs) * 32 + (int)(threadIdx.x >> 5) * 16 + (int)(threadIdx.x & 15);
     const bool on = s0 < (int)a.g.Ns;
     const Lane64 ln = qs_lane64(a.g, on ? s0 : (int)a.g.Ns - 1);
@@ -757,6 +760,7 @@ cudaError_t qs_d32_batch_launch(const D32BatchItem *items, int n, int storage, i
         a.gamma5 = gamma5;
         a.c = a.s1 = a.s2 = 0.f;
         a.coef = a.dmdev = nullptr;
+        a.live = nullptr;
         for (int r = 0; r < it.nrhs; ++r) a.dm[r] = (float)(4.0 + it.m0[r]);
         b.off[i] = off;
         const double items_i = (double)((it.g.Vphys + 127) / 128) * it.nrhs;
@@ -802,6 +806,7 @@ cudaError_t qs_d32_launch(const D32Call &c, int variant, cudaStream_t st)
     for (int r = 0; r < c.nrhs; ++r) a.dm[r] = c.m0 ? (float)(4.0 + c.m0[r]) : 0.f;
     a.coef = c.coef_dev;
     a.dmdev = c.dm_dev;
+    a.live = c.live;
     const bool cheb = c.cheb;
     switch (c.storage) {
     case QS_D32_F32_TILED: return launch_storage<StF32Tiled>(variant, cheb, a, st);

@@ -30,6 +30,9 @@ struct FilterGraph {
 #define QS_GRAPH_MAX_DEG 511
 #define QS_NGRAPH 6
 
+#define CG_LAG 2     // CG flag reads the host may be behind
+#define CG_POLL 4    // iterations between two of them
+
 struct Workspace {
     FilterGraph fg[QS_NGRAPH];
     int nfg;
@@ -43,7 +46,9 @@ struct Workspace {
     double *part;         // reduction partials
     double2 *G, *Rinv, *Hm, *Ym;
     double *ds;           // device scalars, S_NSLOT slots of 64
-    int *di;              // device ints, 64 + 8
+    int *di;              // device ints: 64 CG flags, 8 status words, 64 CG flags
+    int *hlive;           // pinned: CG_LAG + 1 copies of the CG flags
+    cudaEvent_t ev[CG_LAG + 1];
     double *hp;           // pinned host mirror of ds (S_NSLOT x 64)
     int *hi;              // pinned host ints (64 + 8)
     int have_V;
@@ -55,7 +60,7 @@ struct Workspace {
 static float *V32(Workspace *w);
 static float *QV32(Workspace *w);
 static float *T32(Workspace *w);
-enum { S_TMP = 0, S_THETA = 1, S_COEF = 2, S_RR = 3, S_RR0 = 4, S_PAP = 5, S_BETA = 6, S_ONES = 7, S_RN = 8,
+enum { S_TMP = 0, S_THETA = 1, S_COEF = 2, S_RR = 3, S_RR0 = 4, S_RR1 = 5, S_ONES = 7, S_RN = 8,
        S_DOT = 9 /* two slots */, S_VN = 11, S_NSLOT = 12 };
 
 static void ws_free(Workspace *w)
@@ -69,7 +74,9 @@ static void ws_free(Workspace *w)
     for (int i = 0; i < 3; ++i) cudaFree(w->f32b[i]);
     cudaFree(w->part); cudaFree(w->G); cudaFree(w->Rinv); cudaFree(w->Hm); cudaFree(w->Ym);
     cudaFree(w->ds); cudaFree(w->di);
-    cudaFreeHost(w->hp); cudaFreeHost(w->hi);
+    cudaFreeHost(w->hp); cudaFreeHost(w->hi); cudaFreeHost(w->hlive);
+    for (auto e : w->ev)
+        if (e) cudaEventDestroy(e);
     free(w);
 }
 
@@ -103,12 +110,14 @@ static int ws_alloc(qs_lattice *lat, Workspace *w, int k)
     CK(cudaMalloc(&w->Hm, 64 * 64 * sizeof(double2)));
     CK(cudaMalloc(&w->Ym, 64 * 64 * sizeof(double2)));
     CK(cudaMalloc(&w->ds, S_NSLOT * 64 * sizeof(double)));
-    CK(cudaMalloc(&w->di, 72 * sizeof(int)));
+    CK(cudaMalloc(&w->di, 136 * sizeof(int)));
     CK(cudaMallocHost(&w->hp, S_NSLOT * 64 * sizeof(double)));
     CK(cudaMallocHost(&w->hi, 72 * sizeof(int)));
+    CK(cudaMallocHost(&w->hlive, (CG_LAG + 1) * 64 * sizeof(int)));
+    for (auto &e : w->ev) CK(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
     CK(cudaMalloc(&w->coef_dev, (3 * QS_GRAPH_MAX_DEG + 64) * sizeof(float)));
     CK(cudaMallocHost(&w->coef_host, (3 * QS_GRAPH_MAX_DEG + 64) * sizeof(float)));
-    CK(cudaMemsetAsync(w->di, 0, 72 * sizeof(int), lat->stream));
+    CK(cudaMemsetAsync(w->di, 0, 136 * sizeof(int), lat->stream));
     for (int i = 0; i < 64; ++i) w->hp[i] = 1.0;
     CK(cudaMemcpyAsync(DS(w, S_ONES), w->hp, 64 * sizeof(double), cudaMemcpyHostToDevice, lat->stream));
     CK(cudaStreamSynchronize(lat->stream));
@@ -442,33 +451,45 @@ static int cheb_filter64(qs_lattice *lat, Workspace *w, double m0, int k, int d,
     return QS_OK;
 }
 
-// FP32 CG on Q^2 for k right-hand sides in r (overwritten); solution in x.
+// FP32 CG on Q^2 for k right-hand sides in r (overwritten); solution in x.  The host never waits
+// for an iteration it has just launched: every CG_POLL iterations it copies the flags of the
+// vectors that still iterate, and it reads a copy CG_LAG copies later; by then all kernels skip
+// the vectors that have converged, the operator among them.
 static int cg_f32(qs_lattice *lat, Workspace *w, double m0, int k, float *x, float *r, float *p, float *t,
                   float *ap, double tol, int maxit, int *iters)
 {
     cudaStream_t st = lat->stream;
     CgScalars s;
-    s.rr = DS(w, S_RR); s.rr0 = DS(w, S_RR0); s.pap = DS(w, S_PAP); s.beta = DS(w, S_BETA);
-    s.active = w->di;
+    s.rr[0] = DS(w, S_RR); s.rr[1] = DS(w, S_RR1); s.rr0 = DS(w, S_RR0);
+    s.live[0] = w->di; s.live[1] = w->di + 72;
     size_t bytes = (size_t)k * w->nr * sizeof(float);
     CK(cudaMemsetAsync(x, 0, bytes, st));
     CK(cudaMemcpyAsync(p, r, bytes, cudaMemcpyDeviceToDevice, st));
     CK(qs_norm2<float>(r, k, w->nr, w->part, DS(w, S_TMP), st));
     CK(qs_cg_init(s, DS(w, S_TMP), k, st));
-    int it;
-    for (it = 1; it <= maxit; ++it) {
-        QS_TRY(opQ(lat, w, QS_F32, m0, p, t, k));
-        QS_TRY(opQ(lat, w, QS_F32, m0, t, ap, k));
-        CK(qs_norm2<float>(t, k, w->nr, w->part, s.pap, st));        // <p, Q^2 p> = |Q p|^2
-        CK(qs_cg_update(x, r, p, ap, s, k, w->nr, w->part, st));
-        CK(qs_cg_finalize(s, tol * tol, k, w->part, w->di + 70, st));
-        CK(qs_cg_pupdate(p, r, s, k, w->nr, st));
-        if (it % 16 == 0 || it == maxit) {
-            CK(cudaMemcpyAsync(w->hi + 70, w->di + 70, sizeof(int), cudaMemcpyDeviceToHost, st));
-            CK(cudaStreamSynchronize(st));
-            if (w->hi[70] == 0) break;
+    double m[QS_MAX_RHS];
+    for (int i = 0; i < k; ++i) m[i] = m0;
+    int it = 0, polls = 0, seen = 0;
+    bool done = false;
+    while (it < maxit && !done) {
+        const int *live = s.live[it & 1];
+        QS_TRY(qs_d32_run(lat, QS_D32_F32_TILED, m, p, t, k, 1, nullptr, nullptr, 0, 0, 0, nullptr, nullptr, live));
+        QS_TRY(qs_d32_run(lat, QS_D32_F32_TILED, m, t, ap, k, 1, nullptr, nullptr, 0, 0, 0, nullptr, nullptr, live));
+        CK(qs_cg_step(x, r, p, t, ap, s, it, tol * tol, k, w->nr, w->part, st));
+        ++it;
+        if (it % CG_POLL == 0 || it == maxit) {
+            const int slot = polls++ % (CG_LAG + 1);
+            CK(cudaMemcpyAsync(w->hlive + 64 * slot, s.live[it & 1], k * sizeof(int), cudaMemcpyDeviceToHost, st));
+            CK(cudaEventRecord(w->ev[slot], st));
+            if (polls - seen > CG_LAG) {
+                const int old = seen++ % (CG_LAG + 1);
+                CK(cudaEventSynchronize(w->ev[old]));
+                done = true;
+                for (int i = 0; i < k; ++i) done = done && !w->hlive[64 * old + i];
+            }
         }
     }
+    w->f32_count += 2 * (int64_t)k * it;
     w->cg_count += it;
     *iters = it;
     return QS_OK;
