@@ -48,9 +48,13 @@ cudaError_t qs_map_scalars(const double *in, double *out, int k, int mode, cudaS
 // C* partner map P v = C T gamma_5 v^* of k FP64 or FP32 vectors (partner.cu); in != out
 cudaError_t qs_partner(const double *in, double *out, const Geom &g, int k, int tiled, cudaStream_t st);
 cudaError_t qs_partner32(const float *in, float *out, const Geom &g, int k, cudaStream_t st);
-// single-CTA dense kernels (k <= 64)
+// dense kernels (k <= 64), one block per matrix
 cudaError_t qs_chol_rinv(const double2 *G, int k, double2 *Rinv, int *info, cudaStream_t st);
-cudaError_t qs_herm_eig(const double2 *H, int k, double *evals, double2 *Y, int *info, cudaStream_t st);
+// eigenvalues of H0 and eigenpairs H = Y diag(evals) Y^H, both ordered by |eigenvalue|, k even;
+// scratch: QS_EIG_SCRATCH(k) doubles, 16-byte aligned (the rotations of at most 40 sweeps)
+#define QS_EIG_SCRATCH(k) (64 + (size_t)40 * ((k) - 1) * ((k) / 2) * 4)
+cudaError_t qs_herm_eig2(const double2 *H0, double *ev0, int *info0, const double2 *H, double *evals, double2 *Y, int *info,
+                         int k, double *scratch, cudaStream_t st);
 
 // CG helpers (FP32 vectors, per-rhs scalars on device, two slots: see qs_cg_step)
 struct CgScalars {
