@@ -98,29 +98,46 @@ __global__ void __launch_bounds__(256) resid_part(const R *__restrict__ a, const
 }
 
 // Gram partials G[i][j] = sum_e conj(A_i[e]) B_j[e] (i < ka, j < kb <= 64).  A block
-// stages a chunk of GE elements of all ka + kb vectors in shared memory, element-major
+// stages a chunk of GE elements of all vectors in shared memory, element-major
 // ([e][vector], row padded by one complex to spread the banks); each thread owns a 4 x 4
 // tile of (i, j) and a residue class of the chunk's elements, so every staged value it
 // reads feeds four complex multiply-adds.  The element classes of a tile are summed in
 // shared memory at the end, in a fixed order.  LOWP: values rounded to FP32, products
-// and the sum over one chunk in FP32, chunk sums added in FP64.
+// and the sum over one chunk in FP32 (packed, two per instruction), chunk sums in FP64.
+// herm: G is known to be Hermitian (A = B, or B = Q A with Q Hermitian): only the tiles of the
+// upper triangle are computed, and same = 1 stages the vectors of A = B once.  FP64 products
+// are bound by the FP64 pipe (12^3 x 24, 16 vectors: 1.85 -> 1.38 ms with 10 of 16 tiles), FP32
+// ones by issue and by the block's own reduction (8^3 x 12, 32 vectors: 134 -> 87 us with 36 of 64
+// tiles, two blocks per SM instead of four and one conversion per total).
 #define GE 64
+__device__ __forceinline__ float2 pk_fma(float a, float2 b, float2 c) { return __ffma2_rn(make_float2(a, a), b, c); }
+
 template <bool LOWP, typename TIn = double2>
 __global__ void __launch_bounds__(256, LOWP ? 2 : 1) gram_tile_kernel(const TIn *__restrict__ A_, int ka,
                                                            const TIn *__restrict__ B_, int kb, int64_t nc,
-                                                           double *part)
+                                                           double *part, int herm, int same)
 {
     typedef typename std::conditional<LOWP, float2, double2>::type V2;
     typedef typename std::conditional<LOWP, float, double>::type T;
     extern __shared__ __align__(16) unsigned char gsm_raw[];
     V2 *sv = reinterpret_cast<V2 *>(gsm_raw);
-    const int kk = ka + kb, row = kk + 1;            // padded row of one element
-    const int ti_n = (ka + 3) / 4, tj_n = (kb + 3) / 4, ntile = ti_n * tj_n;
+    const int kk = same ? ka : ka + kb, row = kk + 1;   // padded row of one element
+    const int boff = same ? 0 : ka;
+    const int ti_n = (ka + 3) / 4, tj_n = (kb + 3) / 4;
+    const int ntile = herm ? ti_n * (ti_n + 1) / 2 : ti_n * tj_n;
     const int eg_n = 256 / ntile;                     // element classes (>= 1)
     const int t = threadIdx.x;
     const int tile = t % ntile, eg = t / ntile;
     const bool active = eg < eg_n;
-    const int i0 = 4 * (tile / tj_n), j0 = 4 * (tile % tj_n);
+    int ti, tj;   // herm: tiles row by row of the upper triangle
+    auto place = [&](int q, int &i, int &j) {
+        if (!herm) { i = q / tj_n; j = q % tj_n; return; }
+        i = 0;
+        while (q >= ti_n - i) { q -= ti_n - i; ++i; }
+        j = i + q;
+    };
+    place(tile, ti, tj);
+    const int i0 = 4 * ti, j0 = 4 * tj;
     // running totals: FP64 (FP64 products), or an FP32 (hi, lo) pair per real sum kept
     // exact to ~2^-48 by Knuth's two-sum (FP32 products: GB300's FP64 pipe is too slow
     // for a per-chunk FP64 add)
@@ -164,33 +181,34 @@ __global__ void __launch_bounds__(256, LOWP ? 2 : 1) gram_tile_kernel(const TIn 
         __syncthreads();
         if (!active) continue;
         if constexpr (LOWP) {
-            // FP32 sums over the chunk, added to the (hi, lo) totals once per chunk
-            float cr[4][4], ci[4][4];
+            // FP32 sums over the chunk, added to the (hi, lo) totals once per chunk:
+            // conj(x) y = x.re (y.re, y.im) + x.im (y.im, -y.re)
+            float2 c[4][4];
 #pragma unroll
             for (int a = 0; a < 4; ++a)
 #pragma unroll
-                for (int b = 0; b < 4; ++b) cr[a][b] = ci[a][b] = 0.f;
+                for (int b = 0; b < 4; ++b) c[a][b] = make_float2(0.f, 0.f);
             for (int e = eg; e < GE; e += eg_n) {
                 const V2 *r = sv + e * row;
-                V2 x[4], y[4];
+                V2 x[4], y[4], z[4];
 #pragma unroll
                 for (int a = 0; a < 4; ++a) x[a] = (i0 + a < ka) ? r[i0 + a] : V2{0.f, 0.f};
 #pragma unroll
-                for (int b = 0; b < 4; ++b) y[b] = (j0 + b < kb) ? r[ka + j0 + b] : V2{0.f, 0.f};
+                for (int b = 0; b < 4; ++b) {
+                    y[b] = (j0 + b < kb) ? r[boff + j0 + b] : V2{0.f, 0.f};
+                    z[b] = make_float2(y[b].y, -y[b].x);
+                }
 #pragma unroll
                 for (int a = 0; a < 4; ++a)
 #pragma unroll
-                    for (int b = 0; b < 4; ++b) {   // conj(x) y
-                        cr[a][b] = fmaf(x[a].x, y[b].x, fmaf(x[a].y, y[b].y, cr[a][b]));
-                        ci[a][b] = fmaf(x[a].x, y[b].y, fmaf(-x[a].y, y[b].x, ci[a][b]));
-                    }
+                    for (int b = 0; b < 4; ++b) c[a][b] = pk_fma(x[a].y, z[b], pk_fma(x[a].x, y[b], c[a][b]));
             }
 #pragma unroll
             for (int a = 0; a < 4; ++a)
 #pragma unroll
                 for (int b = 0; b < 4; ++b) {
-                    two_sum_acc(acc[a][b][0], accl[a][b][0], cr[a][b]);
-                    two_sum_acc(acc[a][b][1], accl[a][b][1], ci[a][b]);
+                    two_sum_acc(acc[a][b][0], accl[a][b][0], c[a][b].x);
+                    two_sum_acc(acc[a][b][1], accl[a][b][1], c[a][b].y);
                 }
         } else {
             for (int e = eg; e < GE; e += eg_n) {
@@ -199,7 +217,7 @@ __global__ void __launch_bounds__(256, LOWP ? 2 : 1) gram_tile_kernel(const TIn 
 #pragma unroll
                 for (int a = 0; a < 4; ++a) x[a] = (i0 + a < ka) ? r[i0 + a] : V2{0.0, 0.0};
 #pragma unroll
-                for (int b = 0; b < 4; ++b) y[b] = (j0 + b < kb) ? r[ka + j0 + b] : V2{0.0, 0.0};
+                for (int b = 0; b < 4; ++b) y[b] = (j0 + b < kb) ? r[boff + j0 + b] : V2{0.0, 0.0};
 #pragma unroll
                 for (int a = 0; a < 4; ++a)
 #pragma unroll
@@ -210,44 +228,80 @@ __global__ void __launch_bounds__(256, LOWP ? 2 : 1) gram_tile_kernel(const TIn 
             }
         }
     }
-    // sum the element classes of each tile (fixed order), reusing the staging buffer
+    // sum the element classes of each tile (fixed order), reusing the staging buffer; FP32 sums
+    // stay two-sum pairs until the block's total, since each conversion to FP64 costs what an
+    // FP64 addition does
+    typedef typename std::conditional<LOWP, float2, double>::type S;
     __syncthreads();
-    double *red = reinterpret_cast<double *>(gsm_raw);   // [ntile][32] partial of class 0 ...
+    S *red = reinterpret_cast<S *>(gsm_raw);   // [ntile][32]
     for (int c = 0; c < eg_n; ++c) {
         if (active && eg == c) {
 #pragma unroll
             for (int a = 0; a < 4; ++a)
 #pragma unroll
-                for (int b = 0; b < 4; ++b) {
-                    double *d = red + tile * 32 + (a * 4 + b) * 2;
-                    const double v0 = (double)acc[a][b][0] + (double)accl[a][b][0];
-                    const double v1 = (double)acc[a][b][1] + (double)accl[a][b][1];
-                    if (c == 0) { d[0] = v0; d[1] = v1; }
-                    else { d[0] += v0; d[1] += v1; }
-                }
+                for (int b = 0; b < 4; ++b)
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        S &d = red[tile * 32 + (a * 4 + b) * 2 + h];
+                        if constexpr (LOWP) {
+                            if (c == 0) {
+                                d = make_float2(acc[a][b][h], accl[a][b][h]);
+                            } else {
+                                two_sum_acc(d.x, d.y, acc[a][b][h]);
+                                d.y += accl[a][b][h];
+                            }
+                        } else {
+                            d = c == 0 ? acc[a][b][h] : d + acc[a][b][h];
+                        }
+                    }
         }
         __syncthreads();
     }
-    for (int q = t; q < ntile * 16; q += 256) {
-        const int tl = q / 16, ab = q % 16, a = ab / 4, b = ab % 4;
-        const int i = 4 * (tl / tj_n) + a, j = 4 * (tl % tj_n) + b;
+    double *out = part + (int64_t)blockIdx.x * 2 * ka * kb;
+    for (int q = t; q < ntile * 32; q += 256) {
+        const int tl = q / 32, ab = (q % 32) / 2, a = ab / 4, b = ab % 4;
+        int pi, pj;
+        place(tl, pi, pj);
+        const int i = 4 * pi + a, j = 4 * pj + b;
         if (i < ka && j < kb) {
-            const int pq = i * kb + j;
-            part[((int64_t)2 * pq) * gridDim.x + blockIdx.x] = red[tl * 32 + ab * 2];
-            part[((int64_t)2 * pq + 1) * gridDim.x + blockIdx.x] = red[tl * 32 + ab * 2 + 1];
+            if constexpr (LOWP) out[2 * (i * kb + j) + (q & 1)] = (double)red[q].x + (double)red[q].y;
+            else out[2 * (i * kb + j) + (q & 1)] = red[q];
         }
     }
+}
+
+// G from the partials [nb][2 ka kb]: 32 consecutive reals per block, 8 warps over the partials
+// (fixed order); herm: entries below the computed tiles are the conjugates of those above
+__global__ void __launch_bounds__(256) gram_sum_kernel(const double *__restrict__ part, int nb, int n, int kb, int herm, double *G)
+{
+    __shared__ double sh[8][32];
+    const int l = threadIdx.x & 31, w = threadIdx.x >> 5, q = blockIdx.x * 32 + l;
+    const int i = q / 2 / kb, j = q / 2 % kb;
+    const bool on = q < n && !(herm && i / 4 > j / 4);
+    double s = 0;
+    if (on) {
+#pragma unroll 4
+        for (int b = w; b < nb; b += 8) s += part[(int64_t)b * n + q];
+    }
+    sh[w][l] = s;
+    __syncthreads();
+    if (w != 0 || !on) return;
+    for (int v = 1; v < 8; ++v) s += sh[v][l];
+    G[q] = s;
+    if (herm && i / 4 < j / 4) G[2 * (j * kb + i) + (q & 1)] = (q & 1) ? -s : s;
 }
 
 // V_j = sum_i W_i C[i][j] (j < kc): each thread computes RE elements for a block of
 // up to RJ output vectors, the coefficients read from shared memory (the same word for
 // all threads of a warp); each W value it loads feeds RJ multiply-adds.  LOWP: values and
-// coefficients rounded to FP32, the sums in FP32.
+// coefficients rounded to FP32, the sums in FP32.  upper: C is upper triangular (the inverse
+// Cholesky factor), so a pass of RJ columns needs the first j0 + RJ vectors only; FP64 rotations
+// are bound by the FP64 pipe (8^3 x 12, 32 vectors: 1.02 ms whole, 0.64 ms upper).
 #define RE 2
 template <bool LOWP, typename TIn = double2, typename TOut = double2>
 __global__ void __launch_bounds__(256, 2) rotate_tile_kernel(const TIn *__restrict__ W, int ka,
                                                              const double2 *__restrict__ C, int kc, int64_t nc,
-                                                             TOut *__restrict__ V)
+                                                             TOut *__restrict__ V, int upper)
 {
     typedef typename std::conditional<LOWP, float2, double2>::type V2;
     typedef typename std::conditional<LOWP, float, double>::type T;
@@ -269,7 +323,8 @@ __global__ void __launch_bounds__(256, 2) rotate_tile_kernel(const TIn *__restri
             for (int u = 0; u < RE; ++u)
 #pragma unroll
                 for (int jj = 0; jj < RJ; ++jj) ar[u][jj] = ai[u][jj] = (T)0;
-            for (int i0 = 0; i0 < ka; i0 += 4) {
+            const int itop = upper && j0 + RJ < ka ? j0 + RJ : ka;   // C[i][j] = 0 for i > j
+            for (int i0 = 0; i0 < itop; i0 += 4) {
                 // four input vectors' values loaded together (independent loads in flight)
                 T wr[4][RE], wi[4][RE];
 #pragma unroll
@@ -527,31 +582,39 @@ template cudaError_t qs_resid2<double>(const double *, const double *, const dou
 template cudaError_t qs_resid2<float>(const float *, const float *, const double *, int, int64_t, double *, double *,
                                       cudaStream_t);
 
-cudaError_t qs_gram(const double *A, int ka, const double *B, int kb, int64_t nr, double *part,
-                    double2 *G, cudaStream_t st, int lowp)
+template <bool LOWP, typename TIn>
+static cudaError_t gram_launch(const TIn *A, int ka, const TIn *B, int kb, int64_t nc, double *part, double2 *G, int herm,
+                               cudaStream_t st)
 {
     if (ka < 1 || kb < 1 || ka > 64 || kb > 64) return cudaErrorInvalidValue;
-    int64_t nc = nr / 2;
-    const int row = ka + kb + 1;
-    const size_t stage = (size_t)GE * row * (lowp ? sizeof(float2) : sizeof(double2));
-    const size_t red = (size_t)((ka + 3) / 4) * ((kb + 3) / 4) * 32 * sizeof(double);
+    const int same = A == B && ka == kb;
+    herm = ka == kb && (herm || same);
+    const int tn = (ka + 3) / 4, ntile = herm ? tn * (tn + 1) / 2 : tn * ((kb + 3) / 4);
+    const size_t stage = (size_t)GE * ((same ? ka : ka + kb) + 1) * (LOWP ? sizeof(float2) : sizeof(double2));
+    const size_t red = (size_t)ntile * 32 * sizeof(double);
     const size_t sm = stage > red ? stage : red;
     static std::once_flag attr;
     std::call_once(attr, [] {
-        cudaFuncSetAttribute(gram_tile_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024);
-        cudaFuncSetAttribute(gram_tile_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024);
+        cudaFuncSetAttribute(gram_tile_kernel<LOWP, TIn>, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024);
     });
-    int64_t nch = (nc + GE - 1) / GE;
-    int nb = (int)(nch < QS_RED_BLOCKS ? nch : QS_RED_BLOCKS);
-    if (lowp) gram_tile_kernel<true><<<nb, 256, sm, st>>>((const double2 *)A, ka, (const double2 *)B, kb, nc, part);
-    else gram_tile_kernel<false><<<nb, 256, sm, st>>>((const double2 *)A, ka, (const double2 *)B, kb, nc, part);
-    finalize_sum<<<2 * ka * kb, 256, 0, st>>>(part, nb, 1, reinterpret_cast<double *>(G));
+    const int64_t nch = (nc + GE - 1) / GE;
+    const int nb = (int)(nch < QS_RED_BLOCKS / 2 ? nch : QS_RED_BLOCKS / 2), n = 2 * ka * kb;   // two blocks per SM
+    gram_tile_kernel<LOWP, TIn><<<nb, 256, sm, st>>>(A, ka, B, kb, nc, part, herm, same);
+    gram_sum_kernel<<<(n + 31) / 32, 256, 0, st>>>(part, nb, n, kb, herm, reinterpret_cast<double *>(G));
     qs_note_launches(2);
     return cudaGetLastError();
 }
 
+cudaError_t qs_gram(const double *A, int ka, const double *B, int kb, int64_t nr, double *part,
+                    double2 *G, cudaStream_t st, int lowp, int herm)
+{
+    const double2 *a = (const double2 *)A, *b = (const double2 *)B;
+    return lowp ? gram_launch<true, double2>(a, ka, b, kb, nr / 2, part, G, herm, st)
+                : gram_launch<false, double2>(a, ka, b, kb, nr / 2, part, G, herm, st);
+}
+
 cudaError_t qs_rotate(const double *W, int ka, const double2 *C, int kc, int64_t nr, double *V, cudaStream_t st,
-                      int lowp)
+                      int lowp, int upper)
 {
     if (ka < 1 || kc < 1 || ka > 64 || kc > 64) return cudaErrorInvalidValue;
     int64_t nc = nr / 2;
@@ -563,35 +626,21 @@ cudaError_t qs_rotate(const double *W, int ka, const double2 *C, int kc, int64_t
     });
     int64_t blocks = (nc + 256 * RE - 1) / (256 * RE);
     int nb = (int)(blocks < 4 * 152 ? blocks : 4 * 152);
-    if (lowp) rotate_tile_kernel<true><<<nb, 256, sm, st>>>((const double2 *)W, ka, C, kc, nc, (double2 *)V);
-    else rotate_tile_kernel<false><<<nb, 256, sm, st>>>((const double2 *)W, ka, C, kc, nc, (double2 *)V);
+    if (lowp) rotate_tile_kernel<true><<<nb, 256, sm, st>>>((const double2 *)W, ka, C, kc, nc, (double2 *)V, upper);
+    else rotate_tile_kernel<false><<<nb, 256, sm, st>>>((const double2 *)W, ka, C, kc, nc, (double2 *)V, upper);
     qs_note_launches(1);
     return cudaGetLastError();
 }
 
 // the same contractions on FP32 blocks (products and per-chunk sums in FP32)
 cudaError_t qs_gram32(const float *A, int ka, const float *B, int kb, int64_t nr, double *part, double2 *G,
-                      cudaStream_t st)
+                      cudaStream_t st, int herm)
 {
-    if (ka < 1 || kb < 1 || ka > 64 || kb > 64) return cudaErrorInvalidValue;
-    int64_t nc = nr / 2;
-    const int row = ka + kb + 1;
-    const size_t stage = (size_t)GE * row * sizeof(float2);
-    const size_t red = (size_t)((ka + 3) / 4) * ((kb + 3) / 4) * 32 * sizeof(double);
-    const size_t sm = stage > red ? stage : red;
-    static std::once_flag attr;
-    std::call_once(attr, [] {
-        cudaFuncSetAttribute(gram_tile_kernel<true, float2>, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024);
-    });
-    int64_t nch = (nc + GE - 1) / GE;
-    int nb = (int)(nch < QS_RED_BLOCKS ? nch : QS_RED_BLOCKS);
-    gram_tile_kernel<true, float2><<<nb, 256, sm, st>>>((const float2 *)A, ka, (const float2 *)B, kb, nc, part);
-    finalize_sum<<<2 * ka * kb, 256, 0, st>>>(part, nb, 1, reinterpret_cast<double *>(G));
-    qs_note_launches(2);
-    return cudaGetLastError();
+    return gram_launch<true, float2>((const float2 *)A, ka, (const float2 *)B, kb, nr / 2, part, G, herm, st);
 }
 
-cudaError_t qs_rotate32(const float *W, int ka, const double2 *C, int kc, int64_t nr, float *V, cudaStream_t st)
+cudaError_t qs_rotate32(const float *W, int ka, const double2 *C, int kc, int64_t nr, float *V, cudaStream_t st,
+                        int upper)
 {
     if (ka < 1 || kc < 1 || ka > 64 || kc > 64) return cudaErrorInvalidValue;
     int64_t nc = nr / 2;
@@ -603,7 +652,7 @@ cudaError_t qs_rotate32(const float *W, int ka, const double2 *C, int kc, int64_
     });
     int64_t blocks = (nc + 256 * RE - 1) / (256 * RE);
     int nb = (int)(blocks < 4 * 152 ? blocks : 4 * 152);
-    rotate_tile_kernel<true, float2, float2><<<nb, 256, sm, st>>>((const float2 *)W, ka, C, kc, nc, (float2 *)V);
+    rotate_tile_kernel<true, float2, float2><<<nb, 256, sm, st>>>((const float2 *)W, ka, C, kc, nc, (float2 *)V, upper);
     qs_note_launches(1);
     return cudaGetLastError();
 }

@@ -19,8 +19,8 @@ __device__ __forceinline__ double2 cscale(double s, double2 a) { return make_dou
 // numerically positive definite.  256 threads on one SM, whose FP64 pipe (1.6 lanes a clock) and
 // the k dependent steps bound it: the factor is right-looking (each step's rank-1 update is spread
 // over all threads), and column j of the inverse is -X R_j / r_jj with 8 threads per row of
-// the finished part X.  k = 32: 312 us with one thread per column and the inverse in global
-// memory.
+// the finished part X.  k = 32: 95 us (312 us with one thread per column and the inverse in
+// global memory).
 __global__ void __launch_bounds__(256) chol_rinv_kernel(const double2 *G, int k, double2 *Rinv, int *info)
 {
     extern __shared__ double2 sm[];
@@ -93,9 +93,11 @@ __global__ void __launch_bounds__(256) chol_rinv_kernel(const double2 *G, int k,
 // in closed form.  The rotations are logged, and a second kernel applies them to the rows of
 // the identity, one warp per row on its own SM, which gives the eigenvectors.  k must be even.
 //
-// What bounds it: the FP64 pipe of the one SM a matrix lives on.  Full-matrix column and row passes
-// and the eigenvectors in the same block cost 36 k^2 / 2 lane instructions a round (k = 32: 1.5 ms a
-// matrix); this costs 48 (k / 2)^2 / 2.  Up to two matrices run in one launch.
+// What bounds it: the FP64 pipe of the one SM a matrix lives on, and the chain of square roots and
+// divisions of a rotation.  Full-matrix column and row passes and the eigenvectors in the same
+// block cost 36 k^2 / 2 lane instructions a round (k = 32: 1.5 ms a matrix); this costs
+// 48 (k / 2)^2 / 2 (0.95 ms for both matrices of a Rayleigh-Ritz, which share a launch, and 0.12 ms
+// for the vectors).
 __device__ __forceinline__ int rr_player(int j, int r, int k)
 {
     return j == 0 ? 0 : ((j - 1 + r) % (k - 1)) + 1;
@@ -164,15 +166,15 @@ __global__ void __launch_bounds__(256) jacobi_kernel(JacobiJob j0, JacobiJob j1,
                 s_p[t] = p;
                 s_q[t] = q;
                 const double2 h = H[p * k + q];
-                const double c = sqrt(h.x * h.x + h.y * h.y);
+                const double h2 = fma(h.x, h.x, h.y * h.y), ic = rsqrt(h2), c = h2 > 0 ? h2 * ic : 0.0;
                 const double a = H[p * k + p].x, b = H[q * k + q].x;
                 double cs = 0.0, sn = 0.0;
                 double2 u = make_double2(1, 0);
-                if (!(c <= 1e-300 || c <= 1e-18 * (fabs(a) + fabs(b)))) {
-                    u = make_double2(h.x / c, h.y / c);
-                    const double tau = (b - a) / (2.0 * c);
-                    const double tt = (tau >= 0 ? 1.0 : -1.0) / (fabs(tau) + sqrt(1.0 + tau * tau));
-                    cs = 1.0 / sqrt(1.0 + tt * tt);
+                if (!(c <= 1e-150 || c <= 1e-18 * (fabs(a) + fabs(b)))) {
+                    u = make_double2(h.x * ic, h.y * ic);
+                    const double tau = 0.5 * (b - a) * ic;
+                    const double tt = (tau >= 0 ? 1.0 : -1.0) / (fabs(tau) + sqrt(fma(tau, tau, 1.0)));
+                    cs = rsqrt(fma(tt, tt, 1.0));
                     sn = tt * cs;
                     H[p * k + p] = make_double2(a - tt * c, 0.0);
                     H[q * k + q] = make_double2(b + tt * c, 0.0);

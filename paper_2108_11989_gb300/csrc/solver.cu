@@ -182,7 +182,7 @@ static int orthonormalize(qs_lattice *lat, Workspace *w, double *X, double *tmp,
         double *src = pass == 0 ? X : tmp, *dst = pass == 0 ? tmp : X;
         CK(qs_gram(src, k, src, k, w->nr, w->part, w->G, st, glow));
         CK(qs_chol_rinv(w->G, k, w->Rinv, w->di + 64 + pass, st));
-        CK(qs_rotate(src, k, w->Rinv, k, w->nr, dst, st, rlow));
+        CK(qs_rotate(src, k, w->Rinv, k, w->nr, dst, st, rlow, 1));
     }
     return QS_OK;
 }
@@ -242,7 +242,7 @@ static int rayleigh_ritz(qs_lattice *lat, Workspace *w, double m0, int k, Ritz *
     glow = glow || rlow;
     // the Q^2 Ritz values only place the filter interval: FP32 products always
     CK(qs_gram(w->blk64[1], k, w->blk64[1], k, w->nr, w->part, w->G, st, 1));
-    CK(qs_gram(w->blk64[0], k, w->blk64[1], k, w->nr, w->part, w->Hm, st, glow));
+    CK(qs_gram(w->blk64[0], k, w->blk64[1], k, w->nr, w->part, w->Hm, st, glow, 1));   // Q is Hermitian
     CK(qs_herm_eig2(w->G, DS(w, S_RN), w->di + 66, w->Hm, DS(w, S_THETA), w->Ym, w->di + 67, k, w->part, st));
     CK(qs_rotate(w->blk64[0], k, w->Ym, k, w->nr, w->blk64[2], st, rlow));
     CK(qs_rotate(w->blk64[1], k, w->Ym, k, w->nr, w->blk64[3], st, rlow));
@@ -294,7 +294,7 @@ static int orthonormalize32(qs_lattice *lat, Workspace *w, int k)
     for (int pass = 0; pass < 2; ++pass) {
         CK(qs_gram32(V32(w), k, V32(w), k, w->nr, w->part, w->G, st));
         CK(qs_chol_rinv(w->G, k, w->Rinv, w->di + 64 + pass, st));
-        CK(qs_rotate32(V32(w), k, w->Rinv, k, w->nr, T32(w), st));
+        CK(qs_rotate32(V32(w), k, w->Rinv, k, w->nr, T32(w), st, 1));
         std::swap(w->iv, w->it3);
     }
     return QS_OK;
@@ -306,7 +306,7 @@ static int rayleigh_ritz32(qs_lattice *lat, Workspace *w, double m0, int k, Ritz
     cudaStream_t st = lat->stream;
     QS_TRY(opQ(lat, w, QS_F32, m0, V32(w), QV32(w), k));
     CK(qs_gram32(QV32(w), k, QV32(w), k, w->nr, w->part, w->G, st));
-    CK(qs_gram32(V32(w), k, QV32(w), k, w->nr, w->part, w->Hm, st));
+    CK(qs_gram32(V32(w), k, QV32(w), k, w->nr, w->part, w->Hm, st, 1));
     CK(qs_herm_eig2(w->G, DS(w, S_RN), w->di + 66, w->Hm, DS(w, S_THETA), w->Ym, w->di + 67, k, w->part, st));
     CK(qs_rotate32(V32(w), k, w->Ym, k, w->nr, T32(w), st));
     std::swap(w->iv, w->it3);
