@@ -57,11 +57,9 @@ __device__ __forceinline__ double2 diff(double2 a, double t, double2 b) { return
 // blocks per vector whatever its length, an 8^3 x 12 CG update of 16 vectors was 9728 blocks of
 // two reals per thread and took 69 us instead of 15.  FP32 sums are kept as a two-sum pair.
 template <typename R>
-__global__ void __launch_bounds__(256) norm2_part(const R *__restrict__ v, int64_t nr, double *part,
-                                                  const int *__restrict__ live = nullptr)
+__global__ void __launch_bounds__(256) norm2_part(const R *__restrict__ v, int64_t nr, double *part)
 {
     typedef typename Vec16<R>::T T;
-    if (live && !live[blockIdx.y]) return;
     const int64_t n = nr * (int64_t)sizeof(R) / 16;
     const T *x = reinterpret_cast<const T *>(v) + (int64_t)blockIdx.y * n;
     R acc = 0, lo = 0;
@@ -463,69 +461,50 @@ __global__ void map_scalars_kernel(const double *in, double *out, int k, int mod
 }
 
 // ---- CG (FP32 vectors, FP64 scalars) ----------------------------------------
-// An iteration is the operator's launches, the sums of |Q p|^2 and the two kernels below, whose
-// blocks sum the partial sums they need themselves in a fixed order, so that no launch is spent
-// on scalars.  The scalars live in two slots: an iteration reads slot o and writes 1 - o.
-// Vectors that have converged are skipped.
-__device__ double all_parts(const double *part, int nb)
+// An iteration is t = Q p with the shares of |t|^2 (= <p, Q^2 p>), alpha, r -= alpha Q t with the
+// shares of |r|^2, beta, and the update of x and p: five launches, of which only the last streams
+// vectors of its own (Q^2 p is never written, and neither it nor Q p is read for a sum).  Vectors
+// that have converged are skipped.  12^3 x 24, 8 vectors, per iteration: 159 us, 192 with separate
+// passes for |Q p|^2 and r.
+// alpha = |r|^2 / |Q p|^2, one block per vector; 0 for vectors that are done
+__global__ void __launch_bounds__(256) cg_alpha_kernel(CgScalars s, const double *part, int nb)
 {
-    __shared__ double d;
+    const int q = blockIdx.x;
     double acc = 0;
-    for (int i = threadIdx.x; i < nb; i += blockDim.x) acc += part[i];
+    if (s.live[q])
+        for (int i = threadIdx.x; i < nb; i += 256) acc += part[(int64_t)q * nb + i];
     acc = block_sum(acc);
-    if (threadIdx.x == 0) d = acc;
-    __syncthreads();
-    return d;
+    if (threadIdx.x == 0) s.alpha[q] = s.live[q] && acc > 0 ? (float)(s.rr[q] / acc) : 0.f;
 }
 
-// r -= alpha Q^2 p, alpha = |r|^2 / |Q p|^2; rpart = shares of |r|^2
-__global__ void __launch_bounds__(256) cg_r_kernel(float4 *__restrict__ r, const float4 *__restrict__ ap, CgScalars s, int o,
-                                                   int64_t n, const double *__restrict__ ppart, double *__restrict__ rpart)
+// beta = |r|^2 / |r_old|^2; the vector lives on while |r|^2 > tol2 |r_0|^2
+__global__ void __launch_bounds__(256) cg_beta_kernel(CgScalars s, const double *part, int nb, double tol2)
 {
-    const int q = blockIdx.y;
-    if (!s.live[o][q]) return;
-    const double pap = all_parts(ppart + (int64_t)q * gridDim.x, gridDim.x);
-    const float a = pap > 0 ? (float)(s.rr[o][q] / pap) : 0.f;
-    float4 *rq = r + q * n;
-    const float4 *aq = ap + q * n;
-    float acc = 0, lo = 0;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const float4 v = diff(rq[i], a, aq[i]);
-        rq[i] = v;
-        two_sum_acc(acc, lo, sum_sq(v));
-    }
-    const double sm = block_sum((double)acc + (double)lo);
-    if (threadIdx.x == 0) rpart[q * gridDim.x + blockIdx.x] = sm;
+    const int q = blockIdx.x;
+    if (!s.live[q]) return;
+    double acc = 0;
+    for (int i = threadIdx.x; i < nb; i += 256) acc += part[(int64_t)q * nb + i];
+    acc = block_sum(acc);
+    if (threadIdx.x != 0) return;
+    s.beta[q] = s.rr[q] > 0 ? (float)(acc / s.rr[q]) : 0.f;
+    s.rr[q] = acc;
+    s.live[q] = acc > tol2 * s.rr0[q] && isfinite(acc);
 }
 
-// x += alpha p, p = r + beta p, beta = |r|^2 / |r_old|^2; the vector lives on while
-// |r|^2 > tol2 |r_0|^2
+// x += alpha p, p = r + beta p
 __global__ void __launch_bounds__(256) cg_xp_kernel(float4 *__restrict__ x, float4 *__restrict__ p,
-                                                    const float4 *__restrict__ r, CgScalars s, int o, int64_t n,
-                                                    const double *__restrict__ ppart, const double *__restrict__ rpart,
-                                                    double tol2)
+                                                    const float4 *__restrict__ r, CgScalars s, int64_t n)
 {
     const int q = blockIdx.y;
-    const bool first = blockIdx.x == 0 && threadIdx.x == 0;
-    if (!s.live[o][q]) {
-        if (first) s.live[1 - o][q] = 0;
-        return;
-    }
-    const double rr = s.rr[o][q];
-    const double pap = all_parts(ppart + (int64_t)q * gridDim.x, gridDim.x);
-    __syncthreads();
-    const double rn = all_parts(rpart + (int64_t)q * gridDim.x, gridDim.x);
-    const float a = pap > 0 ? (float)(rr / pap) : 0.f, b = rr > 0 ? (float)(rn / rr) : 0.f;
-    if (first) {
-        s.rr[1 - o][q] = rn;
-        s.live[1 - o][q] = rn > tol2 * s.rr0[q] && isfinite(rn);
-    }
+    const float a = s.alpha[q], b = s.beta[q];
+    if (a == 0.f) return;
+    const bool live = s.live[q];
     float4 *xq = x + q * n, *pq = p + q * n;
     const float4 *rq = r + q * n;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         const float4 v = pq[i];
         xq[i] = diff(xq[i], -a, v);
-        pq[i] = diff(rq[i], -b, v);
+        if (live) pq[i] = diff(rq[i], -b, v);
     }
 }
 
@@ -533,9 +512,9 @@ __global__ void cg_init_kernel(CgScalars s, const double *rr, int k)
 {
     int q = threadIdx.x;
     if (q >= k) return;
-    s.rr[0][q] = rr[q];
+    s.rr[q] = rr[q];
     s.rr0[q] = rr[q];
-    s.live[0][q] = rr[q] > 0;
+    s.live[q] = rr[q] > 0;
 }
 
 // blocks per vector of the reductions: two to eight per SM over the k vectors
@@ -735,17 +714,19 @@ cudaError_t qs_map_scalars(const double *in, double *out, int k, int mode, cudaS
     return cudaGetLastError();
 }
 
-// t = Q p, ap = Q t are computed; the rest of iteration `it`
-cudaError_t qs_cg_step(float *x, float *r, float *p, const float *t, const float *ap, const CgScalars &s, int it, double tol2,
-                       int k, int64_t nr, double *part, cudaStream_t st)
+cudaError_t qs_cg_alpha(const CgScalars &s, int k, const double *part, int nb, cudaStream_t st)
 {
-    const int nb = red_blocks(nr, k), o = it & 1;
-    const dim3 g(nb, k);
-    double *rpart = part + (size_t)QS_RED_BLOCKS * 64;
-    norm2_part<float><<<g, 256, 0, st>>>(t, nr, part, s.live[o]);   // <p, Q^2 p> = |Q p|^2
-    cg_r_kernel<<<g, 256, 0, st>>>((float4 *)r, (const float4 *)ap, s, o, nr / 4, part, rpart);
-    cg_xp_kernel<<<g, 256, 0, st>>>((float4 *)x, (float4 *)p, (const float4 *)r, s, o, nr / 4, part, rpart, tol2);
-    qs_note_launches(3);
+    cg_alpha_kernel<<<k, 256, 0, st>>>(s, part, nb);
+    qs_note_launches(1);
+    return cudaGetLastError();
+}
+
+cudaError_t qs_cg_beta_xp(float *x, float *p, const float *r, const CgScalars &s, double tol2, int k, int64_t nr,
+                          const double *part, int nb, cudaStream_t st)
+{
+    cg_beta_kernel<<<k, 256, 0, st>>>(s, part, nb, tol2);
+    cg_xp_kernel<<<dim3(red_blocks(nr, k), k), 256, 0, st>>>((float4 *)x, (float4 *)p, (const float4 *)r, s, nr / 4);
+    qs_note_launches(2);
     return cudaGetLastError();
 }
 

@@ -58,13 +58,16 @@ cudaError_t qs_chol_rinv(const double2 *G, int k, double2 *Rinv, int *info, cuda
 cudaError_t qs_herm_eig2(const double2 *H0, double *ev0, int *info0, const double2 *H, double *evals, double2 *Y, int *info,
                          int k, double *scratch, cudaStream_t st);
 
-// CG helpers (FP32 vectors, per-rhs scalars on device, two slots: see qs_cg_step)
+// CG helpers (FP32 vectors, per-rhs scalars on device)
 struct CgScalars {
-    double *rr[2], *rr0;
-    int *live[2];
+    double *rr, *rr0;
+    float *alpha, *beta;
+    int *live;
 };
-cudaError_t qs_cg_step(float *x, float *r, float *p, const float *t, const float *ap, const CgScalars &s, int it, double tol2,
-                       int k, int64_t nr, double *part, cudaStream_t st);
+// part: [k][nb] shares of |Q p|^2 (alpha), of |r|^2 (beta)
+cudaError_t qs_cg_alpha(const CgScalars &s, int k, const double *part, int nb, cudaStream_t st);
+cudaError_t qs_cg_beta_xp(float *x, float *p, const float *r, const CgScalars &s, double tol2, int k, int64_t nr,
+                          const double *part, int nb, cudaStream_t st);
 cudaError_t qs_cg_init(CgScalars s, const double *rr, int k, cudaStream_t st);
 
 // Ritz values (sorted by |theta|) and residual norms of the current block

@@ -343,10 +343,10 @@ static int prec_of_storage(int storage)
 
 int qs_d32_run(qs_lattice *lat, int storage, const double *m0, const void *in, void *out, int nrhs, int gamma5,
                const void *cheb_y, const void *cheb_x, double cheb_c, double cheb_s1, double cheb_s2,
-               const float *coef_dev, const float *dm_dev, const int *live_dev)
+               const float *coef_dev, const float *dm_dev)
 {
     D32Call c;
-    c.live = live_dev;
+    memset(&c, 0, sizeof(c));
     c.coef_dev = coef_dev;
     c.dm_dev = dm_dev;
     c.g = lat->g;
@@ -359,17 +359,25 @@ int qs_d32_run(qs_lattice *lat, int storage, const double *m0, const void *in, v
     c.storage = storage;
     c.nrhs = nrhs;
     c.gamma5 = gamma5;
-    c.cheb = cheb_y != nullptr;
+    c.epi = cheb_y ? QS_EPI_CHEB : QS_EPI_PLAIN;
     c.cheb_c = cheb_c;
     c.cheb_s1 = cheb_s1;
     c.cheb_s2 = cheb_s2;
     c.m0 = m0;
-    int &tv = lat->tuned32[storage][c.cheb][nrhs];
+    return qs_d32_call(lat, c);
+}
+
+// launch of a filled-in call with the shape's autotuned variant.  NORM and RESID take the plain
+// operator's; a RESID call, whose output may be an input, never times variants itself.
+int qs_d32_call(qs_lattice *lat, const D32Call &c)
+{
+    const int storage = c.storage, nrhs = c.nrhs, cheb = c.epi == QS_EPI_CHEB;
+    int &tv = lat->tuned32[storage][cheb][nrhs];
     if (tv == 0) {
-        const std::string key = tune_key(lat, "dslash32p", storage, c.cheb, nrhs);
+        const std::string key = tune_key(lat, "dslash32p", storage, cheb, nrhs);
         int v = tune_lookup(key);
         if (v < 0 || v >= qs_d32_nvariants()) {
-            if (capturing(lat->stream)) {
+            if (capturing(lat->stream) || c.epi == QS_EPI_RESID) {
                 v = 1;   // no timing inside a capture: a fixed variant
             } else {
                 // timing writes `out` only (in, y and x are read): harmless to the caller
@@ -394,7 +402,7 @@ int qs_d32_run(qs_lattice *lat, int storage, const double *m0, const void *in, v
     // (plus y and x for the Chebyshev epilogue), and once per launch 36 link + 36 SW
     // FP32 reals (each physical link and SW block serves the site and its mirror)
     const double vs = (double)qs_d32_vec_bytes(storage, 1);
-    const double bytes = (double)lat->g.Ns * (vs * (c.cheb ? 4 : 2) * nrhs + 72.0 * 4);
+    const double bytes = (double)lat->g.Ns * (vs * (cheb ? 4 : c.epi == QS_EPI_RESID ? 3 : 2) * nrhs + 72.0 * 4);
     return prof_end(lat, ea, eb, prec_of_storage(storage), bytes);
 }
 

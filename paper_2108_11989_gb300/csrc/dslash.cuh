@@ -55,23 +55,31 @@ int qs_dslash_nvariants();
 enum { QS_D32_F32_TILED = 0, QS_D32_F32_CANON = 1, QS_D32_F16 = 2, QS_D32_BF16 = 3,
        QS_D32_F64_TILED = 4 /* conversions only */ };
 
+// epilogues (dslash32.cu); NORM and RESID in tiled FP32 storage only
+enum { QS_EPI_PLAIN = 0, QS_EPI_CHEB = 1, QS_EPI_NORM = 2, QS_EPI_RESID = 3 };
+
 struct D32Call {
     Geom g;
     const float2 *links;   // [mu][9][Vphys] FP32, times -1/2
     const float2 *clov;    // [2][18][Vphys] FP32 pairs (packed SW blocks)
     const void *in;        // nrhs vectors, vector r at in + r * qs_d32_vec_bytes(storage, Ns)
     void *out;
-    const void *y, *x;     // cheb = 1: out = s1 (Q in - c y) - s2 x
-    int storage, nrhs, gamma5, cheb;
+    const void *y, *x;     // CHEB: out = s1 (Q in - c y) - s2 x; RESID: out = y - alpha Q in
+    int storage, nrhs, gamma5, epi;
     double cheb_c, cheb_s1, cheb_s2;
     const double *m0;      // host, nrhs masses (ignored where dm_dev is set)
     const float *coef_dev; // NULL, or device (c, s1, s2) of the Chebyshev epilogue
     const float *dm_dev;   // NULL, or device 4 + m0 per right-hand side
+    const float *alpha_dev;   // RESID: device, per right-hand side
+    double *part;          // NORM, RESID: device [nrhs][qs_d32_ntile()] shares of |out|^2
     const int *live;       // NULL, or device flags: right-hand sides with 0 are skipped
 };
 int qs_d32_nvariants();
+int64_t qs_d32_ntile(const Geom &g, int nrhs);
 int64_t qs_d32_vec_bytes(int storage, int64_t Ns);
 cudaError_t qs_d32_launch(const D32Call &c, int variant, cudaStream_t st);
+// the same with the handle's autotuned variant and profiling records (capi.cu)
+int qs_d32_call(qs_lattice *lat, const D32Call &c);
 // k vectors from one tiled storage to another (QS_D32_F32_TILED, _F16, _BF16, _F64_TILED)
 cudaError_t qs_convert_tiled(int from, int to, const void *in, void *out, int64_t Ns, int k, cudaStream_t st);
 // FP64 solver-layout block of k vectors <-> 16-bit scaled storage

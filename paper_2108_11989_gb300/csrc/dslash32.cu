@@ -33,7 +33,9 @@
 //
 // Epilogue.  PLAIN: out = D in or Q in.  CHEB: one step of the scaled Chebyshev
 // recurrence of the filter, out = s1 (Q in - c y) - s2 x, with y, x in the same
-// storage (saves a separate pass over four vectors).
+// storage (saves a separate pass over four vectors).  NORM: out = Q in and each warp's share of
+// |out|^2.  RESID: out = y - alpha Q in (y may be out) and the shares of |out|^2; with these two a
+// CG iteration never writes Q^2 p and reads neither it nor Q p for its sums.
 #include "qs_internal.cuh"
 #include "dslash.cuh"
 #include "dslash64.cuh"
@@ -377,6 +379,9 @@ struct D32 {
     // are read from coef[0..2] and 4 + m0 of right-hand side r from dmdev[r]
     const float *coef, *dmdev;
     const int *live;    // NULL, or flags: right-hand sides with live[r] = 0 are skipped
+    const float *alpha; // RESID: per right-hand side
+    double *part;       // NORM, RESID: [nrhs][ntile] shares of |out|^2
+    int ntile;
 };
 
 // acc += upper and lower parts of M h for a neighbour's spinor, M = U (FW, sigma = +1),
@@ -463,14 +468,38 @@ __device__ __forceinline__ void hops(const D32 &a, const Site &c, const char *in
     }
 }
 
-template <class S, bool CHEB>
-__device__ __forceinline__ void finish_site(const D32 &a, int64_t off, int s, cf acc[12])
+// |v|^2 of 12 components
+__device__ __forceinline__ float site_norm2(const cf v[12])
+{
+    cf q = mul2(v[0], v[0]);
+#pragma unroll
+    for (int i = 1; i < 12; ++i) q = fma2(v[i], v[i], q);
+    return q.x + q.y;
+}
+
+// the warp's sum of x, kept as a two-sum pair, to *out by lane 0
+__device__ __forceinline__ void warp_share(float x, double *out)
+{
+    float lo = 0.f;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const float h2 = __shfl_xor_sync(0xffffffffu, x, o), l2 = __shfl_xor_sync(0xffffffffu, lo, o);
+        const float t = x + h2, b = t - x;
+        lo += l2 + ((x - (t - b)) + (h2 - b));
+        x = t;
+    }
+    if ((threadIdx.x & 31) == 0) *out = (double)x + (double)lo;
+}
+
+// returns |out|^2 at the site for NORM and RESID
+template <class S, int EPI>
+__device__ __forceinline__ float finish_site(const D32 &a, int64_t off, int s, int r, bool on, cf acc[12])
 {
     if (a.gamma5) {
 #pragma unroll
         for (int i = 6; i < 12; ++i) acc[i] = cneg(acc[i]);
     }
-    if (CHEB) {
+    if (EPI == QS_EPI_CHEB) {
         cf yv[12], xv[12];
         S::ld(a.y + off, s, yv);
         S::ld(a.x + off, s, xv);
@@ -481,12 +510,20 @@ __device__ __forceinline__ void finish_site(const D32 &a, int64_t off, int s, cf
         for (int i = 0; i < 12; ++i)
             acc[i] = fma2(dup(s1), fma2(dup(-cc), yv[i], acc[i]), mul2(dup(-s2), xv[i]));
     }
-    S::st(a.out + off, s, acc);
+    if (EPI == QS_EPI_RESID) {
+        const float al = a.alpha[r];
+        const cf *y = reinterpret_cast<const cf *>(a.y + off) + ((int64_t)(s >> 4) * 12) * 16 + (s & 15);   // tiled FP32
+#pragma unroll
+        for (int i = 0; i < 12; ++i) acc[i] = fma2(dup(-al), acc[i], y[i * 16]);   // no read-only load: y may be out
+    }
+    if (EPI < QS_EPI_NORM || on) S::st(a.out + off, s, acc);
+    return EPI >= QS_EPI_NORM && on ? site_norm2(acc) : 0.f;
 }
 
-// physical site p and its mirror, right-hand side r
-template <class S, bool CHEB>
-__device__ __forceinline__ void site_kernel(const D32 &a, int p, int r)
+// physical site p and its mirror, right-hand side r (one per warp); on = false: nothing is
+// stored (NORM and RESID keep whole warps for their sums)
+template <class S, int EPI>
+__device__ __forceinline__ void site_kernel(const D32 &a, int p, int r, bool on = true)
 {
     if (a.live && !a.live[r]) return;
     const int row = p / a.g.L;
@@ -515,22 +552,29 @@ __device__ __forceinline__ void site_kernel(const D32 &a, int p, int r)
     hop_begin<0>(a, c, h);
     S::fetch(in, h.n, v);
     hops<0, S>(a, c, in, h, v, acc, accm);
-    finish_site<S, CHEB>(a, off, c.s, acc);
-    finish_site<S, CHEB>(a, off, c.s + a.g.L, accm);
+    float n2 = finish_site<S, EPI>(a, off, c.s, r, on, acc);
+    n2 += finish_site<S, EPI>(a, off, c.s + a.g.L, r, on, accm);
+    if (EPI >= QS_EPI_NORM) warp_share(n2, a.part + (int64_t)r * a.ntile + p / 32);
 }
 
 // A block's NT / 32 warps are WR right-hand sides x (NT / 32 / WR) groups of 32 physical sites;
 // it computes `gpb` groups of WR right-hand sides one after the other.
-template <class S, bool CHEB, int NT, int MINB>
+template <class S, int EPI, int NT, int MINB>
 __global__ void __launch_bounds__(NT, MINB) dslash32_kernel(const __grid_constant__ D32 a, unsigned nchunk, int lwr,
                                                             int gpb)
 {
     const unsigned tile = blockIdx.x / nchunk, chunk = blockIdx.x % nchunk;
     const int w = threadIdx.x >> 5, wr = 1 << lwr;
-    const int p = (int)((tile * (NT / 32 >> lwr) + (w >> lwr)) * 32 + (threadIdx.x & 31));
-    if (p >= (int)a.g.Vphys) return;
+    int p = (int)((tile * (NT / 32 >> lwr) + (w >> lwr)) * 32 + (threadIdx.x & 31));
+    bool on = p < (int)a.g.Vphys;
+    if (EPI >= QS_EPI_NORM) {
+        if ((p & ~31) >= (int)a.g.Vphys) return;   // the whole warp
+        if (!on) p = (int)a.g.Vphys - 1;           // same warp tile as lane 0
+    } else if (!on) {
+        return;
+    }
     int r = (int)(chunk * gpb) * wr + (w & (wr - 1));
-    for (int i = 0; i < gpb && r < a.nrhs; ++i, r += wr) site_kernel<S, CHEB>(a, p, r);
+    for (int i = 0; i < gpb && r < a.nrhs; ++i, r += wr) site_kernel<S, EPI>(a, p, r, on);
 }
 
 // ---- small problems: two threads per site (dslash64.cuh in FP32) ------------------------
@@ -552,7 +596,7 @@ struct Mem32 {
 // alone, so the layouts of one problem always take the same arithmetic.
 constexpr int64_t kSplitSites = 24576;
 
-template <class S, bool CHEB>
+template <class S, int EPI>
 __global__ void __launch_bounds__(64, 10) dslash32_split_kernel(const __grid_constant__ D32 a)
 {
     const int r = (int)(blockIdx.x % (unsigned)a.nrhs);
@@ -570,7 +614,7 @@ __global__ void __launch_bounds__(64, 10) dslash32_split_kernel(const __grid_con
 #pragma unroll
         for (int i = 0; i < 3; ++i) low[i] = cneg(low[i]);
     }
-    if (CHEB) {
+    if (EPI == QS_EPI_CHEB) {
         const float cc = a.coef ? __ldg(a.coef) : a.c;
         const float s1 = a.coef ? __ldg(a.coef + 1) : a.s1;
         const float s2 = a.coef ? __ldg(a.coef + 2) : a.s2;
@@ -583,6 +627,23 @@ __global__ void __launch_bounds__(64, 10) dslash32_split_kernel(const __grid_con
 #pragma unroll
             for (int i = 0; i < 3; ++i) o[i] = fma2(dup(s1), fma2(dup(-cc), yv[i], o[i]), mul2(dup(-s2), xv[i]));
         }
+    }
+    if (EPI == QS_EPI_RESID) {
+        const float al = a.alpha[r];
+#pragma unroll
+        for (int b = 0; b < 2; ++b) {
+            const cf *y = reinterpret_cast<const cf *>(a.y + off) + ((int64_t)(ln.c.s >> 4) * 12 + 6 * b + 3 * ln.q) * 16 + (ln.c.s & 15);
+            cf *o = b ? low : up;
+#pragma unroll
+            for (int i = 0; i < 3; ++i) o[i] = fma2(dup(-al), o[i], y[i * 16]);
+        }
+    }
+    if (EPI >= QS_EPI_NORM) {
+        cf n2 = make_float2(0.f, 0.f);
+#pragma unroll
+        for (int i = 0; i < 3; ++i) n2 = fma2(up[i], up[i], fma2(low[i], low[i], n2));
+        const int tile = (s0 - (int)(threadIdx.x & 15)) >> 4;
+        if (tile < a.ntile) warp_share(on ? n2.x + n2.y : 0.f, a.part + (int64_t)r * a.ntile + tile);
     }
     float m = 0.f;
     if constexpr (S::kScaled) {
@@ -598,12 +659,11 @@ __global__ void __launch_bounds__(64, 10) dslash32_split_kernel(const __grid_con
     S::st3(a.out + off, s0, 2 + ln.q, low, m);
 }
 
-template <class S>
-cudaError_t launch_split(const D32 &a, bool cheb, cudaStream_t st)
+template <class S, int EPI>
+cudaError_t launch_split(const D32 &a, cudaStream_t st)
 {
     const unsigned nb = (unsigned)((a.g.Ns + 31) / 32) * (unsigned)a.nrhs;
-    if (cheb) dslash32_split_kernel<S, true><<<nb, 64, 0, st>>>(a);
-    else dslash32_split_kernel<S, false><<<nb, 64, 0, st>>>(a);
+    dslash32_split_kernel<S, EPI><<<nb, 64, 0, st>>>(a);
     return cudaGetLastError();
 }
 
@@ -627,7 +687,7 @@ __global__ void __launch_bounds__(128, 3) dslash32_batch_kernel(const __grid_con
         while (i + 1 < b.n && w >= b.off[i + 1]) ++i;
         const unsigned local = w - b.off[i];
         const int p = (int)(local / (unsigned)b.item[i].nrhs) * 128 + (int)threadIdx.x;
-        if (p < (int)b.item[i].g.Vphys) site_kernel<S, false>(b.item[i], p, (int)(local % (unsigned)b.item[i].nrhs));
+        if (p < (int)b.item[i].g.Vphys) site_kernel<S, QS_EPI_PLAIN>(b.item[i], p, (int)(local % (unsigned)b.item[i].nrhs));
     }
 }
 
@@ -680,14 +740,14 @@ cudaError_t convert_from(int to, const void *in, void *out, int64_t Ns, int k, c
 }
 
 // ---- launch ------------------------------------------------------------------
-template <class S, bool CHEB, int NT, int MINB>
+template <class S, int EPI, int NT, int MINB>
 cudaError_t launch(const D32 &a, int lwr, int gpb, cudaStream_t st)
 {
     const int spb = NT >> lwr, ngroup = (a.nrhs + (1 << lwr) - 1) >> lwr;
     if (gpb > ngroup) gpb = ngroup;
     const unsigned ntile = (unsigned)((a.g.Vphys + spb - 1) / spb);
     const unsigned nchunk = (unsigned)((ngroup + gpb - 1) / gpb);
-    dslash32_kernel<S, CHEB, NT, MINB><<<ntile * nchunk, NT, 0, st>>>(a, nchunk, lwr, gpb);
+    dslash32_kernel<S, EPI, NT, MINB><<<ntile * nchunk, NT, 0, st>>>(a, nchunk, lwr, gpb);
     return cudaGetLastError();
 }
 
@@ -698,24 +758,33 @@ cudaError_t launch(const D32 &a, int lwr, int gpb, cudaStream_t st)
 // against 308 us); small blocks of one vector spread small problems over the SMs and keep the
 // neighbour rows of large ones close (12^3 x 24, 8 vectors: 62 against 64 us; 32^3 x 64, 24
 // vectors, FP16: 7.4 against 7.8 ms).
-template <class S, bool CHEB>
+template <class S, int EPI>
 cudaError_t launch_variant(int v, const D32 &a, cudaStream_t st)
 {
     switch (v) {
-    case 0: return launch<S, CHEB, 64, 6>(a, 0, 1, st);
-    case 1: return launch<S, CHEB, 32, 12>(a, 0, 1, st);
-    case 2: return launch<S, CHEB, 128, 3>(a, 0, 1, st);
-    case 3: return launch<S, CHEB, 128, 3>(a, 1, 64, st);
-    case 4: return launch<S, CHEB, 128, 3>(a, 2, 64, st);
-    default: return launch<S, CHEB, 384, 1>(a, 2, 64, st);
+    case 0: return launch<S, EPI, 64, 6>(a, 0, 1, st);
+    case 1: return launch<S, EPI, 32, 12>(a, 0, 1, st);
+    case 2: return launch<S, EPI, 128, 3>(a, 0, 1, st);
+    case 3: return launch<S, EPI, 128, 3>(a, 1, 64, st);
+    case 4: return launch<S, EPI, 128, 3>(a, 2, 64, st);
+    default: return launch<S, EPI, 384, 1>(a, 2, 64, st);
     }
 }
 
-template <class S>
-cudaError_t launch_storage(int v, bool cheb, const D32 &a, cudaStream_t st)
+template <class S, int EPI>
+cudaError_t launch_epi(int v, const D32 &a, cudaStream_t st)
 {
-    if (a.g.Ns * a.nrhs <= kSplitSites) return launch_split<S>(a, cheb, st);
-    return cheb ? launch_variant<S, true>(v, a, st) : launch_variant<S, false>(v, a, st);
+    return a.g.Ns * a.nrhs <= kSplitSites ? launch_split<S, EPI>(a, st) : launch_variant<S, EPI>(v, a, st);
+}
+
+template <class S>
+cudaError_t launch_storage(int v, int epi, const D32 &a, cudaStream_t st)
+{
+    switch (epi) {
+    case QS_EPI_PLAIN: return launch_epi<S, QS_EPI_PLAIN>(v, a, st);
+    case QS_EPI_CHEB: return launch_epi<S, QS_EPI_CHEB>(v, a, st);
+    default: return cudaErrorInvalidValue;
+    }
 }
 
 template <class S>
@@ -761,6 +830,9 @@ cudaError_t qs_d32_batch_launch(const D32BatchItem *items, int n, int storage, i
         a.c = a.s1 = a.s2 = 0.f;
         a.coef = a.dmdev = nullptr;
         a.live = nullptr;
+        a.alpha = nullptr;
+        a.part = nullptr;
+        a.ntile = 0;
         for (int r = 0; r < it.nrhs; ++r) a.dm[r] = (float)(4.0 + it.m0[r]);
         b.off[i] = off;
         const double items_i = (double)((it.g.Vphys + 127) / 128) * it.nrhs;
@@ -778,6 +850,11 @@ cudaError_t qs_d32_batch_launch(const D32BatchItem *items, int n, int storage, i
     }
     qs_note_launches(1);
     return e;
+}
+
+int64_t qs_d32_ntile(const Geom &g, int nrhs)
+{
+    return g.Ns * nrhs <= kSplitSites ? g.Ns / 16 : (g.Vphys + 31) / 32;
 }
 
 int qs_d32_nvariants() { return 6; }
@@ -807,12 +884,17 @@ cudaError_t qs_d32_launch(const D32Call &c, int variant, cudaStream_t st)
     a.coef = c.coef_dev;
     a.dmdev = c.dm_dev;
     a.live = c.live;
-    const bool cheb = c.cheb;
+    a.alpha = c.alpha_dev;
+    a.part = c.part;
+    a.ntile = (int)qs_d32_ntile(c.g, c.nrhs);
     switch (c.storage) {
-    case QS_D32_F32_TILED: return launch_storage<StF32Tiled>(variant, cheb, a, st);
-    case QS_D32_F32_CANON: return launch_storage<StF32Canon>(variant, cheb, a, st);
-    case QS_D32_F16: return launch_storage<StF16>(variant, cheb, a, st);
-    case QS_D32_BF16: return launch_storage<StBF16>(variant, cheb, a, st);
+    case QS_D32_F32_TILED:
+        if (c.epi == QS_EPI_NORM) return launch_epi<StF32Tiled, QS_EPI_NORM>(variant, a, st);
+        if (c.epi == QS_EPI_RESID) return launch_epi<StF32Tiled, QS_EPI_RESID>(variant, a, st);
+        return launch_storage<StF32Tiled>(variant, c.epi, a, st);
+    case QS_D32_F32_CANON: return launch_storage<StF32Canon>(variant, c.epi, a, st);
+    case QS_D32_F16: return launch_storage<StF16>(variant, c.epi, a, st);
+    case QS_D32_BF16: return launch_storage<StBF16>(variant, c.epi, a, st);
     default: return cudaErrorInvalidValue;
     }
 }

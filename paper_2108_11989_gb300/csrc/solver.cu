@@ -40,13 +40,14 @@ struct Workspace {
     int k;
     int64_t nr;
     double *blk64[6];     // FP64 blocks [k][nr]
-    float *blk32[5];      // FP32 blocks [k][nr]: filter (captured buffers 0-3) and CG work
+    float *blk32[4];      // FP32 blocks [k][nr]: filter (captured buffers) and CG work
     float *f32b[3];       // FP32 basis of the filter stage: V, QV and a rotation target
     int iv, iq, it3;      // which of f32b holds V, QV and the scratch
     double *part;         // reduction partials
     double2 *G, *Rinv, *Hm, *Ym;
     double *ds;           // device scalars, S_NSLOT slots of 64
-    int *di;              // device ints: 64 CG flags, 8 status words, 64 CG flags
+    double *cgpart;       // shares of the CG's sums, [k][qs_d32_ntile()]
+    int *di;              // device ints, 64 CG flags + 8
     int *hlive;           // pinned: CG_LAG + 1 copies of the CG flags
     cudaEvent_t ev[CG_LAG + 1];
     double *hp;           // pinned host mirror of ds (S_NSLOT x 64)
@@ -60,7 +61,7 @@ struct Workspace {
 static float *V32(Workspace *w);
 static float *QV32(Workspace *w);
 static float *T32(Workspace *w);
-enum { S_TMP = 0, S_THETA = 1, S_COEF = 2, S_RR = 3, S_RR0 = 4, S_RR1 = 5, S_ONES = 7, S_RN = 8,
+enum { S_TMP = 0, S_THETA = 1, S_COEF = 2, S_RR = 3, S_RR0 = 4, S_AB = 5, S_ONES = 7, S_RN = 8,
        S_DOT = 9 /* two slots */, S_VN = 11, S_NSLOT = 12 };
 
 static void ws_free(Workspace *w)
@@ -70,7 +71,8 @@ static void ws_free(Workspace *w)
     cudaFree(w->coef_dev);
     cudaFreeHost(w->coef_host);
     for (int i = 0; i < 6; ++i) cudaFree(w->blk64[i]);
-    for (int i = 0; i < 5; ++i) cudaFree(w->blk32[i]);
+    for (int i = 0; i < 4; ++i) cudaFree(w->blk32[i]);
+    cudaFree(w->cgpart);
     for (int i = 0; i < 3; ++i) cudaFree(w->f32b[i]);
     cudaFree(w->part); cudaFree(w->G); cudaFree(w->Rinv); cudaFree(w->Hm); cudaFree(w->Ym);
     cudaFree(w->ds); cudaFree(w->di);
@@ -101,23 +103,24 @@ static int ws_alloc(qs_lattice *lat, Workspace *w, int k)
     w->nr = lat->g.Ns * 24;
     size_t n64 = (size_t)k * w->nr * sizeof(double), n32 = (size_t)k * w->nr * sizeof(float);
     for (int i = 0; i < 6; ++i) CK(cudaMalloc(&w->blk64[i], n64));
-    for (int i = 0; i < 5; ++i) CK(cudaMalloc(&w->blk32[i], n32));
+    for (int i = 0; i < 4; ++i) CK(cudaMalloc(&w->blk32[i], n32));
+    CK(cudaMalloc(&w->cgpart, (size_t)k * (lat->g.Ns / 16 + 1) * sizeof(double)));   // either tiling of qs_d32_ntile
     for (int i = 0; i < 3; ++i) CK(cudaMalloc(&w->f32b[i], n32));
     w->iv = 0; w->iq = 1; w->it3 = 2;
-    CK(cudaMalloc(&w->part, (size_t)QS_RED_BLOCKS * 2 * 64 * 64 * sizeof(double)));
+    CK(cudaMalloc(&w->part, std::max((size_t)QS_RED_BLOCKS * 2 * 64 * 64, QS_EIG_SCRATCH(64)) * sizeof(double)));
     CK(cudaMalloc(&w->G, 64 * 64 * sizeof(double2)));
     CK(cudaMalloc(&w->Rinv, 64 * 64 * sizeof(double2)));
     CK(cudaMalloc(&w->Hm, 64 * 64 * sizeof(double2)));
     CK(cudaMalloc(&w->Ym, 64 * 64 * sizeof(double2)));
     CK(cudaMalloc(&w->ds, S_NSLOT * 64 * sizeof(double)));
-    CK(cudaMalloc(&w->di, 136 * sizeof(int)));
+    CK(cudaMalloc(&w->di, 72 * sizeof(int)));
     CK(cudaMallocHost(&w->hp, S_NSLOT * 64 * sizeof(double)));
     CK(cudaMallocHost(&w->hi, 72 * sizeof(int)));
     CK(cudaMallocHost(&w->hlive, (CG_LAG + 1) * 64 * sizeof(int)));
     for (auto &e : w->ev) CK(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
     CK(cudaMalloc(&w->coef_dev, (3 * QS_GRAPH_MAX_DEG + 64) * sizeof(float)));
     CK(cudaMallocHost(&w->coef_host, (3 * QS_GRAPH_MAX_DEG + 64) * sizeof(float)));
-    CK(cudaMemsetAsync(w->di, 0, 136 * sizeof(int), lat->stream));
+    CK(cudaMemsetAsync(w->di, 0, 72 * sizeof(int), lat->stream));
     for (int i = 0; i < 64; ++i) w->hp[i] = 1.0;
     CK(cudaMemcpyAsync(DS(w, S_ONES), w->hp, 64 * sizeof(double), cudaMemcpyHostToDevice, lat->stream));
     CK(cudaStreamSynchronize(lat->stream));
@@ -454,12 +457,13 @@ static int cheb_filter64(qs_lattice *lat, Workspace *w, double m0, int k, int d,
 // vectors that still iterate, and it reads a copy CG_LAG copies later; by then all kernels skip
 // the vectors that have converged, the operator among them.
 static int cg_f32(qs_lattice *lat, Workspace *w, double m0, int k, float *x, float *r, float *p, float *t,
-                  float *ap, double tol, int maxit, int *iters)
+                  double tol, int maxit, int *iters)
 {
     cudaStream_t st = lat->stream;
     CgScalars s;
-    s.rr[0] = DS(w, S_RR); s.rr[1] = DS(w, S_RR1); s.rr0 = DS(w, S_RR0);
-    s.live[0] = w->di; s.live[1] = w->di + 72;
+    s.rr = DS(w, S_RR); s.rr0 = DS(w, S_RR0);
+    s.alpha = (float *)DS(w, S_AB); s.beta = s.alpha + 64;
+    s.live = w->di;
     size_t bytes = (size_t)k * w->nr * sizeof(float);
     CK(cudaMemsetAsync(x, 0, bytes, st));
     CK(cudaMemcpyAsync(p, r, bytes, cudaMemcpyDeviceToDevice, st));
@@ -467,17 +471,27 @@ static int cg_f32(qs_lattice *lat, Workspace *w, double m0, int k, float *x, flo
     CK(qs_cg_init(s, DS(w, S_TMP), k, st));
     double m[QS_MAX_RHS];
     for (int i = 0; i < k; ++i) m[i] = m0;
+    D32Call c;
+    memset(&c, 0, sizeof(c));
+    c.g = lat->g; c.links = lat->links32; c.clov = lat->clov32;
+    c.storage = QS_D32_F32_TILED; c.nrhs = k; c.gamma5 = 1; c.m0 = m;
+    c.live = s.live; c.alpha_dev = s.alpha;
+    c.part = w->cgpart;
+    const int nb = (int)qs_d32_ntile(lat->g, k);
+    D32Call c2 = c;
+    c.epi = QS_EPI_NORM; c.in = p; c.out = t;              // t = Q p
+    c2.epi = QS_EPI_RESID; c2.in = t; c2.y = r; c2.out = r;   // r -= alpha Q t
     int it = 0, polls = 0, seen = 0;
     bool done = false;
     while (it < maxit && !done) {
-        const int *live = s.live[it & 1];
-        QS_TRY(qs_d32_run(lat, QS_D32_F32_TILED, m, p, t, k, 1, nullptr, nullptr, 0, 0, 0, nullptr, nullptr, live));
-        QS_TRY(qs_d32_run(lat, QS_D32_F32_TILED, m, t, ap, k, 1, nullptr, nullptr, 0, 0, 0, nullptr, nullptr, live));
-        CK(qs_cg_step(x, r, p, t, ap, s, it, tol * tol, k, w->nr, w->part, st));
+        QS_TRY(qs_d32_call(lat, c));
+        CK(qs_cg_alpha(s, k, w->cgpart, nb, st));
+        QS_TRY(qs_d32_call(lat, c2));
+        CK(qs_cg_beta_xp(x, p, r, s, tol * tol, k, w->nr, w->cgpart, nb, st));
         ++it;
         if (it % CG_POLL == 0 || it == maxit) {
             const int slot = polls++ % (CG_LAG + 1);
-            CK(cudaMemcpyAsync(w->hlive + 64 * slot, s.live[it & 1], k * sizeof(int), cudaMemcpyDeviceToHost, st));
+            CK(cudaMemcpyAsync(w->hlive + 64 * slot, s.live, k * sizeof(int), cudaMemcpyDeviceToHost, st));
             CK(cudaEventRecord(w->ev[slot], st));
             if (polls - seen > CG_LAG) {
                 const int old = seen++ % (CG_LAG + 1);
@@ -521,8 +535,7 @@ static int solve_q2_mixed(qs_lattice *lat, Workspace *w, double m0, int k, const
         CK(qs_d2f(T2, w->blk32[0], DS(w, S_COEF), k, w->nr, st));
         double tin = std::max(2e-6, std::min(0.1, 0.3 * tol / rmax));
         int its = 0;
-        QS_TRY(cg_f32(lat, w, m0, k, w->blk32[1], w->blk32[0], w->blk32[2], w->blk32[3], w->blk32[4], tin,
-                      20000, &its));
+        QS_TRY(cg_f32(lat, w, m0, k, w->blk32[1], w->blk32[0], w->blk32[2], w->blk32[3], tin, 20000, &its));
         if (verbose() > 1) fprintf(stderr, "[qstar]   inner CG %d iterations (tol %.2e)\n", its, tin);
         CK(qs_map_scalars(DS(w, S_RN), DS(w, S_COEF), k, 1, st));             // |r|
         CK(qs_axpy_f2d(X, w->blk32[1], DS(w, S_COEF), k, w->nr, st));
