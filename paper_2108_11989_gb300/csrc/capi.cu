@@ -374,7 +374,7 @@ int qs_d32_call(qs_lattice *lat, const D32Call &c)
     const int storage = c.storage, nrhs = c.nrhs, cheb = c.epi == QS_EPI_CHEB;
     int &tv = lat->tuned32[storage][cheb][nrhs];
     if (tv == 0) {
-        const std::string key = tune_key(lat, "dslash32p", storage, cheb, nrhs);
+        const std::string key = tune_key(lat, "dslash32q", storage, cheb, nrhs);
         int v = tune_lookup(key);
         if (v < 0 || v >= qs_d32_nvariants()) {
             if (capturing(lat->stream) || c.epi == QS_EPI_RESID) {

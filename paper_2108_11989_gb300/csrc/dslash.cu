@@ -18,7 +18,7 @@ __device__ __forceinline__ void dslash_site(const Geom &g, const double2 *__rest
     const Lane64 ln = qs_lane64(g, on ? s : (int)g.Ns - 1);
     double2 up[3], low[3];
     qs_hops64<AT>(g, links, in, ln, up, low);
-    qs_diag64<AT>(SwF64{clov + ln.c.p, g.Vphys}, in, ln, 4.0 + m0, up, low);
+    qs_diag64<AT>(g, clov, in, ln, 4.0 + m0, up, low);
     if (!on) return;
     double2 *out = reinterpret_cast<double2 *>(out_all) + (int64_t)r * g.Ns * 12;
     const unsigned g5 = gamma5 ? 0x80000000u : 0u;

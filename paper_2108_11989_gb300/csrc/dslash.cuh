@@ -72,10 +72,10 @@ struct D32Call {
     const float *dm_dev;   // NULL, or device 4 + m0 per right-hand side
     const float *alpha_dev;   // RESID: device, per right-hand side
     double *part;          // NORM, RESID: device [nrhs][qs_d32_ntile()] shares of |out|^2
-    const int *live;       // NULL, or device flags: right-hand sides with 0 are skipped
+    const int *live;       // NORM, RESID: NULL, or device flags: right-hand sides with 0 are skipped
 };
 int qs_d32_nvariants();
-int64_t qs_d32_ntile(const Geom &g, int nrhs);
+int64_t qs_d32_ntile(const Geom &g);
 int64_t qs_d32_vec_bytes(int storage, int64_t Ns);
 cudaError_t qs_d32_launch(const D32Call &c, int variant, cudaStream_t st);
 // the same with the handle's autotuned variant and profiling records (capi.cu)

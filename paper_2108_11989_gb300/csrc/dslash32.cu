@@ -38,7 +38,6 @@
 // CG iteration never writes Q^2 p and reads neither it nor Q p for its sums.
 #include "qs_internal.cuh"
 #include "dslash.cuh"
-#include "dslash64.cuh"
 #include "stencil.cuh"
 
 #include <cuda_bf16.h>
@@ -110,19 +109,6 @@ struct StF32Tiled {
 #pragma unroll
         for (int c = 0; c < 12; ++c) v[c] = __ldg(b + c * 16);
     }
-    // the 3 components of one spin
-    __device__ static void ld3(const char *__restrict__ base, int s, int spin, cf v[3])
-    {
-        const cf *b = reinterpret_cast<const cf *>(base) + ((int64_t)(s >> 4) * 12 + 3 * spin) * 16 + (s & 15);
-#pragma unroll
-        for (int c = 0; c < 3; ++c) v[c] = __ldg(b + c * 16);
-    }
-    __device__ static void st3(char *__restrict__ base, int s, int spin, const cf v[3], float)
-    {
-        cf *b = reinterpret_cast<cf *>(base) + ((int64_t)(s >> 4) * 12 + 3 * spin) * 16 + (s & 15);
-#pragma unroll
-        for (int c = 0; c < 3; ++c) b[c * 16] = v[c];
-    }
     // the 6 components of chiral block `blk` (spins 2 blk, 2 blk + 1)
     __device__ static void ld6(const char *__restrict__ base, int s, int blk, cf v[6])
     {
@@ -165,18 +151,6 @@ struct StF32Canon {
             v[2 * i] = make_float2(a.x, a.y);
             v[2 * i + 1] = make_float2(a.z, a.w);
         }
-    }
-    __device__ static void ld3(const char *__restrict__ base, int s, int spin, cf v[3])
-    {
-        const cf *b = reinterpret_cast<const cf *>(base) + (int64_t)s * 12 + 3 * spin;
-#pragma unroll
-        for (int c = 0; c < 3; ++c) v[c] = __ldg(b + c);
-    }
-    __device__ static void st3(char *__restrict__ base, int s, int spin, const cf v[3], float)
-    {
-        cf *b = reinterpret_cast<cf *>(base) + (int64_t)s * 12 + 3 * spin;
-#pragma unroll
-        for (int c = 0; c < 3; ++c) b[c] = v[c];
     }
     __device__ static void ld6(const char *__restrict__ base, int s, int blk, cf v[6])
     {
@@ -232,30 +206,6 @@ struct StScaled {
             float2 f = cvt(h);
             v[c] = make_float2(f.x * sc, f.y * sc);
         }
-    }
-    __device__ static void ld3(const char *__restrict__ base, int s, int spin, cf v[3])
-    {
-        const char *t = base + (int64_t)(s >> 4) * kTile;
-        const unsigned *w = reinterpret_cast<const unsigned *>(t) + 48 * spin + (s & 15);
-        const float sc = __ldg(reinterpret_cast<const float *>(t + 768) + (s & 15));
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            const unsigned u = __ldg(w + c * 16);
-            v[c] = mul2(dup(sc), cvt(*reinterpret_cast<const H2 *>(&u)));
-        }
-    }
-    // m: the site's largest component
-    __device__ static void st3(char *__restrict__ base, int s, int spin, const cf v[3], float m)
-    {
-        char *t = base + (int64_t)(s >> 4) * kTile;
-        const float inv = m > 0.f ? 1.0f / m : 0.f;
-        unsigned *w = reinterpret_cast<unsigned *>(t) + 48 * spin + (s & 15);
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            H2 h = pack(v[c].x * inv, v[c].y * inv);
-            w[c * 16] = *reinterpret_cast<unsigned *>(&h);
-        }
-        if (spin == 0) reinterpret_cast<float *>(t + 768)[s & 15] = m;
     }
     __device__ static void ld6(const char *__restrict__ base, int s, int blk, cf v[6])
     {
@@ -378,7 +328,7 @@ struct D32 {
     // device-side overrides (for launches replayed from a CUDA graph): if set, (c, s1, s2)
     // are read from coef[0..2] and 4 + m0 of right-hand side r from dmdev[r]
     const float *coef, *dmdev;
-    const int *live;    // NULL, or flags: right-hand sides with live[r] = 0 are skipped
+    const int *live;    // NORM, RESID: NULL, or flags: right-hand sides with live[r] = 0 are skipped
     const float *alpha; // RESID: per right-hand side
     double *part;       // NORM, RESID: [nrhs][ntile] shares of |out|^2
     int ntile;
@@ -477,6 +427,24 @@ __device__ __forceinline__ float site_norm2(const cf v[12])
     return q.x + q.y;
 }
 
+// hops D .. 7 of one site only (sg = 1: the physical one, -1: its mirror), the next neighbour's
+// spinor and link in flight while the current one is multiplied
+template <int D, class S>
+__device__ __forceinline__ void hops_one(const D32 &a, const Site &c, const char *in, bool mir, float sg, const Hop &h,
+                                         const typename S::Raw &v, cf acc[12])
+{
+    if constexpr (D < 7) {
+        Hop h2;
+        typename S::Raw w;
+        hop_begin<D + 1>(a, c, h2);
+        S::fetch(in, mir ? h2.nm : h2.n, w);
+        hop_apply<D / 2, D % 2 == 0, S>(h.U, sg * h.sigma, h.f, a.g.t_anti, v, acc);
+        hops_one<D + 1, S>(a, c, in, mir, sg, h2, w, acc);
+    } else {
+        hop_apply<D / 2, D % 2 == 0, S>(h.U, sg * h.sigma, h.f, a.g.t_anti, v, acc);
+    }
+}
+
 // the warp's sum of x, kept as a two-sum pair, to *out by lane 0
 __device__ __forceinline__ void warp_share(float x, double *out)
 {
@@ -525,7 +493,7 @@ __device__ __forceinline__ float finish_site(const D32 &a, int64_t off, int s, i
 template <class S, int EPI>
 __device__ __forceinline__ void site_kernel(const D32 &a, int p, int r, bool on = true)
 {
-    if (a.live && !a.live[r]) return;
+    if (EPI >= QS_EPI_NORM && a.live && !a.live[r]) return;
     const int row = p / a.g.L;
     const Site c = site_of(a.g, p + row * a.g.L);   // x < L: s = row 2L + x, p = row L + x
     const int64_t off = (int64_t)r * a.vbytes;
@@ -554,7 +522,41 @@ __device__ __forceinline__ void site_kernel(const D32 &a, int p, int r, bool on 
     hops<0, S>(a, c, in, h, v, acc, accm);
     float n2 = finish_site<S, EPI>(a, off, c.s, r, on, acc);
     n2 += finish_site<S, EPI>(a, off, c.s + a.g.L, r, on, accm);
-    if (EPI >= QS_EPI_NORM) warp_share(n2, a.part + (int64_t)r * a.ntile + p / 32);
+    if (EPI >= QS_EPI_NORM) {   // two shares per 32 physical sites, as one_kernel leaves them
+        double *sh = a.part + (int64_t)r * a.ntile + 2 * (p / 32);
+        warp_share(n2, sh);
+        if ((threadIdx.x & 31) == 0) sh[1] = 0.0;
+    }
+}
+
+// physical site p (mir = false) or its mirror alone: the same arithmetic as site_kernel's for that
+// site, in half the chain of loads and products.  mir is the same in the whole warp.
+template <class S, int EPI>
+__device__ __forceinline__ void one_kernel(const D32 &a, int p, int r, bool mir, bool on)
+{
+    if (EPI >= QS_EPI_NORM && a.live && !a.live[r]) return;
+    const Site c = site_of(a.g, p + (p / a.g.L) * a.g.L);
+    const int s = mir ? c.s + a.g.L : c.s;
+    const int64_t off = (int64_t)r * a.vbytes;
+    const char *in = a.in + off;
+    cf acc[12];
+    const float dm = a.dmdev ? __ldg(a.dmdev + r) : a.dm[r];
+#pragma unroll
+    for (int b = 0; b < 2; ++b) {
+        cf P[18], v[6];
+#pragma unroll
+        for (int q = 0; q < 18; ++q) P[q] = __ldg(a.clov + (int64_t)(b * 18 + q) * a.g.Vphys + p);
+        S::ld6(in, s, b, v);
+        if (mir) sw_block<true>(P, dm, v, acc + 6 * b);
+        else sw_block<false>(P, dm, v, acc + 6 * b);
+    }
+    Hop h;
+    typename S::Raw v;
+    hop_begin<0>(a, c, h);
+    S::fetch(in, mir ? h.nm : h.n, v);
+    hops_one<0, S>(a, c, in, mir, mir ? -1.f : 1.f, h, v, acc);
+    const float n2 = finish_site<S, EPI>(a, off, s, r, on, acc);
+    if (EPI >= QS_EPI_NORM) warp_share(n2, a.part + (int64_t)r * a.ntile + 2 * (p / 32) + (mir ? 1 : 0));
 }
 
 // A block's NT / 32 warps are WR right-hand sides x (NT / 32 / WR) groups of 32 physical sites;
@@ -577,93 +579,25 @@ __global__ void __launch_bounds__(NT, MINB) dslash32_kernel(const __grid_constan
     for (int i = 0; i < gpb && r < a.nrhs; ++i, r += wr) site_kernel<S, EPI>(a, p, r, on);
 }
 
-// ---- small problems: two threads per site (dslash64.cuh in FP32) ------------------------
-template <class S>
-struct Mem32 {
-    typedef float R;
-    typedef float2 V2;
-    __device__ static void ld3(const cf *__restrict__ in, int s, int spin, cf v[3])
-    {
-        S::ld3(reinterpret_cast<const char *>(in), s, spin, v);
-    }
-};
-
-// A pair thread's chain of loads and products is about 17 k cycles long, which is all the time
-// there is when the lattice has too few sites to fill the SMs; a quarter of the work per
-// thread then wins although links and SW words are loaded four times as often.  Up to 16 k
-// sites x right-hand sides 6.2 us against 8.2 us back to back, the same at 32 k, and slower from 48 k
-// on (FP32 and FP16 alike), hence the line at 24 k.  It is a line in the sites and vectors
-// alone, so the layouts of one problem always take the same arithmetic.
-constexpr int64_t kSplitSites = 24576;
-
+// Problems that fill the SMs a few times at most: a block is 32 physical sites and one right-hand
+// side, its first warp on the sites and its second on their mirrors.  A pair thread's chain is about
+// 17 k cycles, all the time there is when few warps run: 4^3 x 8, 24 vectors, 8.2 -> 6.2 us back to
+// back, even with the pairs at 100 k sites x vectors, slower beyond (12^3 x 24, 8 vectors: 71
+// against 61 us).
 template <class S, int EPI>
-__global__ void __launch_bounds__(64, 10) dslash32_split_kernel(const __grid_constant__ D32 a)
+__global__ void __launch_bounds__(64, 8) dslash32_one_kernel(const __grid_constant__ D32 a)
 {
-    const int r = (int)(blockIdx.x % (unsigned)a.nrhs);
-    if (a.live && !a.live[r]) return;
-    const int s0 = (int)(blockIdx.x / (unsigned)a.nrhs) * 32 + (int)(threadIdx.x >> 5) * 16 + (int)(threadIdx.x & 15);
-    const bool on = s0 < (int)a.g.Ns;
-    const Lane64 ln = qs_lane64(a.g, on ? s0 : (int)a.g.Ns - 1);
-    const int64_t off = (int64_t)r * a.vbytes;
-    const cf *in = reinterpret_cast<const cf *>(a.in + off);
-    const float dm = a.dmdev ? __ldg(a.dmdev + r) : a.dm[r];
-    cf up[3], low[3];
-    qs_hops64<Mem32<S>>(a.g, a.links, in, ln, up, low);
-    qs_diag64<Mem32<S>>(SwF32{a.clov + ln.c.p, a.g.Vphys}, in, ln, dm, up, low);
-    if (a.gamma5) {
-#pragma unroll
-        for (int i = 0; i < 3; ++i) low[i] = cneg(low[i]);
-    }
-    if (EPI == QS_EPI_CHEB) {
-        const float cc = a.coef ? __ldg(a.coef) : a.c;
-        const float s1 = a.coef ? __ldg(a.coef + 1) : a.s1;
-        const float s2 = a.coef ? __ldg(a.coef + 2) : a.s2;
-#pragma unroll
-        for (int b = 0; b < 2; ++b) {
-            cf yv[3], xv[3];
-            S::ld3(a.y + off, ln.c.s, 2 * b + ln.q, yv);
-            S::ld3(a.x + off, ln.c.s, 2 * b + ln.q, xv);
-            cf *o = b ? low : up;
-#pragma unroll
-            for (int i = 0; i < 3; ++i) o[i] = fma2(dup(s1), fma2(dup(-cc), yv[i], o[i]), mul2(dup(-s2), xv[i]));
-        }
-    }
-    if (EPI == QS_EPI_RESID) {
-        const float al = a.alpha[r];
-#pragma unroll
-        for (int b = 0; b < 2; ++b) {
-            const cf *y = reinterpret_cast<const cf *>(a.y + off) + ((int64_t)(ln.c.s >> 4) * 12 + 6 * b + 3 * ln.q) * 16 + (ln.c.s & 15);
-            cf *o = b ? low : up;
-#pragma unroll
-            for (int i = 0; i < 3; ++i) o[i] = fma2(dup(-al), o[i], y[i * 16]);
-        }
-    }
-    if (EPI >= QS_EPI_NORM) {
-        cf n2 = make_float2(0.f, 0.f);
-#pragma unroll
-        for (int i = 0; i < 3; ++i) n2 = fma2(up[i], up[i], fma2(low[i], low[i], n2));
-        const int tile = (s0 - (int)(threadIdx.x & 15)) >> 4;
-        if (tile < a.ntile) warp_share(on ? n2.x + n2.y : 0.f, a.part + (int64_t)r * a.ntile + tile);
-    }
-    float m = 0.f;
-    if constexpr (S::kScaled) {
-#pragma unroll
-        for (int i = 0; i < 3; ++i) {
-            m = fmaxf(m, fmaxf(fabsf(up[i].x), fabsf(up[i].y)));
-            m = fmaxf(m, fmaxf(fabsf(low[i].x), fabsf(low[i].y)));
-        }
-        m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 16));
-    }
-    if (!on) return;
-    S::st3(a.out + off, s0, ln.q, up, m);
-    S::st3(a.out + off, s0, 2 + ln.q, low, m);
+    const int r = (int)(blockIdx.x % (unsigned)a.nrhs), p0 = (int)(blockIdx.x / (unsigned)a.nrhs) * 32;
+    const int p = p0 + (int)(threadIdx.x & 31);
+    const bool on = p < (int)a.g.Vphys;
+    if (EPI < QS_EPI_NORM && !on) return;
+    one_kernel<S, EPI>(a, on ? p : (int)a.g.Vphys - 1, r, threadIdx.x >= 32, on);
 }
 
 template <class S, int EPI>
-cudaError_t launch_split(const D32 &a, cudaStream_t st)
+cudaError_t launch_one(const D32 &a, cudaStream_t st)
 {
-    const unsigned nb = (unsigned)((a.g.Ns + 31) / 32) * (unsigned)a.nrhs;
-    dslash32_split_kernel<S, EPI><<<nb, 64, 0, st>>>(a);
+    dslash32_one_kernel<S, EPI><<<(unsigned)((a.g.Vphys + 31) / 32) * (unsigned)a.nrhs, 64, 0, st>>>(a);
     return cudaGetLastError();
 }
 
@@ -756,8 +690,9 @@ cudaError_t launch(const D32 &a, int lwr, int gpb, cudaStream_t st)
 // sides side by side or in turn read a site's links and SW words from L1 instead of L2, which
 // pays from about 16 vectors on a lattice that fills the chip (16^3 x 32, 16 vectors, FP32: 298
 // against 308 us); small blocks of one vector spread small problems over the SMs and keep the
-// neighbour rows of large ones close (12^3 x 24, 8 vectors: 62 against 64 us; 32^3 x 64, 24
-// vectors, FP16: 7.4 against 7.8 ms).
+// neighbour rows of large ones close (12^3 x 24, 8 vectors: 61 against 63 us; 32^3 x 64, 24
+// vectors, FP16: 7.4 against 7.8 ms); the smallest problems take a thread per site.  All variants
+// compute a site in the same order, so the choice does not show in the result.
 template <class S, int EPI>
 cudaError_t launch_variant(int v, const D32 &a, cudaStream_t st)
 {
@@ -767,22 +702,17 @@ cudaError_t launch_variant(int v, const D32 &a, cudaStream_t st)
     case 2: return launch<S, EPI, 128, 3>(a, 0, 1, st);
     case 3: return launch<S, EPI, 128, 3>(a, 1, 64, st);
     case 4: return launch<S, EPI, 128, 3>(a, 2, 64, st);
+    case 5: return launch_one<S, EPI>(a, st);
     default: return launch<S, EPI, 384, 1>(a, 2, 64, st);
     }
-}
-
-template <class S, int EPI>
-cudaError_t launch_epi(int v, const D32 &a, cudaStream_t st)
-{
-    return a.g.Ns * a.nrhs <= kSplitSites ? launch_split<S, EPI>(a, st) : launch_variant<S, EPI>(v, a, st);
 }
 
 template <class S>
 cudaError_t launch_storage(int v, int epi, const D32 &a, cudaStream_t st)
 {
     switch (epi) {
-    case QS_EPI_PLAIN: return launch_epi<S, QS_EPI_PLAIN>(v, a, st);
-    case QS_EPI_CHEB: return launch_epi<S, QS_EPI_CHEB>(v, a, st);
+    case QS_EPI_PLAIN: return launch_variant<S, QS_EPI_PLAIN>(v, a, st);
+    case QS_EPI_CHEB: return launch_variant<S, QS_EPI_CHEB>(v, a, st);
     default: return cudaErrorInvalidValue;
     }
 }
@@ -852,12 +782,9 @@ cudaError_t qs_d32_batch_launch(const D32BatchItem *items, int n, int storage, i
     return e;
 }
 
-int64_t qs_d32_ntile(const Geom &g, int nrhs)
-{
-    return g.Ns * nrhs <= kSplitSites ? g.Ns / 16 : (g.Vphys + 31) / 32;
-}
+int64_t qs_d32_ntile(const Geom &g) { return 2 * ((g.Vphys + 31) / 32); }
 
-int qs_d32_nvariants() { return 6; }
+int qs_d32_nvariants() { return 7; }
 
 int64_t qs_d32_vec_bytes(int storage, int64_t Ns)
 {
@@ -886,11 +813,11 @@ cudaError_t qs_d32_launch(const D32Call &c, int variant, cudaStream_t st)
     a.live = c.live;
     a.alpha = c.alpha_dev;
     a.part = c.part;
-    a.ntile = (int)qs_d32_ntile(c.g, c.nrhs);
+    a.ntile = (int)qs_d32_ntile(c.g);
     switch (c.storage) {
     case QS_D32_F32_TILED:
-        if (c.epi == QS_EPI_NORM) return launch_epi<StF32Tiled, QS_EPI_NORM>(variant, a, st);
-        if (c.epi == QS_EPI_RESID) return launch_epi<StF32Tiled, QS_EPI_RESID>(variant, a, st);
+        if (c.epi == QS_EPI_NORM) return launch_variant<StF32Tiled, QS_EPI_NORM>(variant, a, st);
+        if (c.epi == QS_EPI_RESID) return launch_variant<StF32Tiled, QS_EPI_RESID>(variant, a, st);
         return launch_storage<StF32Tiled>(variant, c.epi, a, st);
     case QS_D32_F32_CANON: return launch_storage<StF32Canon>(variant, c.epi, a, st);
     case QS_D32_F16: return launch_storage<StF16>(variant, c.epi, a, st);

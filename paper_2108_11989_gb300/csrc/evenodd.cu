@@ -261,7 +261,7 @@ __global__ void __launch_bounds__(128, 4) hat_even_kernel(const __grid_constant_
     const Lane64 ln = qs_lane64(a.g, parity_site(a.g, j, 0));
     double2 w[2][3];
     qs_hops64<At64Half>(a.g, a.links, v + (int64_t)r * nh * 12, ln, w[0], w[1]);
-    if constexpr (DIAG) qs_diag64<AT>(SwF64{a.clov + ln.c.p, a.g.Vphys}, x + r * len, ln, a.dm, w[0], w[1]);
+    if constexpr (DIAG) qs_diag64<AT>(a.g, a.clov, x + r * len, ln, a.dm, w[0], w[1]);
     const unsigned g5 = a.gamma5 ? 0x80000000u : 0u;
     double acc = 0.0;
     double2 *o = out + r * len;

@@ -104,7 +104,7 @@ static int ws_alloc(qs_lattice *lat, Workspace *w, int k)
     size_t n64 = (size_t)k * w->nr * sizeof(double), n32 = (size_t)k * w->nr * sizeof(float);
     for (int i = 0; i < 6; ++i) CK(cudaMalloc(&w->blk64[i], n64));
     for (int i = 0; i < 4; ++i) CK(cudaMalloc(&w->blk32[i], n32));
-    CK(cudaMalloc(&w->cgpart, (size_t)k * (lat->g.Ns / 16 + 1) * sizeof(double)));   // either tiling of qs_d32_ntile
+    CK(cudaMalloc(&w->cgpart, (size_t)k * qs_d32_ntile(lat->g) * sizeof(double)));
     for (int i = 0; i < 3; ++i) CK(cudaMalloc(&w->f32b[i], n32));
     w->iv = 0; w->iq = 1; w->it3 = 2;
     CK(cudaMalloc(&w->part, std::max((size_t)QS_RED_BLOCKS * 2 * 64 * 64, QS_EIG_SCRATCH(64)) * sizeof(double)));
@@ -477,7 +477,7 @@ static int cg_f32(qs_lattice *lat, Workspace *w, double m0, int k, float *x, flo
     c.storage = QS_D32_F32_TILED; c.nrhs = k; c.gamma5 = 1; c.m0 = m;
     c.live = s.live; c.alpha_dev = s.alpha;
     c.part = w->cgpart;
-    const int nb = (int)qs_d32_ntile(lat->g, k);
+    const int nb = (int)qs_d32_ntile(lat->g);
     D32Call c2 = c;
     c.epi = QS_EPI_NORM; c.in = p; c.out = t;              // t = Q p
     c2.epi = QS_EPI_RESID; c2.in = t; c2.y = r; c2.out = r;   // r -= alpha Q t

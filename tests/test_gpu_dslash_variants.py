@@ -2,12 +2,11 @@
 
 The autotuner picks one variant per shape, so each is forced in turn (a child process with a
 tune cache that names it) on lattices whose sites fill no block (6^3 x 5: 1080 physical sites,
-10^3 x 3: 3000) and on blocks of vectors that fill no group of 2 or 4.  Problems of up to 24576
-sites x vectors (2^3 x 3, 4^4 and the small blocks of 6^3 x 5) take the FP32 kernel with two
-threads per site instead, whichever variant is named.  Tolerances, max-norm
-relative to the largest output component: 1e-5 for FP32 storage; for FP16 storage half a unit
-in the last place at 1 relative to the site's largest component (2^-11), twice that allowed.  FP64: 1e-13 (about 300 roundings of
-2^-53 each on the longest chain, of terms no larger than the output's scale).
+10^3 x 3: 3000, 2^3 x 3: 24) and on blocks of vectors that fill no group of 2 or 4.  Tolerances,
+max-norm relative to the largest output component: 1e-5 for FP32 storage; for FP16 storage half
+a unit in the last place at 1 relative to the site's largest component (2^-11), twice that
+allowed; for FP64 1e-13 (about 300 roundings of 2^-53 each on the longest chain, of terms no
+larger than the output's scale).
 """
 import os
 import subprocess
@@ -59,12 +58,12 @@ for L, T, mask, anti, rhs in %(shapes)r:
 """
 
 
-@pytest.mark.parametrize("variant", range(6))
+@pytest.mark.parametrize("variant", range(7))
 def test_forced_variant_matches_oracle(variant, tmp_path):
     import torch
     gpu = torch.cuda.get_device_name(0).replace(" ", "_")
     cache = tmp_path / "tune"
-    cache.write_text("".join(f"{gpu}|dslash32p|{st}|0|{n}|{L}x{T} {variant}\n"
+    cache.write_text("".join(f"{gpu}|dslash32q|{st}|0|{n}|{L}x{T} {variant}\n"
                              for L, T, _, _, rhs in SHAPES + SMALL for n in rhs for st in range(4)))
     r = subprocess.run([sys.executable, "-c", CHILD % {"root": ROOT, "shapes": SHAPES + SMALL}],
                        env=dict(os.environ, QS_TUNE_CACHE=str(cache)), capture_output=True, text=True, timeout=300)
