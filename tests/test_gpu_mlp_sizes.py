@@ -1,6 +1,5 @@
-"""The step network at sizes that fill no tile (products are tiled 32 x 32 x 32, the batch is cut
-into slices of at least 64 rows for the weight gradients) against the FP64 oracle: loss and
-gradients to 1e-4 of the largest entry (FP32 sums of at most 600 terms)."""
+"""The step network at sizes that fill no tile (products are tiled 32 x 32 x 32) against the FP64
+oracle: loss and gradients to 1e-4 of the largest entry (FP32 sums of at most 600 terms)."""
 import numpy as np
 import pytest
 
