@@ -3,6 +3,7 @@
 // eigensolver for the Rayleigh-Ritz matrix.  Complex matrices are row-major
 // double2 [k][k].
 #include "blas.cuh"
+#include "rank.h"
 
 #include <mutex>
 
@@ -159,6 +160,7 @@ __global__ void __launch_bounds__(256) jacobi_kernel(JacobiJob j0, JacobiJob j1,
         for (int w = 0; w < (nt >> 5); ++w) { off += red[0][w]; tot += red[1][w]; }
         __syncthreads();
         if (off <= 1e-30 * tot || off == 0.0) break;
+        if (isnan(off) || isnan(tot)) { sweep = JAC_SWEEPS; break; }   // no sweep can help
         for (int r = 0; r < k - 1; ++r, ++rounds) {
             if (t < half) {
                 int p = rr_player(t, r, k), q = rr_player(k - 1 - t, r, k);
@@ -221,13 +223,10 @@ __global__ void __launch_bounds__(256) jacobi_kernel(JacobiJob j0, JacobiJob j1,
             __syncthreads();
         }
     }
-    for (int i = t; i < k; i += nt) {   // stable order by |ev|
+    for (int i = t; i < k; i += nt) {   // stable order by |ev|; a permutation for any values
         const double e = fabs(H[i * k + i].x);
         int rank = 0;
-        for (int j = 0; j < k; ++j) {
-            const double f = fabs(H[j * k + j].x);
-            rank += f < e || (f == e && j < i);
-        }
+        for (int j = 0; j < k; ++j) rank += qs_abs_before(fabs(H[j * k + j].x), j, e, i);
         job.ev[rank] = H[i * k + i].x;
         if (job.nround) job.nround[1 + rank] = i;
     }
