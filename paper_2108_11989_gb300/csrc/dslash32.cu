@@ -520,12 +520,12 @@ __device__ __forceinline__ void site_kernel(const D32 &a, int p, int r, bool on 
     hop_begin<0>(a, c, h);
     S::fetch(in, h.n, v);
     hops<0, S>(a, c, in, h, v, acc, accm);
-    float n2 = finish_site<S, EPI>(a, off, c.s, r, on, acc);
-    n2 += finish_site<S, EPI>(a, off, c.s + a.g.L, r, on, accm);
-    if (EPI >= QS_EPI_NORM) {   // two shares per 32 physical sites, as one_kernel leaves them
+    const float n2 = finish_site<S, EPI>(a, off, c.s, r, on, acc);
+    const float m2 = finish_site<S, EPI>(a, off, c.s + a.g.L, r, on, accm);
+    if (EPI >= QS_EPI_NORM) {   // two shares per 32 physical sites, the ones that one_kernel leaves
         double *sh = a.part + (int64_t)r * a.ntile + 2 * (p / 32);
         warp_share(n2, sh);
-        if ((threadIdx.x & 31) == 0) sh[1] = 0.0;
+        warp_share(m2, sh + 1);
     }
 }
 
@@ -692,7 +692,9 @@ cudaError_t launch(const D32 &a, int lwr, int gpb, cudaStream_t st)
 // against 308 us); small blocks of one vector spread small problems over the SMs and keep the
 // neighbour rows of large ones close (12^3 x 24, 8 vectors: 61 against 63 us; 32^3 x 64, 24
 // vectors, FP16: 7.4 against 7.8 ms); the smallest problems take a thread per site.  All variants
-// compute a site in the same order, so the choice does not show in the result.
+// compute a site in the same order, and NORM and RESID leave the same shares of |out|^2 (the 32
+// sites of a warp, their mirrors apart), so the choice, which is made by timing, does not show in
+// any result.
 template <class S, int EPI>
 cudaError_t launch_variant(int v, const D32 &a, cudaStream_t st)
 {
