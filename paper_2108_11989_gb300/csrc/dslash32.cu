@@ -418,13 +418,21 @@ __device__ __forceinline__ void hops(const D32 &a, const Site &c, const char *in
     }
 }
 
-// |v|^2 of 12 components
-__device__ __forceinline__ float site_norm2(const cf v[12])
+// |v|^2 of 12 components as an unevaluated sum q + lo: exact squares by fused multiply-adds, their
+// sums by two-sum (hi + v v = s + e with s rounded, b = s - hi, e = (v v - b) + (hi - (s - b))).
+// A plain FP32 chain of the 24 squares is three to six times further from the 64-bit sum
+// on 4^4 to 8^3 x 12 than reductions with one or two squares per thread.
+__device__ __forceinline__ cf site_norm2(const cf v[12])
 {
-    cf q = mul2(v[0], v[0]);
+    cf q = mul2(v[0], v[0]), lo = fma2(v[0], v[0], cneg(q));
 #pragma unroll
-    for (int i = 1; i < 12; ++i) q = fma2(v[i], v[i], q);
-    return q.x + q.y;
+    for (int i = 1; i < 12; ++i) {
+        const cf s = fma2(v[i], v[i], q), nb = sub2(q, s);   // -b
+        lo = add2(lo, add2(fma2(v[i], v[i], nb), sub2(q, add2(s, nb))));
+        q = s;
+    }
+    const float t = q.x + q.y, b = t - q.x;
+    return make_float2(t, lo.x + lo.y + ((q.x - (t - b)) + (q.y - b)));
 }
 
 // hops D .. 7 of one site only (sg = 1: the physical one, -1: its mirror), the next neighbour's
@@ -445,23 +453,22 @@ __device__ __forceinline__ void hops_one(const D32 &a, const Site &c, const char
     }
 }
 
-// the warp's sum of x, kept as a two-sum pair, to *out by lane 0
-__device__ __forceinline__ void warp_share(float x, double *out)
+// the warp's sum of x.x + x.y, kept as a two-sum pair, to *out by lane 0
+__device__ __forceinline__ void warp_share(cf x, double *out)
 {
-    float lo = 0.f;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
-        const float h2 = __shfl_xor_sync(0xffffffffu, x, o), l2 = __shfl_xor_sync(0xffffffffu, lo, o);
-        const float t = x + h2, b = t - x;
-        lo += l2 + ((x - (t - b)) + (h2 - b));
-        x = t;
+        const float h2 = __shfl_xor_sync(0xffffffffu, x.x, o), l2 = __shfl_xor_sync(0xffffffffu, x.y, o);
+        const float t = x.x + h2, b = t - x.x;
+        x.y += l2 + ((x.x - (t - b)) + (h2 - b));
+        x.x = t;
     }
-    if ((threadIdx.x & 31) == 0) *out = (double)x + (double)lo;
+    if ((threadIdx.x & 31) == 0) *out = (double)x.x + (double)x.y;
 }
 
-// returns |out|^2 at the site for NORM and RESID
+// returns |out|^2 at the site for NORM and RESID (site_norm2)
 template <class S, int EPI>
-__device__ __forceinline__ float finish_site(const D32 &a, int64_t off, int s, int r, bool on, cf acc[12])
+__device__ __forceinline__ cf finish_site(const D32 &a, int64_t off, int s, int r, bool on, cf acc[12])
 {
     if (a.gamma5) {
 #pragma unroll
@@ -485,7 +492,7 @@ __device__ __forceinline__ float finish_site(const D32 &a, int64_t off, int s, i
         for (int i = 0; i < 12; ++i) acc[i] = fma2(dup(-al), acc[i], y[i * 16]);   // no read-only load: y may be out
     }
     if (EPI < QS_EPI_NORM || on) S::st(a.out + off, s, acc);
-    return EPI >= QS_EPI_NORM && on ? site_norm2(acc) : 0.f;
+    return EPI >= QS_EPI_NORM && on ? site_norm2(acc) : make_float2(0.f, 0.f);
 }
 
 // physical site p and its mirror, right-hand side r (one per warp); on = false: nothing is
@@ -520,8 +527,8 @@ __device__ __forceinline__ void site_kernel(const D32 &a, int p, int r, bool on 
     hop_begin<0>(a, c, h);
     S::fetch(in, h.n, v);
     hops<0, S>(a, c, in, h, v, acc, accm);
-    const float n2 = finish_site<S, EPI>(a, off, c.s, r, on, acc);
-    const float m2 = finish_site<S, EPI>(a, off, c.s + a.g.L, r, on, accm);
+    const cf n2 = finish_site<S, EPI>(a, off, c.s, r, on, acc);
+    const cf m2 = finish_site<S, EPI>(a, off, c.s + a.g.L, r, on, accm);
     if (EPI >= QS_EPI_NORM) {   // two shares per 32 physical sites, the ones that one_kernel leaves
         double *sh = a.part + (int64_t)r * a.ntile + 2 * (p / 32);
         warp_share(n2, sh);
@@ -555,7 +562,7 @@ __device__ __forceinline__ void one_kernel(const D32 &a, int p, int r, bool mir,
     hop_begin<0>(a, c, h);
     S::fetch(in, mir ? h.nm : h.n, v);
     hops_one<0, S>(a, c, in, mir, mir ? -1.f : 1.f, h, v, acc);
-    const float n2 = finish_site<S, EPI>(a, off, s, r, on, acc);
+    const cf n2 = finish_site<S, EPI>(a, off, s, r, on, acc);
     if (EPI >= QS_EPI_NORM) warp_share(n2, a.part + (int64_t)r * a.ntile + 2 * (p / 32) + (mir ? 1 : 0));
 }
 

@@ -129,3 +129,23 @@ def test_chebyshev_step(lib, shape):
                 assert np.abs(got - ref).max() <= tol * np.abs(ref).max(), storage
             assert torch.equal(out, first), (variant, storage)
     lat.close()
+
+
+@pytest.mark.parametrize("shape", SHAPES + [(8, 8, 0b111, False, 3)], ids=str)
+def test_shares_against_64_bits(lib, shape):
+    """The shares' sum against the FP64 sum of the stored outputs' squares to 4e-12: the high parts
+    of a site's 24 squares and of a warp's 32 sites are summed without error, and the low parts,
+    at most 18 roundings of 2^-24 of the sum, in at most 54 FP32 operations: 972 x 2^-48."""
+    import torch
+    qs, lat, cfg, n, v, dev = problem(shape)
+    ns, nt = cfg.n_sites, lib.t_ntile(lat.h)
+    x, y = [qs.to_tiled(t, ns) for t in dev[:2]]
+    alpha = torch.linspace(-0.8, 1.3, n, device="cuda")
+    for variant in (1, 5):
+        for epi in (NORM, RESID):
+            out = y.clone()
+            part = torch.zeros((n, nt), dtype=torch.float64, device="cuda")
+            call(lib, lat, variant, F32, epi, n, x, out, y=out if epi == RESID else None, alpha=alpha, part=part)
+            want = (out.reshape(n, -1).double() ** 2).sum(1)
+            assert bool(((part.sum(1) - want).abs() <= 4e-12 * want).all()), (variant, epi, (part.sum(1) / want - 1).tolist())
+    lat.close()
