@@ -1,6 +1,7 @@
 // Vector, block and reduction kernels of the eigensolver and the CG.
-// Reductions are two-stage with a fixed grid (QS_RED_BLOCKS partials per
-// vector, then one fixed-order pass), so results are bit-reproducible.
+// Reductions are two-stage: partial sums of a grid that depends on the vector's length alone
+// (red_blocks), then one fixed-order pass.  So results are bit-reproducible, and a vector's sum
+// does not depend on how many others it is summed with.
 #include "blas.cuh"
 
 #include <mutex>
@@ -52,10 +53,9 @@ __device__ __forceinline__ float4 diff(float4 a, float t, float4 b)
 }
 __device__ __forceinline__ double2 diff(double2 a, double t, double2 b) { return make_double2(fma(-t, b.x, a.x), fma(-t, b.y, a.y)); }
 
-// Streaming kernels over [k][nr]: 16-byte words (nr is a multiple of 24 x 16), blocks of
-// red_blocks(nr, k) per vector, so that a block has some two thousand reals to itself; with 608
-// blocks per vector whatever its length, an 8^3 x 12 CG update of 16 vectors was 9728 blocks of
-// two reals per thread and took 69 us instead of 15.  FP32 sums are kept as a two-sum pair.
+// Streaming kernels over [k][nr]: 16-byte words (nr is a multiple of 24 x 16), red_blocks(nr) blocks
+// per vector, so that a block has some two thousand reals to itself; with 608 blocks per vector
+// whatever its length a thread of an 8^3 x 12 problem has two.  FP32 sums are kept as a two-sum pair.
 template <typename R>
 __global__ void __launch_bounds__(256) norm2_part(const R *__restrict__ v, int64_t nr, double *part)
 {
@@ -517,13 +517,20 @@ __global__ void cg_init_kernel(CgScalars s, const double *rr, int k)
     s.live[q] = rr[q] > 0;
 }
 
-// blocks per vector of the reductions: two to eight per SM over the k vectors
-inline int red_blocks(int64_t nr, int k)
+// blocks per vector of the reductions, from the length alone: a count that fell with k (two to eight
+// blocks per SM over all k vectors) made a vector's sum depend on its neighbours, and at k = 64
+// each thread added thousands of terms in sequence
+inline int red_blocks(int64_t nr)
 {
-    int64_t b = nr / 2048, top = 1216 / k;
-    if (b > top) b = top;
-    if (b > QS_RED_BLOCKS) b = QS_RED_BLOCKS;
-    return b < 1 ? 1 : (int)b;
+    const int64_t b = nr / 2048;
+    return b < 1 ? 1 : b > QS_RED_BLOCKS ? QS_RED_BLOCKS : (int)b;
+}
+
+// blocks per vector of the streaming updates: two to eight per SM over the k vectors
+inline int stream_blocks(int64_t nr, int k)
+{
+    const int64_t b = red_blocks(nr), top = 1216 / k;
+    return (int)(b < top ? b : top);
 }
 
 inline int grid_for(int64_t n, int per = 256)
@@ -537,7 +544,7 @@ inline int grid_for(int64_t n, int per = 256)
 template <typename R>
 cudaError_t qs_norm2(const R *v, int k, int64_t nr, double *part, double *out, cudaStream_t st)
 {
-    const int nb = red_blocks(nr, k);
+    const int nb = red_blocks(nr);
     norm2_part<R><<<dim3(nb, k), 256, 0, st>>>(v, nr, part);
     finalize_sum<<<k, 256, 0, st>>>(part, nb, 1, out);
     qs_note_launches(2);
@@ -550,7 +557,7 @@ template <typename R>
 cudaError_t qs_resid2(const R *a, const R *b, const double *theta, int k, int64_t nr,
                       double *part, double *out, cudaStream_t st)
 {
-    const int nb = red_blocks(nr, k);
+    const int nb = red_blocks(nr);
     resid_part<R><<<dim3(nb, k), 256, 0, st>>>(a, b, theta, nr, part);
     finalize_sum<<<k, 256, 0, st>>>(part, nb, 1, out);
     qs_note_launches(2);
@@ -725,7 +732,7 @@ cudaError_t qs_cg_beta_xp(float *x, float *p, const float *r, const CgScalars &s
                           const double *part, int nb, cudaStream_t st)
 {
     cg_beta_kernel<<<k, 256, 0, st>>>(s, part, nb, tol2);
-    cg_xp_kernel<<<dim3(red_blocks(nr, k), k), 256, 0, st>>>((float4 *)x, (float4 *)p, (const float4 *)r, s, nr / 4);
+    cg_xp_kernel<<<dim3(stream_blocks(nr, k), k), 256, 0, st>>>((float4 *)x, (float4 *)p, (const float4 *)r, s, nr / 4);
     qs_note_launches(2);
     return cudaGetLastError();
 }

@@ -1,0 +1,33 @@
+"""Norms of block vectors: a vector's norm is the same, bit for bit, alone and in a block of any
+size (through the public allocation-free entry, whose output is the same in both)."""
+import numpy as np
+import pytest
+
+from synth_inputs import make_config
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("dtype", ["float32", "float64"])
+@pytest.mark.parametrize("L,T", [(2, 3), (4, 6), (8, 8), (12, 12)])
+def test_norm_does_not_depend_on_the_block(L, T, dtype):
+    import torch
+    import paper_2108_11989_gb300 as qs
+    cfg = make_config(T=T, L=L, eps=0.4, theta_sigma=0.3, csw_su3=1.9, csw_u1=1.0, seed=5)
+    lat = qs.Lattice(L, T)
+    lat.load_gauge(cfg.su3, cfg.theta, cfg.csw_su3, cfg.csw_u1)
+    g = torch.Generator(device="cuda")
+    g.manual_seed(1)
+    x = torch.randn((64, cfg.n_sites * 24), dtype=getattr(torch, dtype), device="cuda", generator=g)
+    norms = {}
+    for n in (1, 3, 16, 64):
+        out = torch.empty_like(x[:n])
+        nrm = torch.empty(n, dtype=torch.float64, device="cuda")
+        qs.apply_Q_norm2_noalloc(lat.h, -0.1, x[:n], out, nrm)
+        torch.cuda.synchronize()
+        norms[n] = nrm.cpu().numpy()
+        want = (out.double() ** 2).sum(1).cpu().numpy()
+        assert np.all(np.abs(norms[n] - want) <= 1e-6 * want)
+    for n in (1, 3, 16):
+        assert np.array_equal(norms[n], norms[64][:n]), (n, norms[n] / norms[64][:n] - 1)
+    lat.close()
