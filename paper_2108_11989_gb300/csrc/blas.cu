@@ -41,6 +41,9 @@ __device__ __forceinline__ void two_sum_acc(float &hi, float &lo, float x)
     lo += err;
 }
 __device__ __forceinline__ void two_sum_acc(double &hi, double &, double x) { hi += x; }
+// the pair's value; a sum that has left the range is infinite (its error term is then NaN)
+__device__ __forceinline__ double pair_value(float hi, float lo) { return isinf(hi) ? (double)hi : (double)hi + (double)lo; }
+__device__ __forceinline__ double pair_value(double hi, double) { return hi; }
 
 template <typename R> struct Vec16;   // 16 bytes of reals
 template <> struct Vec16<float> { typedef float4 T; };
@@ -65,7 +68,7 @@ __global__ void __launch_bounds__(256) norm2_part(const R *__restrict__ v, int64
     R acc = 0, lo = 0;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
         two_sum_acc(acc, lo, sum_sq(x[i]));
-    double s = block_sum((double)acc + (double)lo);
+    double s = block_sum(pair_value(acc, lo));
     if (threadIdx.x == 0) part[blockIdx.y * gridDim.x + blockIdx.x] = s;
 }
 
@@ -91,7 +94,7 @@ __global__ void __launch_bounds__(256) resid_part(const R *__restrict__ a, const
     R acc = 0, lo = 0;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
         two_sum_acc(acc, lo, sum_sq(diff(x[i], t, y[i])));
-    double s = block_sum((double)acc + (double)lo);
+    double s = block_sum(pair_value(acc, lo));
     if (threadIdx.x == 0) part[blockIdx.y * gridDim.x + blockIdx.x] = s;
 }
 

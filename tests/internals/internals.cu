@@ -37,6 +37,15 @@ QS_API int t_norm2(qs_lattice *lat, int f64, const void *v, int k, int64_t nr, d
     return QS_OK;
 }
 
+// |a_r - theta_r b_r|^2 of k pairs of FP32 device vectors of nr reals
+QS_API int t_resid2(qs_lattice *lat, const float *a, const float *b, const double *theta, int k, int64_t nr, double *part,
+                    double *out)
+{
+    CK(qs_resid2<float>(a, b, theta, k, nr, part, out, lat->stream));
+    CK(cudaStreamSynchronize(lat->stream));
+    return QS_OK;
+}
+
 // FP32 CG on Q(m0)^2 for the k device vectors b (solver layout); counts: f32_count, cg_count, iterations
 QS_API int t_cg(qs_lattice *lat, int k, double m0, double tol, int maxit, const float *b, float *x, int64_t *counts)
 {

@@ -31,3 +31,34 @@ def test_norm_does_not_depend_on_the_block(L, T, dtype):
     for n in (1, 3, 16):
         assert np.array_equal(norms[n], norms[64][:n]), (n, norms[n] / norms[64][:n] - 1)
     lat.close()
+
+
+def sums(v, theta=None, b=None):
+    """|v_r|^2, or |v_r - theta_r b_r|^2, of FP32 vectors by the solver's reductions."""
+    import torch
+    import internals
+    import paper_2108_11989_gb300 as qs
+    lib, lat = internals.load(), qs.Lattice(2, 2)
+    k, nr = v.shape
+    part = torch.full((k, 608), float("nan"), dtype=torch.float64, device="cuda")
+    out = torch.full((k,), float("nan"), dtype=torch.float64, device="cuda")
+    torch.cuda.synchronize()
+    if b is None:
+        s = lib.t_norm2(lat.h, 0, v.data_ptr(), k, nr, part.data_ptr(), out.data_ptr())
+    else:
+        s = lib.t_resid2(lat.h, v.data_ptr(), b.data_ptr(), theta.data_ptr(), k, nr, part.data_ptr(), out.data_ptr())
+    assert s == 0
+    lat.close()
+    return out.cpu().numpy()
+
+
+def test_sum_beyond_the_range_is_infinite():
+    """Squares whose FP32 sum overflows: infinity (which the solver reports), never NaN (whose square
+    root it would take for a zero residual)."""
+    import torch
+    v = torch.zeros((3, 4608), device="cuda")
+    v[1] = 1.5e19          # each square is a number, their sums are not
+    v[2, 17] = 1e30
+    zero, theta = torch.zeros_like(v), torch.zeros(3, dtype=torch.float64, device="cuda")
+    for got in (sums(v), sums(v, theta, zero)):
+        assert got[0] == 0 and np.isposinf(got[1:]).all(), got
