@@ -48,8 +48,24 @@ __device__ __forceinline__ double pair_value(double hi, double) { return hi; }
 template <typename R> struct Vec16;   // 16 bytes of reals
 template <> struct Vec16<float> { typedef float4 T; };
 template <> struct Vec16<double> { typedef double2 T; };
-__device__ __forceinline__ float sum_sq(float4 a) { return fmaf(a.w, a.w, fmaf(a.z, a.z, fmaf(a.y, a.y, a.x * a.x))); }
-__device__ __forceinline__ double sum_sq(double2 a) { return fma(a.y, a.y, a.x * a.x); }
+// (hi, lo) += the squares of a word's reals.  FP32: exact squares by fused multiply-adds and two-sum
+// (hi + a a = s + e with s rounded, b = s - hi, e = (a a - b) + (hi - (s - b))); a plain chain of the
+// word's four is about twice as far from the 64-bit sum on 4^4 to 6^3 x 8 as one or two squares per
+// thread are
+__device__ __forceinline__ void add_sq(float &hi, float &lo, float a)
+{
+    const float s = fmaf(a, a, hi), nb = hi - s;
+    lo += fmaf(a, a, nb) + (hi - (s + nb));
+    hi = s;
+}
+__device__ __forceinline__ void add_sq(float &hi, float &lo, float4 a)
+{
+    add_sq(hi, lo, a.x);
+    add_sq(hi, lo, a.y);
+    add_sq(hi, lo, a.z);
+    add_sq(hi, lo, a.w);
+}
+__device__ __forceinline__ void add_sq(double &hi, double &, double2 a) { hi += fma(a.y, a.y, a.x * a.x); }
 __device__ __forceinline__ float4 diff(float4 a, float t, float4 b)
 {
     return make_float4(fmaf(-t, b.x, a.x), fmaf(-t, b.y, a.y), fmaf(-t, b.z, a.z), fmaf(-t, b.w, a.w));
@@ -67,7 +83,7 @@ __global__ void __launch_bounds__(256) norm2_part(const R *__restrict__ v, int64
     const T *x = reinterpret_cast<const T *>(v) + (int64_t)blockIdx.y * n;
     R acc = 0, lo = 0;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        two_sum_acc(acc, lo, sum_sq(x[i]));
+        add_sq(acc, lo, x[i]);
     double s = block_sum(pair_value(acc, lo));
     if (threadIdx.x == 0) part[blockIdx.y * gridDim.x + blockIdx.x] = s;
 }
@@ -93,7 +109,7 @@ __global__ void __launch_bounds__(256) resid_part(const R *__restrict__ a, const
     const R t = (R)theta[blockIdx.y];
     R acc = 0, lo = 0;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        two_sum_acc(acc, lo, sum_sq(diff(x[i], t, y[i])));
+        add_sq(acc, lo, diff(x[i], t, y[i]));
     double s = block_sum(pair_value(acc, lo));
     if (threadIdx.x == 0) part[blockIdx.y * gridDim.x + blockIdx.x] = s;
 }

@@ -62,3 +62,23 @@ def test_sum_beyond_the_range_is_infinite():
     zero, theta = torch.zeros_like(v), torch.zeros(3, dtype=torch.float64, device="cuda")
     for got in (sums(v), sums(v, theta, zero)):
         assert got[0] == 0 and np.isposinf(got[1:]).all(), got
+
+
+@pytest.mark.parametrize("L,T", [(2, 3), (4, 4), (4, 8), (6, 8), (8, 12)])
+def test_fp32_sums_against_64_bits(L, T):
+    """FP32 vectors' norms and residuals to 3e-12 of the FP64 sum of the same squares: a thread adds
+    at most 16 squares, the high parts without error, the low parts (16 x 2^-24 of the sum at most)
+    in 48 FP32 operations: 768 x 2^-48; the threads' sums are added in FP64."""
+    import torch
+    g = torch.Generator(device="cuda")
+    g.manual_seed(L * T)
+    v = torch.randn((4, 2 * L ** 3 * T * 24), device="cuda", generator=g)
+    b = torch.randn(v.shape, device="cuda", generator=g)
+    want = (v.double() ** 2).sum(1).cpu().numpy()
+    got = sums(v)
+    assert np.all(np.abs(got - want) <= 3e-12 * want), got / want - 1
+    theta = torch.tensor([0.0, 1.0, 0.5, -2.0], dtype=torch.float64, device="cuda")
+    d = (v.double() - theta[:, None] * b.double()).float()   # one rounding, as a fused multiply-add has
+    want = (d.double() ** 2).sum(1).cpu().numpy()
+    got = sums(v, theta, b)
+    assert np.all(np.abs(got - want) <= 3e-12 * want), got / want - 1
