@@ -608,9 +608,19 @@ cudaError_t launch_one(const D32 &a, cudaStream_t st)
     return cudaGetLastError();
 }
 
-// Batched persistent form: work items (lattice i, site tile, right-hand side) numbered
-// lattice by lattice, right-hand sides fastest; each block takes items w = blockIdx.x,
-// blockIdx.x + gridDim.x, ...
+// Batched form: work items (lattice i, tile of physical sites, right-hand side) numbered lattice by
+// lattice, right-hand sides fastest.  Large batches are persistent: each block takes items
+// w = blockIdx.x, blockIdx.x + gridDim.x, ... of 128 sites.  Small ones launch a block per item of 32
+// sites, as dslash32_one_kernel.
+#define QS_BATCH_TILE 128     // physical sites per work item
+#define QS_BATCH_ONE_TILE 32
+// Physical sites x right-hand sides of a batch up to which a block per 32 sites and its mirrors is the
+// faster form: below it the pair threads do not fill the chip, and their chain is the time.
+// Device time, in a graph: two 4^3 x 3 of one vector, FP32, 5.7 -> 4.1 us and FP16 6.0 -> 4.0; 4^3 x 4, 6^3 x 5
+// and 8^3 x 8 of 3, 5 and 2 vectors 7.0 -> 5.2; even at 32 k (two 8^3 x 8 of 4 vectors: 8.1 and 7.9, FP16 7.9
+// and 7.8), slower at 49 k (10.7 against 11.4 us).
+#define QS_BATCH_ONE_MAX 32768
+
 struct D32B {
     int n;
     unsigned off[QS_BATCH_MAX + 1];   // first work item of lattice i; off[n] = all items
@@ -627,9 +637,21 @@ __global__ void __launch_bounds__(128, 3) dslash32_batch_kernel(const __grid_con
 #pragma unroll 1
         while (i + 1 < b.n && w >= b.off[i + 1]) ++i;
         const unsigned local = w - b.off[i];
-        const int p = (int)(local / (unsigned)b.item[i].nrhs) * 128 + (int)threadIdx.x;
+        const int p = (int)(local / (unsigned)b.item[i].nrhs) * QS_BATCH_TILE + (int)threadIdx.x;
         if (p < (int)b.item[i].g.Vphys) site_kernel<S, QS_EPI_PLAIN>(b.item[i], p, (int)(local % (unsigned)b.item[i].nrhs));
     }
+}
+
+template <class S>
+__global__ void __launch_bounds__(64, 8) dslash32_batch_one_kernel(const __grid_constant__ D32B b)
+{
+    int i = 0;
+#pragma unroll 1
+    while (i + 1 < b.n && blockIdx.x >= b.off[i + 1]) ++i;
+    const D32 &a = b.item[i];
+    const unsigned local = blockIdx.x - b.off[i], nrhs = (unsigned)a.nrhs;
+    const int p = (int)(local / nrhs) * 32 + (int)(threadIdx.x & 31);
+    if (p < (int)a.g.Vphys) one_kernel<S, QS_EPI_PLAIN>(a, p, (int)(local % nrhs), threadIdx.x >= 32, true);
 }
 
 // ---- conversions between tiled storages (per right-hand side and site) -----------
@@ -727,8 +749,12 @@ cudaError_t launch_storage(int v, int epi, const D32 &a, cudaStream_t st)
 }
 
 template <class S>
-cudaError_t batch_launch(const D32B &b, cudaStream_t st)
+cudaError_t batch_launch(const D32B &b, bool one, cudaStream_t st)
 {
+    if (one) {
+        dslash32_batch_one_kernel<S><<<b.off[b.n], 64, 0, st>>>(b);
+        return cudaGetLastError();
+    }
     static int per_sm = 0, nsm = 0;
     static std::once_flag once;
     std::call_once(once, [] {
@@ -753,6 +779,10 @@ cudaError_t qs_d32_batch_launch(const D32BatchItem *items, int n, int storage, i
     D32B b;
     memset(&b, 0, sizeof(b));
     b.n = n;
+    int64_t work = 0;
+    for (int i = 0; i < n; ++i) work += items[i].g.Vphys * items[i].nrhs;
+    const bool one = work <= QS_BATCH_ONE_MAX;
+    const int tile = one ? QS_BATCH_ONE_TILE : QS_BATCH_TILE;
     unsigned off = 0;
     for (int i = 0; i < n; ++i) {
         D32 &a = b.item[i];
@@ -774,17 +804,17 @@ cudaError_t qs_d32_batch_launch(const D32BatchItem *items, int n, int storage, i
         a.ntile = 0;
         for (int r = 0; r < it.nrhs; ++r) a.dm[r] = (float)(4.0 + it.m0[r]);
         b.off[i] = off;
-        const double items_i = (double)((it.g.Vphys + 127) / 128) * it.nrhs;
+        const double items_i = (double)((it.g.Vphys + tile - 1) / tile) * it.nrhs;
         if (off + items_i > 4e9) return cudaErrorInvalidValue;
         off += (unsigned)items_i;
     }
     b.off[n] = off;
     cudaError_t e;
     switch (storage) {
-    case QS_D32_F32_TILED: e = batch_launch<StF32Tiled>(b, st); break;
-    case QS_D32_F32_CANON: e = batch_launch<StF32Canon>(b, st); break;
-    case QS_D32_F16: e = batch_launch<StF16>(b, st); break;
-    case QS_D32_BF16: e = batch_launch<StBF16>(b, st); break;
+    case QS_D32_F32_TILED: e = batch_launch<StF32Tiled>(b, one, st); break;
+    case QS_D32_F32_CANON: e = batch_launch<StF32Canon>(b, one, st); break;
+    case QS_D32_F16: e = batch_launch<StF16>(b, one, st); break;
+    case QS_D32_BF16: e = batch_launch<StBF16>(b, one, st); break;
     default: return cudaErrorInvalidValue;
     }
     qs_note_launches(1);
