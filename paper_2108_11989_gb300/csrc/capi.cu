@@ -378,7 +378,7 @@ int qs_d32_call(qs_lattice *lat, const D32Call &c)
         int v = tune_lookup(key);
         if (v < 0 || v >= qs_d32_nvariants()) {
             if (capturing(lat->stream) || c.epi == QS_EPI_RESID) {
-                v = 1;   // no timing inside a capture: a fixed variant
+                v = qs_d32_fixed_variant(c.g, nrhs);   // no timing inside a capture
             } else {
                 // timing writes `out` only (in, y and x are read): harmless to the caller
                 int st = QS_OK;

@@ -75,6 +75,7 @@ struct D32Call {
     const int *live;       // NORM, RESID: NULL, or device flags: right-hand sides with 0 are skipped
 };
 int qs_d32_nvariants();
+int qs_d32_fixed_variant(const Geom &g, int nrhs);   // where the variants cannot be timed
 int64_t qs_d32_ntile(const Geom &g);
 int64_t qs_d32_vec_bytes(int storage, int64_t Ns);
 cudaError_t qs_d32_launch(const D32Call &c, int variant, cudaStream_t st);

@@ -614,12 +614,12 @@ cudaError_t launch_one(const D32 &a, cudaStream_t st)
 // sites, as dslash32_one_kernel.
 #define QS_BATCH_TILE 128     // physical sites per work item
 #define QS_BATCH_ONE_TILE 32
-// Physical sites x right-hand sides of a batch up to which a block per 32 sites and its mirrors is the
-// faster form: below it the pair threads do not fill the chip, and their chain is the time.
-// Device time, in a graph: two 4^3 x 3 of one vector, FP32, 5.7 -> 4.1 us and FP16 6.0 -> 4.0; 4^3 x 4, 6^3 x 5
+// Physical sites x right-hand sides up to which a block per 32 sites and its mirrors is the faster
+// form, of a batch and of a single launch whose variants are not timed: below it the pair threads do
+// not fill the chip, and their chain is the time.  Batches: device time, in a graph: two 4^3 x 3 of one vector, FP32, 5.7 -> 4.1 us and FP16 6.0 -> 4.0; 4^3 x 4, 6^3 x 5
 // and 8^3 x 8 of 3, 5 and 2 vectors 7.0 -> 5.2; even at 32 k (two 8^3 x 8 of 4 vectors: 8.1 and 7.9, FP16 7.9
 // and 7.8), slower at 49 k (10.7 against 11.4 us).
-#define QS_BATCH_ONE_MAX 32768
+#define QS_ONE_MAX 32768
 
 struct D32B {
     int n;
@@ -781,7 +781,7 @@ cudaError_t qs_d32_batch_launch(const D32BatchItem *items, int n, int storage, i
     b.n = n;
     int64_t work = 0;
     for (int i = 0; i < n; ++i) work += items[i].g.Vphys * items[i].nrhs;
-    const bool one = work <= QS_BATCH_ONE_MAX;
+    const bool one = work <= QS_ONE_MAX;
     const int tile = one ? QS_BATCH_ONE_TILE : QS_BATCH_TILE;
     unsigned off = 0;
     for (int i = 0; i < n; ++i) {
@@ -824,6 +824,11 @@ cudaError_t qs_d32_batch_launch(const D32BatchItem *items, int n, int storage, i
 int64_t qs_d32_ntile(const Geom &g) { return 2 * ((g.Vphys + 31) / 32); }
 
 int qs_d32_nvariants() { return 7; }
+
+// Device time of an application in FP32 and FP16, thread per site against variant 1: 4^3 x 4, one vector,
+// 3.8 and 3.9 us against 5.2 and 5.7; 6^3 x 6, 3 vectors, 4.0 and 4.3 against 6.1 and 6.6; 8^3 x 8, 4 vectors,
+// 5.3 and 5.3 against 6.7 and 7.0.
+int qs_d32_fixed_variant(const Geom &g, int nrhs) { return g.Vphys * nrhs <= QS_ONE_MAX ? 5 : 1; }
 
 int64_t qs_d32_vec_bytes(int storage, int64_t Ns)
 {

@@ -52,7 +52,7 @@ static int run(qs_lattice *lat, double m0, const void *in, void *out, int nrhs, 
         c.gamma5 = 1;
         c.m0 = m;
         const int tv = lat->tuned32[QS_D32_F32_CANON][0][nrhs];
-        QS_CUDA(qs_d32_launch(c, tv > 0 ? tv - 1 : 1, lat->stream));
+        QS_CUDA(qs_d32_launch(c, tv > 0 ? tv - 1 : qs_d32_fixed_variant(c.g, nrhs), lat->stream));
     }
     qs_note_launches(1);
     QS_CUDA(qs_norm2<R>((const R *)out, nrhs, lat->g.Ns * 24, scratch, norm2, lat->stream));

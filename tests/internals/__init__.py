@@ -24,7 +24,8 @@ def load():
         subprocess.run([b.NVCC, *b.ARCH, "-shared", "-o", so, obj, *objs], check=True)
     lib = ctypes.CDLL(so)
     P, I, D, L = ctypes.c_void_p, ctypes.c_int, ctypes.c_double, ctypes.c_int64
-    for name, args in {"t_ntile": [P], "t_nvariants": [], "t_d32": [P, I, I, I, I, D, P, P, P, P, D, D, D, P, P, P],
+    for name, args in {"t_ntile": [P], "t_nvariants": [], "t_fixed_variant": [P, I],
+                      "t_d32": [P, I, I, I, I, D, P, P, P, P, D, D, D, P, P, P],
                        "t_norm2": [P, I, P, I, L, P, P], "t_resid2": [P, P, P, P, I, L, P, P],
                        "t_cg": [P, I, D, D, I, P, P, P],
                        "t_rr32": [P, I, D, P, P, P]}.items():

@@ -8,6 +8,8 @@ extern "C" {
 QS_API int64_t t_ntile(qs_lattice *lat) { return qs_d32_ntile(lat->g); }
 QS_API int t_nvariants() { return qs_d32_nvariants(); }
 
+QS_API int t_fixed_variant(qs_lattice *lat, int nrhs) { return qs_d32_fixed_variant(lat->g, nrhs); }
+
 // one launch of the FP32-arithmetic operator Q with a given variant and epilogue
 QS_API int t_d32(qs_lattice *lat, int variant, int storage, int epi, int nrhs, double m0, const void *in, void *out,
                  const void *y, const void *x, double c, double s1, double s2, const float *alpha, const int *live,
