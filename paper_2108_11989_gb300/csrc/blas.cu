@@ -507,6 +507,7 @@ __global__ void __launch_bounds__(256) cg_beta_kernel(CgScalars s, const double 
     if (threadIdx.x != 0) return;
     s.beta[q] = s.rr[q] > 0 ? (float)(acc / s.rr[q]) : 0.f;
     s.rr[q] = acc;
+    ++s.iters[q];
     s.live[q] = acc > tol2 * s.rr0[q] && isfinite(acc);
 }
 
@@ -534,6 +535,7 @@ __global__ void cg_init_kernel(CgScalars s, const double *rr, int k)
     s.rr[q] = rr[q];
     s.rr0[q] = rr[q];
     s.live[q] = rr[q] > 0;
+    s.iters[q] = 0;
 }
 
 // blocks per vector of the reductions, from the length alone: a count that fell with k (two to eight

@@ -62,7 +62,7 @@ cudaError_t qs_herm_eig2(const double2 *H0, double *ev0, int *info0, const doubl
 struct CgScalars {
     double *rr, *rr0;
     float *alpha, *beta;
-    int *live;
+    int *live, *iters;   // still iterating; iterations done
 };
 // part: [k][nb] shares of |Q p|^2 (alpha), of |r|^2 (beta)
 cudaError_t qs_cg_alpha(const CgScalars &s, int k, const double *part, int nb, cudaStream_t st);

@@ -305,6 +305,11 @@ int qs_prof_end(qs_lattice *lat, cudaEvent_t ea, cudaEvent_t eb, int prec, doubl
     return QS_OK;
 }
 
+void qs_prof_skipped(qs_lattice *lat, int prec, double bytes)
+{
+    if (lat->prof && lat->prof->on) lat->prof->acc.dslash[prec].bytes -= bytes;
+}
+
 static int run64(qs_lattice *lat, const double *m0, const void *in, void *out, int nrhs, int gamma5, int soa)
 {
     DslashArgs<double> d = make_args64(lat, m0, in, out, nrhs, gamma5);

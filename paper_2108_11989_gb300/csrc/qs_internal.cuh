@@ -162,4 +162,6 @@ int qs_d32_run(qs_lattice *lat, int storage, const double *m0, const void *in, v
                const float *dm_dev = nullptr);
 // record one profiling interval covering `launches` operator launches (graph replays)
 int qs_prof_begin(qs_lattice *lat, cudaEvent_t *ea, cudaEvent_t *eb);
+// take back bytes of recorded launches that skipped some of their right-hand sides
+void qs_prof_skipped(qs_lattice *lat, int prec, double bytes);
 int qs_prof_end(qs_lattice *lat, cudaEvent_t ea, cudaEvent_t eb, int prec, double bytes, int launches);

@@ -47,8 +47,8 @@ struct Workspace {
     double2 *G, *Rinv, *Hm, *Ym;
     double *ds;           // device scalars, S_NSLOT slots of 64
     double *cgpart;       // shares of the CG's sums, [k][qs_d32_ntile()]
-    int *di;              // device ints, 64 CG flags + 8
-    int *hlive;           // pinned: CG_LAG + 1 copies of the CG flags
+    int *di;              // device ints: 64 + 8 flags, then the CG's 64 live flags and 64 iteration counts
+    int *hlive;           // pinned: CG_LAG + 1 copies of the CG's flags and counts
     cudaEvent_t ev[CG_LAG + 1];
     double *hp;           // pinned host mirror of ds (S_NSLOT x 64)
     int *hi;              // pinned host ints (64 + 8)
@@ -113,14 +113,14 @@ static int ws_alloc(qs_lattice *lat, Workspace *w, int k)
     CK(cudaMalloc(&w->Hm, 64 * 64 * sizeof(double2)));
     CK(cudaMalloc(&w->Ym, 64 * 64 * sizeof(double2)));
     CK(cudaMalloc(&w->ds, S_NSLOT * 64 * sizeof(double)));
-    CK(cudaMalloc(&w->di, 72 * sizeof(int)));
+    CK(cudaMalloc(&w->di, (72 + 128) * sizeof(int)));
     CK(cudaMallocHost(&w->hp, S_NSLOT * 64 * sizeof(double)));
     CK(cudaMallocHost(&w->hi, 72 * sizeof(int)));
-    CK(cudaMallocHost(&w->hlive, (CG_LAG + 1) * 64 * sizeof(int)));
+    CK(cudaMallocHost(&w->hlive, (CG_LAG + 1) * 128 * sizeof(int)));
     for (auto &e : w->ev) CK(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
     CK(cudaMalloc(&w->coef_dev, (3 * QS_GRAPH_MAX_DEG + 64) * sizeof(float)));
     CK(cudaMallocHost(&w->coef_host, (3 * QS_GRAPH_MAX_DEG + 64) * sizeof(float)));
-    CK(cudaMemsetAsync(w->di, 0, 72 * sizeof(int), lat->stream));
+    CK(cudaMemsetAsync(w->di, 0, (72 + 128) * sizeof(int), lat->stream));
     for (int i = 0; i < 64; ++i) w->hp[i] = 1.0;
     CK(cudaMemcpyAsync(DS(w, S_ONES), w->hp, 64 * sizeof(double), cudaMemcpyHostToDevice, lat->stream));
     CK(cudaStreamSynchronize(lat->stream));
@@ -455,7 +455,8 @@ static int cheb_filter64(qs_lattice *lat, Workspace *w, double m0, int k, int d,
 // FP32 CG on Q^2 for k right-hand sides in r (overwritten); solution in x.  The host never waits
 // for an iteration it has just launched: every CG_POLL iterations it copies the flags of the
 // vectors that still iterate, and it reads a copy CG_LAG copies later; by then all kernels skip
-// the vectors that have converged, the operator among them.
+// the vectors that have converged, the operator among them.  *iters is the iteration at which the
+// last vector converged, and the counters hold the work done, not the skipped.
 static int cg_f32(qs_lattice *lat, Workspace *w, double m0, int k, float *x, float *r, float *p, float *t,
                   double tol, int maxit, int *iters)
 {
@@ -463,7 +464,7 @@ static int cg_f32(qs_lattice *lat, Workspace *w, double m0, int k, float *x, flo
     CgScalars s;
     s.rr = DS(w, S_RR); s.rr0 = DS(w, S_RR0);
     s.alpha = (float *)DS(w, S_AB); s.beta = s.alpha + 64;
-    s.live = w->di;
+    s.live = w->di + 72; s.iters = s.live + 64;
     size_t bytes = (size_t)k * w->nr * sizeof(float);
     CK(cudaMemsetAsync(x, 0, bytes, st));
     CK(cudaMemcpyAsync(p, r, bytes, cudaMemcpyDeviceToDevice, st));
@@ -481,7 +482,7 @@ static int cg_f32(qs_lattice *lat, Workspace *w, double m0, int k, float *x, flo
     D32Call c2 = c;
     c.epi = QS_EPI_NORM; c.in = p; c.out = t;              // t = Q p
     c2.epi = QS_EPI_RESID; c2.in = t; c2.y = r; c2.out = r;   // r -= alpha Q t
-    int it = 0, polls = 0, seen = 0;
+    int it = 0, polls = 0, seen = 0, last = 0;
     bool done = false;
     while (it < maxit && !done) {
         QS_TRY(qs_d32_call(lat, c));
@@ -491,19 +492,32 @@ static int cg_f32(qs_lattice *lat, Workspace *w, double m0, int k, float *x, flo
         ++it;
         if (it % CG_POLL == 0 || it == maxit) {
             const int slot = polls++ % (CG_LAG + 1);
-            CK(cudaMemcpyAsync(w->hlive + 64 * slot, s.live, k * sizeof(int), cudaMemcpyDeviceToHost, st));
+            CK(cudaMemcpyAsync(w->hlive + 128 * slot, s.live, 128 * sizeof(int), cudaMemcpyDeviceToHost, st));
             CK(cudaEventRecord(w->ev[slot], st));
             if (polls - seen > CG_LAG) {
-                const int old = seen++ % (CG_LAG + 1);
-                CK(cudaEventSynchronize(w->ev[old]));
+                last = seen++ % (CG_LAG + 1);
+                CK(cudaEventSynchronize(w->ev[last]));
                 done = true;
-                for (int i = 0; i < k; ++i) done = done && !w->hlive[64 * old + i];
+                for (int i = 0; i < k; ++i) done = done && !w->hlive[128 * last + i];
             }
         }
     }
-    w->f32_count += 2 * (int64_t)k * it;
-    w->cg_count += it;
-    *iters = it;
+    if (!done && polls > 0) {   // the cap: the last copy holds the counts
+        last = (polls - 1) % (CG_LAG + 1);
+        CK(cudaEventSynchronize(w->ev[last]));
+    }
+    int64_t live = 0;   // iterations of all vectors
+    int top = 0;
+    for (int i = 0; i < k && polls > 0; ++i) {
+        const int n = w->hlive[128 * last + 64 + i];
+        live += n;
+        top = std::max(top, n);
+    }
+    // an iteration's two launches move five FP32 vectors per live right-hand side, and the fields twice
+    qs_prof_skipped(lat, QS_F32, (double)lat->g.Ns * (5.0 * 96 * ((double)k * it - live) + 2.0 * 72 * 4 * (it - top)));
+    w->f32_count += 2 * live;
+    w->cg_count += top;
+    *iters = top;
     return QS_OK;
 }
 
