@@ -121,25 +121,26 @@ __global__ void __launch_bounds__(256) resid_part(const R *__restrict__ a, const
 // reads feeds four complex multiply-adds.  The element classes of a tile are summed in
 // shared memory at the end, in a fixed order.  LOWP: values rounded to FP32, products
 // and the sum over one chunk in FP32 (packed, two per instruction), chunk sums in FP64.
-// herm: G is known to be Hermitian (A = B, or B = Q A with Q Hermitian): only the tiles of the
-// upper triangle are computed, and same = 1 stages the vectors of A = B once.  FP64 products
-// are bound by the FP64 pipe (12^3 x 24, 16 vectors: 1.85 -> 1.38 ms with 10 of 16 tiles), FP32
-// ones by issue and by the block's own reduction (8^3 x 12, 32 vectors: 134 -> 87 us with 36 of 64
-// tiles, two blocks per SM instead of four and one conversion per total).
+// herm (A = B): G is Hermitian, only the tiles of the upper triangle are computed and the vectors are
+// staged once.  FP64 products are bound by the FP64 pipe (12^3 x 24, 16 vectors: 1.85 -> 1.38 ms with
+// 10 of 16 tiles), FP32 ones by issue and by the block's own reduction (8^3 x 12, 32 vectors:
+// 134 -> 87 us with 36 of 64 tiles, two blocks per SM instead of four and one conversion per total).
+// V^H (Q V) is Hermitian only up to rounding, and its reader takes the mean of both triangles, which
+// halves the error's variance: it is computed whole.
 #define GE 64
 __device__ __forceinline__ float2 pk_fma(float a, float2 b, float2 c) { return __ffma2_rn(make_float2(a, a), b, c); }
 
 template <bool LOWP, typename TIn = double2>
 __global__ void __launch_bounds__(256, LOWP ? 2 : 1) gram_tile_kernel(const TIn *__restrict__ A_, int ka,
                                                            const TIn *__restrict__ B_, int kb, int64_t nc,
-                                                           double *part, int herm, int same)
+                                                           double *part, int herm)
 {
     typedef typename std::conditional<LOWP, float2, double2>::type V2;
     typedef typename std::conditional<LOWP, float, double>::type T;
     extern __shared__ __align__(16) unsigned char gsm_raw[];
     V2 *sv = reinterpret_cast<V2 *>(gsm_raw);
-    const int kk = same ? ka : ka + kb, row = kk + 1;   // padded row of one element
-    const int boff = same ? 0 : ka;
+    const int kk = herm ? ka : ka + kb, row = kk + 1;   // padded row of one element
+    const int boff = herm ? 0 : ka;
     const int ti_n = (ka + 3) / 4, tj_n = (kb + 3) / 4;
     const int ntile = herm ? ti_n * (ti_n + 1) / 2 : ti_n * tj_n;
     const int eg_n = 256 / ntile;                     // element classes (>= 1)
@@ -590,14 +591,13 @@ template cudaError_t qs_resid2<float>(const float *, const float *, const double
                                       cudaStream_t);
 
 template <bool LOWP, typename TIn>
-static cudaError_t gram_launch(const TIn *A, int ka, const TIn *B, int kb, int64_t nc, double *part, double2 *G, int herm,
+static cudaError_t gram_launch(const TIn *A, int ka, const TIn *B, int kb, int64_t nc, double *part, double2 *G,
                                cudaStream_t st)
 {
     if (ka < 1 || kb < 1 || ka > 64 || kb > 64) return cudaErrorInvalidValue;
-    const int same = A == B && ka == kb;
-    herm = ka == kb && (herm || same);
+    const int herm = A == B && ka == kb;
     const int tn = (ka + 3) / 4, ntile = herm ? tn * (tn + 1) / 2 : tn * ((kb + 3) / 4);
-    const size_t stage = (size_t)GE * ((same ? ka : ka + kb) + 1) * (LOWP ? sizeof(float2) : sizeof(double2));
+    const size_t stage = (size_t)GE * ((herm ? ka : ka + kb) + 1) * (LOWP ? sizeof(float2) : sizeof(double2));
     const size_t red = (size_t)ntile * 32 * sizeof(double);
     const size_t sm = stage > red ? stage : red;
     static std::once_flag attr;
@@ -606,18 +606,18 @@ static cudaError_t gram_launch(const TIn *A, int ka, const TIn *B, int kb, int64
     });
     const int64_t nch = (nc + GE - 1) / GE;
     const int nb = (int)(nch < QS_RED_BLOCKS / 2 ? nch : QS_RED_BLOCKS / 2), n = 2 * ka * kb;   // two blocks per SM
-    gram_tile_kernel<LOWP, TIn><<<nb, 256, sm, st>>>(A, ka, B, kb, nc, part, herm, same);
+    gram_tile_kernel<LOWP, TIn><<<nb, 256, sm, st>>>(A, ka, B, kb, nc, part, herm);
     gram_sum_kernel<<<(n + 31) / 32, 256, 0, st>>>(part, nb, n, kb, herm, reinterpret_cast<double *>(G));
     qs_note_launches(2);
     return cudaGetLastError();
 }
 
 cudaError_t qs_gram(const double *A, int ka, const double *B, int kb, int64_t nr, double *part,
-                    double2 *G, cudaStream_t st, int lowp, int herm)
+                    double2 *G, cudaStream_t st, int lowp)
 {
     const double2 *a = (const double2 *)A, *b = (const double2 *)B;
-    return lowp ? gram_launch<true, double2>(a, ka, b, kb, nr / 2, part, G, herm, st)
-                : gram_launch<false, double2>(a, ka, b, kb, nr / 2, part, G, herm, st);
+    return lowp ? gram_launch<true, double2>(a, ka, b, kb, nr / 2, part, G, st)
+                : gram_launch<false, double2>(a, ka, b, kb, nr / 2, part, G, st);
 }
 
 cudaError_t qs_rotate(const double *W, int ka, const double2 *C, int kc, int64_t nr, double *V, cudaStream_t st,
@@ -641,9 +641,9 @@ cudaError_t qs_rotate(const double *W, int ka, const double2 *C, int kc, int64_t
 
 // the same contractions on FP32 blocks (products and per-chunk sums in FP32)
 cudaError_t qs_gram32(const float *A, int ka, const float *B, int kb, int64_t nr, double *part, double2 *G,
-                      cudaStream_t st, int herm)
+                      cudaStream_t st)
 {
-    return gram_launch<true, float2>((const float2 *)A, ka, (const float2 *)B, kb, nr / 2, part, G, herm, st);
+    return gram_launch<true, float2>((const float2 *)A, ka, (const float2 *)B, kb, nr / 2, part, G, st);
 }
 
 cudaError_t qs_rotate32(const float *W, int ka, const double2 *C, int kc, int64_t nr, float *V, cudaStream_t st,

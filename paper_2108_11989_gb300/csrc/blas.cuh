@@ -13,16 +13,16 @@ cudaError_t qs_resid2(const R *a, const R *b, const double *theta, int k, int64_
                       double *part, double *out, cudaStream_t st);
 // G[i][j] = <A_i, B_j>, i < ka, j < kb, complex row-major [ka][kb] (FP64 vectors);
 // lowp: products and per-chunk sums in FP32, chunk sums accumulated in FP64
-// herm: G is Hermitian (implied by A == B): half of it is computed
+// A == B: half of the Hermitian G is computed
 cudaError_t qs_gram(const double *A, int ka, const double *B, int kb, int64_t nr, double *part,
-                    double2 *G, cudaStream_t st, int lowp = 0, int herm = 0);
+                    double2 *G, cudaStream_t st, int lowp = 0);
 // V_j = sum_i W_i C[i][j], j < kc (C complex row-major [ka][kc]); V must not alias W;
 // lowp: the k-term sums in FP32; upper: C[i][j] = 0 for i > j
 cudaError_t qs_rotate(const double *W, int ka, const double2 *C, int kc, int64_t nr, double *V,
                       cudaStream_t st, int lowp = 0, int upper = 0);
 // the Gram matrix and the rotation on FP32 blocks (FP32 products, FP64 Gram totals)
 cudaError_t qs_gram32(const float *A, int ka, const float *B, int kb, int64_t nr, double *part, double2 *G,
-                      cudaStream_t st, int herm = 0);
+                      cudaStream_t st);
 cudaError_t qs_rotate32(const float *W, int ka, const double2 *C, int kc, int64_t nr, float *V, cudaStream_t st,
                         int upper = 0);
 // y_r = (float)(x_r * scale[r])  (scale on device, may be NULL for 1)

@@ -245,7 +245,7 @@ static int rayleigh_ritz(qs_lattice *lat, Workspace *w, double m0, int k, Ritz *
     glow = glow || rlow;
     // the Q^2 Ritz values only place the filter interval: FP32 products always
     CK(qs_gram(w->blk64[1], k, w->blk64[1], k, w->nr, w->part, w->G, st, 1));
-    CK(qs_gram(w->blk64[0], k, w->blk64[1], k, w->nr, w->part, w->Hm, st, glow, 1));   // Q is Hermitian
+    CK(qs_gram(w->blk64[0], k, w->blk64[1], k, w->nr, w->part, w->Hm, st, glow));
     CK(qs_herm_eig2(w->G, DS(w, S_RN), w->di + 66, w->Hm, DS(w, S_THETA), w->Ym, w->di + 67, k, w->part, st));
     CK(qs_rotate(w->blk64[0], k, w->Ym, k, w->nr, w->blk64[2], st, rlow));
     CK(qs_rotate(w->blk64[1], k, w->Ym, k, w->nr, w->blk64[3], st, rlow));
@@ -309,7 +309,7 @@ static int rayleigh_ritz32(qs_lattice *lat, Workspace *w, double m0, int k, Ritz
     cudaStream_t st = lat->stream;
     QS_TRY(opQ(lat, w, QS_F32, m0, V32(w), QV32(w), k));
     CK(qs_gram32(QV32(w), k, QV32(w), k, w->nr, w->part, w->G, st));
-    CK(qs_gram32(V32(w), k, QV32(w), k, w->nr, w->part, w->Hm, st, 1));
+    CK(qs_gram32(V32(w), k, QV32(w), k, w->nr, w->part, w->Hm, st));
     CK(qs_herm_eig2(w->G, DS(w, S_RN), w->di + 66, w->Hm, DS(w, S_THETA), w->Ym, w->di + 67, k, w->part, st));
     CK(qs_rotate32(V32(w), k, w->Ym, k, w->nr, T32(w), st));
     std::swap(w->iv, w->it3);
