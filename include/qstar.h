@@ -340,7 +340,8 @@ QS_API int qs_w_mass(qs_lattice *lat, double m, double mp, int n, const double *
  * Q_hat^2 (half the sites, better conditioned), x_o = (D_oo)^-1 (b_o - D_oe x_e); requires even
  * T and L.  even_odd = 0: conjugate gradients on the full-lattice Q^2 (for comparison).
  * b, x: DEVICE buffers of nrhs <= 64 FP64 spinors, canonical layout, not overlapping.  The CG
- * stops at ||r|| <= tol ||rhs|| for every right-hand side (QS_ENOCONV after max_iter);
+ * stops at ||r|| <= tol ||rhs|| for every right-hand side (QS_ENOCONV after max_iter; QS_ENUMERIC if
+ * one holds a NaN, with the solutions of the others in x);
  * *iterations (may be NULL) gets the count.  Allocates 9 nrhs vectors of work (half-lattice ones
  * with even_odd, plus the odd-site inverses, 1152 bytes per odd physical site); synchronises
  * the stream. */

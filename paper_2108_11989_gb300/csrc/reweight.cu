@@ -459,6 +459,8 @@ struct RwWork {
     double *part, *rpart, *dots;
     RwScal sc;
     int *hflag;           // pinned, RW_LAG + 1 copies of the live flags
+    double *hnorm;        // pinned, |b|^2 of the last rw_cg
+    bool nan_rhs;         // a right-hand side of a rw_cg was not a number (it was not iterated)
     cudaEvent_t ev[RW_LAG + 1];
     int full;             // 1: Q^2 of the full-lattice operator instead of Q_hat^2
     // odd-site block inverses at the two masses of the estimate
@@ -484,8 +486,10 @@ int rw_begin(RwWork &w, double *buf)
         w.sc.live[o] = (int *)(d + (4 + o) * w.nrhs);
     }
     w.hflag = nullptr;
+    w.nan_rhs = false;
     for (auto &e : w.ev) e = nullptr;
-    QS_CUDA(cudaMallocHost(&w.hflag, (RW_LAG + 1) * 64 * sizeof(int)));
+    QS_CUDA(cudaMallocHost(&w.hflag, (RW_LAG + 1) * 64 * sizeof(int) + 64 * sizeof(double)));
+    w.hnorm = (double *)(w.hflag + (RW_LAG + 1) * 64);
     for (auto &e : w.ev) QS_CUDA(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
     return QS_OK;
 }
@@ -564,7 +568,9 @@ int rw_cg(RwWork &w, double m, double sigma, const double *b, double *x, double 
     qs_note_launches(2);
     QS_TRY(rw_check("rw_cg"));
     QS_CUDA(cudaMemcpyAsync(w.hflag, w.sc.live[0], w.nrhs * sizeof(int), cudaMemcpyDeviceToHost, st));
+    QS_CUDA(cudaMemcpyAsync(w.hnorm, w.sc.rr[0], w.nrhs * sizeof(double), cudaMemcpyDeviceToHost, st));
     QS_CUDA(cudaStreamSynchronize(st));
+    for (int r = 0; r < w.nrhs; ++r) w.nan_rhs = w.nan_rhs || std::isnan(w.hnorm[r]);
     auto any = [&](const int *f) {
         for (int r = 0; r < w.nrhs; ++r)
             if (f[r]) return true;
@@ -758,6 +764,7 @@ extern "C" int qs_solve_D(qs_lattice *lat, double m0, const void *b, void *x, in
         if ((s = rw_check("qs_solve_D")) != QS_OK) break;
         const cudaError_t e = cudaStreamSynchronize(st);
         if (e != cudaSuccess) { qs_record_cuda_error(e, "qs_solve_D"); s = QS_ECUDA; }
+        else if (w.nan_rhs) s = QS_ENUMERIC;   // the others are solved
     } while (0);
     rw_end(w);
     cudaFree(buf);
