@@ -372,20 +372,22 @@ int qs_d32_run(qs_lattice *lat, int storage, const double *m0, const void *in, v
     return qs_d32_call(lat, c);
 }
 
-// launch of a filled-in call with the shape's autotuned variant.  NORM and RESID take the plain
-// operator's; a RESID call, whose output may be an input, never times variants itself.
+// launch of a filled-in call with the shape's autotuned variant.  NORM is timed for itself: its order
+// of variants is not the plain operator's (16^3 x 32, 16 vectors: variants 3 and 1 take 311 and 321 us
+// plain, 370 and 353 us with the sums).  RESID, whose output may be an input, takes NORM's.
 int qs_d32_call(qs_lattice *lat, const D32Call &c)
 {
     const int storage = c.storage, nrhs = c.nrhs, cheb = c.epi == QS_EPI_CHEB;
-    int &tv = lat->tuned32[storage][cheb][nrhs];
+    const int form = c.epi == QS_EPI_RESID ? QS_EPI_NORM : c.epi;
+    int &tv = lat->tuned32[storage][form][nrhs];
     if (tv == 0) {
-        const std::string key = tune_key(lat, "dslash32q", storage, cheb, nrhs);
+        const std::string key = tune_key(lat, "dslash32q", storage, form, nrhs);
         int v = tune_lookup(key);
         if (v < 0 || v >= qs_d32_nvariants()) {
             if (capturing(lat->stream) || c.epi == QS_EPI_RESID) {
                 v = qs_d32_fixed_variant(c.g, nrhs);   // no timing inside a capture
             } else {
-                // timing writes `out` only (in, y and x are read): harmless to the caller
+                // timing writes `out` (and NORM's shares) only: harmless to the caller
                 int st = QS_OK;
                 v = time_variants(lat, qs_d32_nvariants(), [&](int q) { return qs_d32_launch(c, q, lat->stream); }, &st);
                 if (st != QS_OK) return st;

@@ -53,9 +53,9 @@ struct qs_lattice {
     double *clov64;
     float2 *clov32;
     // autotuned launch variant + 1 (0: not tuned): FP64 operator per [layout][nrhs],
-    // FP32-arithmetic operator per [storage][Chebyshev epilogue][nrhs]
+    // FP32-arithmetic operator per [storage][plain, Chebyshev, with sums][nrhs]
     int tuned64[2][65];
-    int tuned32[4][2][65];
+    int tuned32[4][3][65];
     // solver workspace (allocated on first use, see solver.cu)
     struct Workspace *ws;
     // kernel profiling state (capi.cu), NULL when off
