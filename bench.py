@@ -12,8 +12,9 @@ per vector) is far larger than the 129 MB L2.
 
 value   = operator throughput over the whole step: algorithmic bytes of every operator
           launch in the step (per doubled site: each right-hand side's spinor in and out,
-          two more spinors for the fused Chebyshev step, and once per launch 36 link + 36
-          SW-term reals) / step time (GB/s).  ms_per_step is the Pf-sign time per
+          two more spinors for the fused Chebyshev step, one more for the CG's residual
+          update, and once per launch 36 link + 36 SW-term reals; right-hand sides that have
+          converged are skipped and not counted) / step time (GB/s).  ms_per_step is the Pf-sign time per
           configuration.
 e2e     = the same metric through the C-ABI with HOST inputs: the step loads the gauge
           field from host arrays (qs_load_gauge: copy, doubling, SW build) and returns the
@@ -63,20 +64,30 @@ def kernel_source_hash():
     return h.hexdigest()
 
 
-def measured_traffic(kind, algorithmic_bytes_per_launch):
-    """DRAM bytes per launch of the operator, from the committed ncu summary of one launch
-    of the current kernel source: the capture's ratio of DRAM bytes (read + write) to
-    algorithmic bytes, applied to this launch's algorithmic bytes (traffic scales with the
-    sites and right-hand sides a launch processes).  None if no capture of the current
-    source and storage exists."""
+def measured_traffic(kinds, algorithmic_bytes_per_launch):
+    """DRAM bytes per launch of operator launches of the given kinds, equally often each, from
+    the committed ncu summary of one launch of each kind of the current kernel source: the
+    captures' ratio of DRAM bytes (read + write) to algorithmic bytes, applied to this
+    launch's algorithmic bytes (traffic scales with the sites and right-hand sides a launch
+    processes).  None if a kind has no capture of the current source."""
     p = os.path.join(ROOT, "profiles", "dslash32_traffic.json")
     if not os.path.exists(p):
         return None
     d = json.load(open(p))
-    e = d.get(kind)
-    if not e or d.get("source_sha256") != kernel_source_hash():
+    e = [d.get(k) for k in kinds]
+    if not e or None in e or d.get("source_sha256") != kernel_source_hash():
         return None
-    return algorithmic_bytes_per_launch * e["dram_bytes"] / e["algorithmic_bytes"]
+    return algorithmic_bytes_per_launch * sum(k["dram_bytes"] for k in e) / sum(k["algorithmic_bytes"] for k in e)
+
+
+def step_kinds(name, eig_prec):
+    """The kinds of operator launch that the entry `name` of a sign computation's profile holds:
+    with 16-bit filter storage the FP32 entry is the inner CG's two launches (and few plain
+    ones), the 16-bit entry the filter's plain and Chebyshev ones; with an FP32 filter the FP32
+    entry mixes all four in unknown shares."""
+    if name == "f32" and eig_prec in ("f16", "bf16"):
+        return ["f32_norm", "f32_resid"]
+    return [name, name + "_cheb"] if name in ("f16", "bf16") else []
 
 
 def peaks():
@@ -434,13 +445,14 @@ def run_sign(args):
                     "operator_ms_share_of_step": {n: p["ms"] / total_ms for n, p in prof.items() if p["ms"] > 0}},
         "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                      "frac": achieved / peak,
-                     "traffic": measured_traffic(dname, dom["bytes"] / max(1, dom["launches"])),
+                     "traffic": measured_traffic(step_kinds(dname, args.eig_prec), dom["bytes"] / max(1, dom["launches"])),
                      "kernel": f"dslash32_kernel ({dname} storage, FP32 arithmetic)" if dname != "f64"
                      else "dslash_kernel<double>",
                      "launches": dom["launches"], "avg_launch_us": 1e3 * dom["ms"] / max(1, dom["launches"]),
                      "peak_source": f"{src} hbm_gbs (of measured)",
                      "bytes_model": "per doubled site: spinor in + out per right-hand side (+ 2 spinors for the "
-                                    "fused Chebyshev step) + 72 link/SW reals per launch"},
+                                    "fused Chebyshev step, + 1 for the CG's residual update) + 72 link/SW reals "
+                                    "per launch; converged right-hand sides, which are skipped, not counted"},
         "e2e": {"value": e2e, "unit": "GB/s", "h2d_bytes_per_step": h2d, "d2h_bytes_per_step": 4,
                 "s_per_config": e_s},
         "gpu_launches": launches,
@@ -550,7 +562,7 @@ def run_op_only(args):
                    "l2": "inputs rotated over buffer sets larger than L2",
                    "parallelism": "replicas" if ws > 1 else "single"},
         "roofline": {"bound": "hbm", "achieved": gbs, "peak": peak, "unit": "GB/s", "frac": gbs / peak,
-                     "traffic": measured_traffic(prec, bytes_per_launch), "peak_source": f"{src} hbm_gbs (of measured)",
+                     "traffic": measured_traffic([prec], bytes_per_launch), "peak_source": f"{src} hbm_gbs (of measured)",
                      "bytes_model": f"{op_bytes_per_site(R, prec)} B/site"},
         "e2e": {"value": e2e, "unit": "GB/s", "h2d_bytes_per_step": hx.numel() * hx.element_size(),
                 "d2h_bytes_per_step": hy.numel() * hy.element_size()},
