@@ -149,3 +149,34 @@ def test_shares_against_64_bits(lib, shape):
             want = (out.reshape(n, -1).double() ** 2).sum(1)
             assert bool(((part.sum(1) - want).abs() <= 4e-12 * want).all()), (variant, epi, (part.sum(1) / want - 1).tolist())
     lat.close()
+
+
+@pytest.mark.parametrize("shape", SHAPES, ids=str)
+def test_plain_in_every_storage(lib, shape):
+    """The plain operator in all storages, BF16 among them: every variant gives the same bits, and
+    the oracle's values to the tolerances above."""
+    import torch
+    from test_gpu_dslash import TOL16, pack16
+    qs, lat, cfg, n, v, dev = problem(shape)
+    ns = cfg.n_sites
+    op = WilsonDirac(cfg)
+    for storage, kind in ((F32, None), (CANON, None), (F16, "f16"), (BF16, "bf16")):
+        if kind:
+            buf, rep = pack16(v[0].reshape(n, ns, 12), kind)
+            x, w, tol = torch.from_numpy(buf).cuda(), rep.reshape(n, -1), TOL16[kind]
+        else:
+            x, w, tol = qs.to_tiled(dev[0], ns) if storage == F32 else dev[0], v[0], 1e-5
+        ref = np.stack([op.apply_Q(w[r], M0) for r in range(n)])
+        outs = []
+        for variant in range(lib.t_nvariants()):
+            outs.append(torch.zeros_like(x))
+            call(lib, lat, variant, storage, 0, n, x, outs[-1])
+            assert torch.equal(outs[-1], outs[0]), (variant, storage)
+        e = outs[0]
+        if kind:
+            e = torch.empty(n * ns * 24, dtype=torch.float32, device="cuda")
+            qs.convert_spinors(lat.h, outs[0], qs.QS_F16 if storage == F16 else qs.QS_BF16, e, qs.QS_F32, n)
+            torch.cuda.synchronize()
+        got = host(e if storage == CANON else qs.from_tiled(e, ns), n)
+        assert np.abs(got - ref).max() <= tol * np.abs(ref).max(), storage
+    lat.close()
